@@ -231,7 +231,8 @@ struct ChangeList {
 void launch_lb_step(int dtype, const LatticeView &lv, int par, const WallAcc &wa, int *status, cudaStream_t st);
 // the persistent row sweep's grid per instantiation (LatticeView::rows_grid)
 void lb_rows_grids(int dtype, int out[8]);
-void launch_fields(int dtype, const LatticeView &lv, int par, double *rho, double *u, int32_t *owner,
+// pend: add the pending moving-boundary terms (there are cells)
+void launch_fields(int dtype, const LatticeView &lv, int par, int pend, double *rho, double *u, int32_t *owner,
                    cudaStream_t st);
 void launch_pop_io(int dtype, const LatticeView &lv, int par, double *buf, int to_storage, cudaStream_t st);
 void launch_init(int dtype, const LatticeView &lv, cudaStream_t st);

@@ -224,8 +224,8 @@ static int build_surface_bits(bl_ctx *c) {
 
 // The steps leave the moving-boundary term C of their last bounces off cells
 // pending (the next sweep adds it as it reads the populations): before the
-// populations are read out or the cells are set anew, it is given to the
-// stored populations here.
+// populations are read out or set or the cells are set anew, it is given to
+// the stored populations here (the field read-out adds it as it reads).
 static int flush_pending(bl_ctx *c) {
   if (c->np == 0) return BL_OK;  // nothing pends without cells (a removal flushes first)
   launch_flush_pending(c->dtype, c->lv, c->parity, c->stream, &c->launches);
@@ -832,17 +832,16 @@ extern "C" int bl_sync(bl_ctx *c) {
 extern "C" int bl_fields_get(bl_ctx *c, double *rho, double *u, int32_t *owner, int on_device) {
   if (!c) return BL_EINVAL;
   if (c->sticky) return c->sticky;
-  if (flush_pending(c)) return c->sticky;
   const size_t N = c->lv.N;
   if (on_device) {
-    launch_fields(c->dtype, c->lv, c->parity, rho, u, owner, c->stream);
+    launch_fields(c->dtype, c->lv, c->parity, c->np > 0, rho, u, owner, c->stream);
     c->launches++;
     return check_launch(c, "fields");
   }
   if (ensure_scratch(c, N * sizeof(double) * 4 + N * sizeof(int32_t))) return c->sticky;
   double *drho = c->scratch, *du = c->scratch + N;
   int32_t *down = (int32_t *)(c->scratch + 4 * N);
-  launch_fields(c->dtype, c->lv, c->parity, drho, du, down, c->stream);
+  launch_fields(c->dtype, c->lv, c->parity, c->np > 0, drho, du, down, c->stream);
   c->launches++;
   if (check_launch(c, "fields")) return c->sticky;
   if (rho) CU(cudaMemcpyAsync(rho, drho, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "../../include/bloodlb.h"
+#include "lb_moments.cuh"
 #include "lb_sweep.cuh"
 
 namespace bl {
@@ -162,25 +163,25 @@ __device__ __forceinline__ size_t sparse_src(const SparseView &sv, int par, unsi
   return s >= 0 ? (size_t)D3Q19::opp(r) * sv.Nf + (unsigned)s : (size_t)r * sv.Nf + i;
 }
 
-// moments on the dense grid (zero at walls): rho and u = (j + rho g / 2) / rho
+// moments on the dense grid (zero at walls): rho and u = j / rho + g / 2
 template <class S>
-__global__ void k_sparse_fields(SparseView sv, int par, double *rho, double *u) {
+__global__ void __launch_bounds__(256) k_sparse_fields(SparseView sv, int par, double rho0, double hg0, double hg1,
+                                                       double hg2, double *rho, double *u) {
   const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= sv.Nf) return;
   const S *pop = reinterpret_cast<const S *>(sv.pop);
-  double d = 0.0, j[3] = {0.0, 0.0, 0.0};
-  for (int r = 0; r < Q; ++r) {
-    const double v = (double)Store<S>::ld(pop + sparse_src(sv, par, i, r));
-    d += v;
-    j[0] += D3Q19::cx(r) * v;
-    j[1] += D3Q19::cy(r) * v;
-    j[2] += D3Q19::cz(r) * v;
-  }
-  const double rh = (double)sv.rho0 + d;
+  float f[Q];
+  sfor<0, Q>([&](auto R) {
+    constexpr int r = decltype(R)::value;
+    f[r] = Store<S>::ld(pop + sparse_src(sv, par, i, r));
+  });
+  const double hg[3] = {hg0, hg1, hg2};
+  double rh, uu[3];
+  node_fields(f, rho0, hg, rh, uu);
   const unsigned n = (unsigned)sv.dense[i];
   if (rho) rho[n] = rh;
   if (u)
-    for (int k = 0; k < 3; ++k) u[3 * (size_t)n + k] = (j[k] + 0.5 * rh * (double)sv.g[k]) / rh;
+    for (int k = 0; k < 3; ++k) u[3 * (size_t)n + k] = uu[k];
 }
 
 // populations n_r (unshifted) on the dense grid, N x 19, to (0) or from (1) storage
@@ -490,9 +491,13 @@ extern "C" int bl_sparse_fields_get(bl_sparse *s, double *rho, double *u, int on
   if (dr) SPCU(cudaMemsetAsync(dr, 0, sizeof(double) * N, s->stream));
   if (du) SPCU(cudaMemsetAsync(du, 0, sizeof(double) * 3 * N, s->stream));
   const unsigned b = 256, g = nblk(s->sv.Nf, b);
-  if (s->lp.store_dtype == BL_STORE_F32) k_sparse_fields<float><<<g, b, 0, s->stream>>>(s->sv, s->parity, dr, du);
-  else if (s->lp.store_dtype == BL_STORE_BF16) k_sparse_fields<__nv_bfloat16><<<g, b, 0, s->stream>>>(s->sv, s->parity, dr, du);
-  else k_sparse_fields<__half><<<g, b, 0, s->stream>>>(s->sv, s->parity, dr, du);
+  const double r0 = (double)s->sv.rho0, h0 = 0.5 * (double)s->sv.g[0], h1 = 0.5 * (double)s->sv.g[1],
+               h2 = 0.5 * (double)s->sv.g[2];
+#define BL_SPF(S_) k_sparse_fields<S_><<<g, b, 0, s->stream>>>(s->sv, s->parity, r0, h0, h1, h2, dr, du)
+  if (s->lp.store_dtype == BL_STORE_F32) BL_SPF(float);
+  else if (s->lp.store_dtype == BL_STORE_BF16) BL_SPF(__nv_bfloat16);
+  else BL_SPF(__half);
+#undef BL_SPF
   s->launches++;
   if (sp_check(s, "fields")) return s->sticky;
   if (!on_device) {

@@ -10,6 +10,7 @@
 // contact links.  Inside the steps the same results come incrementally
 // (particle_kernels.cu: k_nbm_update, k_contacts).
 #include "bl_internal.cuh"
+#include "lb_moments.cuh"
 
 namespace bl {
 
@@ -107,42 +108,65 @@ __global__ void __launch_bounds__(128) k_geometry(LatticeView lv, PartView pv) {
 }
 
 // ---------------------------------------------------------------------------
-// moments of the current populations (layout of parity par)
+// moments of the current populations (layout of parity par), with the pending
+// moving-boundary terms of the last step's bounces off cells (pend: there are
+// cells) added to the populations as they are read, so that a read-out leaves
+// the stored state as it is.  One thread per node, a warp's velocities written
+// together.  Bound: HBM in the end (76 + 16 + 4 bytes read, 36 written per
+// node with FP32 storage and cells); with the FP64 sums of before it was bound
+// by FP64 issue (lb_moments.cuh).
+constexpr int FT = 256;
 
-template <class S>
-__global__ void k_fields(LatticeView lv, int par, double *rho_out, double *u_out, int32_t *owner_out) {
+template <class S, bool PEND>
+__global__ void __launch_bounds__(FT) k_fields(LatticeView lv, int par, double rho0, double hg0, double hg1, double hg2,
+                                               double *rho_out, double *u_out, int32_t *owner_out) {
   using D = D3Q19;
-  const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= lv.N) return;
+  __shared__ double su[FT / 32][96];
+  const unsigned n0 = blockIdx.x * FT + threadIdx.x;
+  const bool valid = n0 < lv.N;
+  const unsigned n = valid ? n0 : lv.N - 1u;
   const int own = lv.owner[n];
-  if (owner_out) owner_out[n] = own;
-  if (own != FLUID) {
-    if (rho_out) rho_out[n] = 0.0;
-    if (u_out) u_out[3 * n] = u_out[3 * n + 1] = u_out[3 * n + 2] = 0.0;
-    return;
-  }
-  const int nx = lv.nx, ny = lv.ny, nz = lv.nz;
-  const int x = n % nx, y = (n / nx) % ny, z = n / ((unsigned)nx * ny);
-  const S *pop = reinterpret_cast<const S *>(lv.pop);
-  double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
-  for (int r = 0; r < Q; ++r) {
-    unsigned src;
-    if (par == 0 || r == 0) {
-      src = (unsigned)r * lv.N + n;
-    } else {
-      const int xs = wrapi(x - D::cx(r), nx), ys = wrapi(y - D::cy(r), ny), zs = wrapi(z - D::cz(r), nz);
-      src = (unsigned)D::opp(r) * lv.N + (unsigned)xs + (unsigned)nx * ((unsigned)ys + (unsigned)ny * zs);
+  if (owner_out && valid) owner_out[n] = own;
+  double rho = 0.0, u[3] = {0.0, 0.0, 0.0};
+  if (own == FLUID && (rho_out || u_out)) {
+    int c[3];
+    node_xyz(lv, n, c);
+    const unsigned nx = (unsigned)lv.nx, nxy = nx * (unsigned)lv.ny;
+    const unsigned xo[3] = {(unsigned)(c[0] == 0 ? lv.nx - 1 : c[0] - 1), (unsigned)c[0],
+                            (unsigned)(c[0] == lv.nx - 1 ? 0 : c[0] + 1)};
+    const unsigned yo[3] = {(unsigned)(c[1] == 0 ? lv.ny - 1 : c[1] - 1) * nx, (unsigned)c[1] * nx,
+                            (unsigned)(c[1] == lv.ny - 1 ? 0 : c[1] + 1) * nx};
+    const unsigned zo[3] = {(unsigned)(c[2] == 0 ? lv.nz - 1 : c[2] - 1) * nxy, (unsigned)c[2] * nxy,
+                            (unsigned)(c[2] == lv.nz - 1 ? 0 : c[2] + 1) * nxy};
+    const S *pop = reinterpret_cast<const S *>(lv.pop);
+    float f[Q];
+    sfor<0, Q>([&](auto R) {
+      constexpr int r = decltype(R)::value;
+      const unsigned src = par == 0 || r == 0
+                               ? (unsigned)r * lv.N + n
+                               : (unsigned)D::opp(r) * lv.N + xo[1 - D::cx(r)] + yo[1 - D::cy(r)] + zo[1 - D::cz(r)];
+      f[r] = Store<S>::ld(pop + src);
+    });
+    if constexpr (PEND) {
+      const float4 pu = lv.pu[n];
+      const uint32_t pm = __float_as_uint(pu.w);
+      if (pm)
+        sfor<1, Q>([&](auto R) {
+          constexpr int r = decltype(R)::value;
+          if ((pm >> r) & 1u) {
+            const float C = -(D::m(r) / 6.0f) * (D::cx(r) * pu.x + D::cy(r) * pu.y + D::cz(r) * pu.z);
+            // in the storage type, as a read-out has always shown it
+            S v;
+            Store<S>::st(&v, f[D::opp(r)] + C);
+            f[D::opp(r)] = Store<S>::ld(&v);
+          }
+        });
     }
-    const double v = Store<S>::ld(pop + src);
-    drho += v;
-    j[0] += v * D::cx(r);
-    j[1] += v * D::cy(r);
-    j[2] += v * D::cz(r);
+    const double hg[3] = {hg0, hg1, hg2};
+    node_fields(f, rho0, hg, rho, u);
   }
-  const double rho = (double)lv.rho0 + drho;
-  if (rho_out) rho_out[n] = rho;
-  if (u_out)
-    for (int k = 0; k < 3; ++k) u_out[3 * n + k] = (j[k] + 0.5 * rho * (double)lv.g[k]) / rho;
+  if (rho_out && valid) rho_out[n] = rho;
+  if (u_out) store_u_rows(u_out, (size_t)(n0 & ~31u), lv.N, su[threadIdx.x >> 5], u);
 }
 
 // node-major unshifted FP64 populations <-> storage (layout of parity par)
@@ -335,11 +359,21 @@ void launch_geometry(const LatticeView &lv, const PartView &pv, cudaStream_t st,
   if (nl) ++*nl;
 }
 
-void launch_fields(int dtype, const LatticeView &lv, int par, double *rho, double *u, int32_t *owner, cudaStream_t st) {
-  const unsigned b = 256, g = nblk(lv.N, b);
-  if (dtype == 0) k_fields<float><<<g, b, 0, st>>>(lv, par, rho, u, owner);
-  else if (dtype == 1) k_fields<__nv_bfloat16><<<g, b, 0, st>>>(lv, par, rho, u, owner);
-  else k_fields<__half><<<g, b, 0, st>>>(lv, par, rho, u, owner);
+void launch_fields(int dtype, const LatticeView &lv, int par, int pend, double *rho, double *u, int32_t *owner,
+                   cudaStream_t st) {
+  const unsigned g = nblk(lv.N, FT);
+  const double r0 = (double)lv.rho0, h0 = 0.5 * (double)lv.g[0], h1 = 0.5 * (double)lv.g[1], h2 = 0.5 * (double)lv.g[2];
+#define BL_FIELDS(S_)                                                                         \
+  if (pend) k_fields<S_, true><<<g, FT, 0, st>>>(lv, par, r0, h0, h1, h2, rho, u, owner);     \
+  else k_fields<S_, false><<<g, FT, 0, st>>>(lv, par, r0, h0, h1, h2, rho, u, owner)
+  if (dtype == 0) {
+    BL_FIELDS(float);
+  } else if (dtype == 1) {
+    BL_FIELDS(__nv_bfloat16);
+  } else {
+    BL_FIELDS(__half);
+  }
+#undef BL_FIELDS
 }
 
 void launch_pop_io(int dtype, const LatticeView &lv, int par, double *buf, int to_storage, cudaStream_t st) {
