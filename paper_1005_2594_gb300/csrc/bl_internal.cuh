@@ -99,6 +99,7 @@ struct LatticeView {
   int32_t *owner;  // N
   uint32_t *nbm;   // N neighbour words of the current owner map (NB_* bits), written by the geometry pass
   uint32_t *nbc;   // N neighbour-cell words (NBC_*), written with the neighbour words
+  uint4 *nbx;      // N mixed words (NBX_*): read for nodes between a cell and another cell or a wall
   // Cell links of the sweep.  A fluid node next to a cell writes one link
   // record per cell into that cell's bucket, for the link-momentum sums.
   // The moving-boundary term C of its bounced populations needs the cell's
@@ -154,6 +155,12 @@ constexpr uint32_t NB_CELL = 1u << 20;
 // second cell among them: the sweep then reads the neighbours' owners)
 constexpr uint32_t NBC_MIXED = 1u << 31;
 constexpr uint32_t NBC_CELL = 0x7FFFFFFFu;
+// mixed word of a fluid node with NB_CELL and NBC_MIXED: .x the first cell in
+// direction order and, shifted by 16, the second one (NBX_NONE: none; a
+// context holds at most 65535 cells), .y and .z the neighbours (bits 1..18)
+// each of them owns, .w those that are walls; what is left of the solid
+// neighbours belongs to a third cell
+constexpr uint32_t NBX_NONE = 0xFFFFu;
 
 // momentum given to each wall id by its bounce-back links: variable part in
 // FP64, constant part 2 alpha_r rho_bar c_r as exact integer sums of m_r c_r
@@ -343,6 +350,25 @@ __device__ __forceinline__ void unpack_xyzr(unsigned long long e, int xyz[3], in
   xyz[2] = (int)(e >> 45);
 }
 
+// the mixed word from the owners of a node and its 18 neighbours (on[r]: x + c_r)
+__device__ __forceinline__ uint4 mixed_word(const int (&on)[Q]) {
+  uint4 w = make_uint4(0u, 0u, 0u, 0u);
+  int p1 = -1, p2 = -1;
+  sfor<1, Q>([&](auto R) {
+    constexpr int r = decltype(R)::value;
+    if (on[r] <= -2) {
+      w.w |= 1u << r;
+    } else if (on[r] >= 0) {
+      if (p1 < 0) p1 = on[r];
+      else if (p2 < 0 && on[r] != p1) p2 = on[r];
+      w.y |= (on[r] == p1 ? 1u : 0u) << r;
+      w.z |= (on[r] == p2 ? 1u : 0u) << r;
+    }
+  });
+  w.x = ((uint32_t)p1 & NBX_NONE) | ((uint32_t)p2 << 16);
+  return w;
+}
+
 // direction masks of the lattice (bit r), for the record sums by popcount
 template <class P>
 __host__ __device__ constexpr uint32_t dir_mask(P pred) {
@@ -407,19 +433,113 @@ __device__ __forceinline__ int mask_Mab(uint32_t m) {
   return popm(m, PairDirs<A, B, 1>::v) - popm(m, PairDirs<A, B, -1>::v);
 }
 
-// post-collision shifted population at tau = 1: the third-order equilibrium
-// w (drho + rho t), t = 4.5 cu^2 - 1.5 uu + cu (3 - 4.5 uu + 4.5 cu^2), with
-// rho t taken as rho_bar t + drho t (exact for small drho in FP32), plus the
-// Guo source src_w w (3 (cF - uF) + 9 cu cF) when a force acts; the sweep and
-// the link sums evaluate this same function, so the bounced populations the
-// fluid keeps and those the cell's momentum counts agree
-__device__ __forceinline__ float post_tau1(float w, float drho, float rho0, float cu, float uu, bool force, float cF,
-                                           float uF, float src_w) {
-  const float q = 4.5f * cu * cu;
-  const float t = (q - 1.5f * uu) + cu * ((3.0f - 4.5f * uu) + q);
-  float fs = w * (drho + fmaf(drho, t, rho0 * t));
-  if (force) fs += src_w * w * (3.0f * (cF - uF) + 9.0f * cu * cF);
-  return fs;
+// The populations an opposite pair r, rbar relaxes toward: the third-order
+// equilibrium w (drho + rho t), t = 4.5 cu^2 - 1.5 uu +- cu (3 - 4.5 uu + 4.5
+// cu^2), plus the Guo source over omega, src w (3 (cF - uF) + 9 cu cF) / omega
+// with src = 1 - omega / 2 (so that f - omega (f - this) is the collision).
+// The even and the odd part of t and of the source are shared by the pair, and
+// rho t + drho is one fused multiply-add: 9 operations a pair, 13 with a
+// force, where each direction by itself took 16 and 27.  Folding rho and the
+// weight into the node's coefficients would save two more, but rounds each
+// population twice more and raised the density error at tau = 0.8 by half.
+// The sweeps of the dense and the indexed lattice and the link sums evaluate
+// this same function, so the bounced populations the fluid keeps and those
+// the cell's momentum counts agree.
+struct Collide {
+  float ux, uy, uz, rho;
+  float a, b;        // 3 - 4.5 uu, 1.5 uu
+  float drho;        // with a force drho - u . H
+  float Hx, Hy, Hz;  // 3 src F / omega
+};
+
+template <bool FORCE>
+__device__ __forceinline__ Collide collide_coeffs(float drho, float rho, float ux, float uy, float uz, float uu,
+                                                  float omega, float Fx, float Fy, float Fz, float uF) {
+  Collide k;
+  k.ux = ux;
+  k.uy = uy;
+  k.uz = uz;
+  k.rho = rho;
+  k.a = fmaf(-4.5f, uu, 3.0f);
+  k.b = 1.5f * uu;
+  k.drho = drho;
+  k.Hx = k.Hy = k.Hz = 0.f;
+  if constexpr (FORCE) {
+    const float h = 3.0f * (1.0f / omega - 0.5f);
+    k.drho = fmaf(-h, uF, drho);
+    k.Hx = h * Fx;
+    k.Hy = h * Fy;
+    k.Hz = h * Fz;
+  }
+  return k;
+}
+
+// component of c_R for odd R along u: at most two additions
+template <int R>
+__device__ __forceinline__ float dir_dot(float x, float y, float z) {
+  using D = D3Q19;
+  float v = 0.f;
+  if constexpr (D::cx(R) != 0) v = D::cx(R) > 0 ? x : -x;
+  if constexpr (D::cy(R) != 0) v = D::cy(R) > 0 ? v + y : v - y;
+  if constexpr (D::cz(R) != 0) v = D::cz(R) > 0 ? v + z : v - z;
+  return v;
+}
+
+// targets of populations R and R + 1 (odd R, opposite directions) over their
+// weight
+template <int R, bool FORCE>
+__device__ __forceinline__ void collide_pair(const Collide &k, float &xr, float &xb) {
+  const float cu = dir_dot<R>(k.ux, k.uy, k.uz);
+  const float s = cu * cu;
+  const float E = fmaf(4.5f, s, -k.b), q = fmaf(4.5f, s, k.a);
+  const float tr = fmaf(cu, q, E), tb = fmaf(-cu, q, E);
+  if constexpr (FORCE) {
+    const float cH = dir_dot<R>(k.Hx, k.Hy, k.Hz), e = fmaf(3.0f * cu, cH, k.drho);
+    xr = fmaf(k.rho, tr, e + cH);
+    xb = fmaf(k.rho, tb, e - cH);
+  } else {
+    xr = fmaf(k.rho, tr, k.drho);
+    xb = fmaf(k.rho, tb, k.drho);
+  }
+}
+
+// the target of population 0 over its weight
+__device__ __forceinline__ float collide_rest(const Collide &k) { return fmaf(-k.rho, k.b, k.drho); }
+
+// relaxation of population R toward w x: f - omega (f - w x), at tau = 1 w x
+template <int R, bool TAU1>
+__device__ __forceinline__ float relax_to(float f, float x, float omega) {
+  constexpr float w = (float)D3Q19::m(R) / 36.0f;
+  return TAU1 ? __fmul_rn(w, x) : fmaf(-omega, fmaf(-w, x, f), f);
+}
+
+// velocity (j + F / 2) / rho of a node, its square and u . F, F = rho g, with
+// every contraction written out: the two lattices' sweeps agree bit for bit
+template <bool FORCE>
+__device__ __forceinline__ void node_velocity(float rho, float jx, float jy, float jz, const float (&g)[3], float (&u)[3],
+                                              float (&F)[3], float &uu, float &uF) {
+  const float inv = 1.0f / rho;
+  F[0] = F[1] = F[2] = uF = 0.f;
+  if constexpr (FORCE) {
+    for (int k = 0; k < 3; ++k) F[k] = __fmul_rn(rho, g[k]);
+    jx = fmaf(0.5f, F[0], jx);
+    jy = fmaf(0.5f, F[1], jy);
+    jz = fmaf(0.5f, F[2], jz);
+  }
+  u[0] = __fmul_rn(jx, inv);
+  u[1] = __fmul_rn(jy, inv);
+  u[2] = __fmul_rn(jz, inv);
+  uu = fmaf(u[2], u[2], fmaf(u[1], u[1], __fmul_rn(u[0], u[0])));
+  if constexpr (FORCE) uF = fmaf(u[2], F[2], fmaf(u[1], F[1], __fmul_rn(u[0], F[0])));
+}
+
+// moving-wall term of a link along c_R into a wall of velocity v (Eq. c):
+// 6 alpha rho c_rbar . v, added to the population that returns along rbar
+template <int R>
+__device__ __forceinline__ float wall_term(float rho, const float (&v)[3]) {
+  using D = D3Q19;
+  const float cv = fmaf((float)D::cz(R), v[2], fmaf((float)D::cy(R), v[1], __fmul_rn((float)D::cx(R), v[0])));
+  return __fmul_rn(__fmul_rn(-(D::m(R) / 6.0f), rho), cv);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

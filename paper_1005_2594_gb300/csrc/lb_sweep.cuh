@@ -52,6 +52,11 @@ namespace bl {
 #ifndef BL_ONE_MINB
 #define BL_ONE_MINB 9
 #endif
+// with cells at tau != 1 the old populations stay live through the collision:
+// 72 registers instead of 190 spilled bytes
+#ifndef BL_ONE_MINB_BGK
+#define BL_ONE_MINB_BGK 7
+#endif
 // the bulk-copy sweep: resident blocks per SM (its register cap) and stages
 #ifndef BL_BULK_MINB
 #define BL_BULK_MINB 6
@@ -186,45 +191,23 @@ __device__ __forceinline__ void emit_second(const LatticeView &lv, const CellLin
   write_second<TAU1>(lv, cl, n, sl2);
 }
 
-// the neighbour n + c_r for a direction r known only at run time: the
-// components of c_r + 1 from their packed form, the coordinate chosen by
-// selects (no indexing of the xo, yo, zo arrays)
-__device__ __forceinline__ unsigned pick3(unsigned k, const unsigned v[3]) { return k == 0 ? v[0] : (k == 1 ? v[1] : v[2]); }
-__device__ __forceinline__ unsigned neighbour_rt(int r, const unsigned xo[3], const unsigned yo[3], const unsigned zo[3]) {
-  constexpr unsigned long long PX = packed_dirs<0>(), PY = packed_dirs<1>(), PZ = packed_dirs<2>();
-  return pick3((unsigned)(PX >> (2 * r)) & 3u, xo) + pick3((unsigned)(PY >> (2 * r)) & 3u, yo) +
-         pick3((unsigned)(PZ >> (2 * r)) & 3u, zo);
-}
-
 // the pending C of the last step's bounces off a cell: pu.xyz = rho (V + W x
 // d) of the cell at the node, pu.w the bounced directions (bit r); C_r =
 // -(m_r / 6) c_r . pu is added to the incoming population of direction rbar
-// (every direction computed, the masked ones kept: no branch per direction)
+// (every pair computed once, the masked directions kept: no branch per
+// direction).  Taken into the populations at tau = 1 too: summing it into the
+// moments by popcounts of the mask took 24 of them, which issue at a quarter
+// of the rate of these adds
 __device__ __forceinline__ void apply_pending(const float4 &pu, float (&f)[Q]) {
   using D = D3Q19;
   const uint32_t mask = __float_as_uint(pu.w);
-  sfor<1, Q>([&](auto R) {
-    constexpr int r = decltype(R)::value;
-    float cu = 0.f;
-    if constexpr (D::cx(r) != 0) cu += D::cx(r) * pu.x;
-    if constexpr (D::cy(r) != 0) cu += D::cy(r) * pu.y;
-    if constexpr (D::cz(r) != 0) cu += D::cz(r) * pu.z;
-    f[D::opp(r)] -= ((mask >> r) & 1u) ? (D::m(r) / 6.0f) * cu : 0.0f;
+  const float sx = (1.0f / 6.0f) * pu.x, sy = (1.0f / 6.0f) * pu.y, sz = (1.0f / 6.0f) * pu.z;
+  sfor<0, 9>([&](auto P) {
+    constexpr int r = 2 * decltype(P)::value + 1, rb = r + 1;
+    const float cu = (float)D::m(r) * dir_dot<r>(sx, sy, sz);
+    if ((mask >> r) & 1u) f[rb] -= cu;
+    if ((mask >> rb) & 1u) f[r] += cu;
   });
-}
-
-// the same C taken into the moments alone (enough at tau = 1, where the
-// collision keeps nothing of a population but its moments):
-// drho -= K . pu / 6, j += M pu / 6, K = sum m_r c_r, M = sum m_r c_r c_r^T
-// over the bounced directions
-__device__ __forceinline__ void pending_moments(const float4 &pu, float &drho, float &jx, float &jy, float &jz) {
-  const uint32_t m = __float_as_uint(pu.w);
-  const float s = 1.0f / 6.0f;
-  drho -= s * ((float)mask_K<0>(m) * pu.x + (float)mask_K<1>(m) * pu.y + (float)mask_K<2>(m) * pu.z);
-  const float mxy = (float)mask_Mab<0, 1>(m), mxz = (float)mask_Mab<0, 2>(m), myz = (float)mask_Mab<1, 2>(m);
-  jx += s * ((float)mask_Maa<0>(m) * pu.x + mxy * pu.y + mxz * pu.z);
-  jy += s * (mxy * pu.x + (float)mask_Maa<1>(m) * pu.y + myz * pu.z);
-  jz += s * (mxz * pu.x + myz * pu.y + (float)mask_Maa<2>(m) * pu.z);
 }
 
 // sum of 2 f~*_r c_r over the directions in mask (no branch per direction)
@@ -261,8 +244,9 @@ __device__ __forceinline__ void append_link(const LatticeView &lv, unsigned n, i
 // cell links.  load(r, slot) gives the incoming population of direction r
 // (from the slot src_slot names); pu is the node's pending velocity.
 // FORCE: a body force is set (Guo forcing); TAU1: tau = 1, where the
-// relaxation gives the equilibrium itself
-template <class S, int PAR, bool FORCE, bool TAU1, class Load>
+// relaxation gives the equilibrium itself; CELLS: the context has cells
+// (without them no node has a cell neighbour or a pending C)
+template <class S, int PAR, bool FORCE, bool TAU1, bool CELLS, class Load>
 __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc &wa, unsigned n, const int xyz[3],
                                             const unsigned xo[3], const unsigned yo[3], const unsigned zo[3],
                                             uint32_t nbw, uint32_t nbc, float4 pu, Load load, int &wkey,
@@ -274,110 +258,73 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
   cl.p2 = -1;
   if (nbw & NB_FLUID) {
     const unsigned solid = nbw & NB_SOLID;
+    // a node between a cell and something else: its mixed word, in one load
+    // that the collision hides (the owners of its neighbours, read here one
+    // after the other, were the sweep's longest chain of waits)
+    const bool mixed = CELLS && (nbw & NB_CELL) && (nbc & NBC_MIXED);
+    uint4 xw = make_uint4(0u, 0u, 0u, 0u);
+    if (mixed) xw = lv.nbx[n];
     // incoming populations of this node (layout of the step's parity)
     float f[Q];
     sfor<0, Q>([&](auto R) {
       constexpr int r = decltype(R)::value;
-      unsigned src;
-      if constexpr (PAR == 0 || r == 0) {
-        src = (unsigned)r * N + n;
-      } else {
-        src = (unsigned)D::opp(r) * N + xo[1 - D::cx(r)] + yo[1 - D::cy(r)] + zo[1 - D::cz(r)];
-      }
-      f[r] = load(r, src);
+      f[r] = load(r, src_slot<PAR>(r, N, n, xo, yo, zo));
     });
-    // C of the last step's bounces off a cell (reading Q3): into the
-    // populations, or at tau = 1 into the moments
-    const uint32_t pm = __float_as_uint(pu.w);
-    if constexpr (!TAU1) {
+    // C of the last step's bounces off a cell (reading Q3)
+    const uint32_t pm = CELLS ? __float_as_uint(pu.w) : 0u;
+    if constexpr (CELLS) {
       if (pm) apply_pending(pu, f);
     }
     // moments (shifted: rho = rho_bar + sum f~, j = sum f~ c)
-    float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
-    sfor<0, Q>([&](auto R) {
-      constexpr int r = decltype(R)::value;
-      drho += f[r];
-      if constexpr (D::cx(r) != 0) jx += D::cx(r) * f[r];
-      if constexpr (D::cy(r) != 0) jy += D::cy(r) * f[r];
-      if constexpr (D::cz(r) != 0) jz += D::cz(r) * f[r];
+    float drho = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
+    sfor<0, 9>([&](auto P) {
+      constexpr int r = 2 * decltype(P)::value + 1;
+      const float s = f[r] + f[r + 1], d = f[r] - f[r + 1];
+      drho += s;
+      if constexpr (D::cx(r) != 0) jx += D::cx(r) > 0 ? d : -d;
+      if constexpr (D::cy(r) != 0) jy += D::cy(r) > 0 ? d : -d;
+      if constexpr (D::cz(r) != 0) jz += D::cz(r) > 0 ? d : -d;
     });
-    if constexpr (TAU1) {
-      if (pm) pending_moments(pu, drho, jx, jy, jz);
-    }
     const float rho = lv.rho0 + drho;
-    const float inv = 1.0f / rho;
-    float Fx = 0.f, Fy = 0.f, Fz = 0.f;
-    if constexpr (FORCE) {
-      Fx = rho * lv.g[0];
-      Fy = rho * lv.g[1];
-      Fz = rho * lv.g[2];
-    }
-    const float ux = (jx + 0.5f * Fx) * inv, uy = (jy + 0.5f * Fy) * inv, uz = (jz + 0.5f * Fz) * inv;
-    const float uu = ux * ux + uy * uy + uz * uz;
+    float u[3], F[3], uu, uF;
+    node_velocity<FORCE>(rho, jx, jy, jz, lv.g, u, F, uu, uF);
+    const float ux = u[0], uy = u[1], uz = u[2];
     if (!(rho > 0.f) || !(uu < 0.09f)) atomicOr(lv.status, ST_UNSTABLE);
     // the moments of the nodes beside a sheared plane, for its passes
     if (lv.le_mom != nullptr && (xyz[0] == 0 || xyz[0] == lv.nx - 1))
       lv.le_mom[(xyz[0] == 0 ? 0u : (unsigned)lv.ny * (unsigned)lv.nz) + (unsigned)xyz[1] +
                 (unsigned)lv.ny * (unsigned)xyz[2]] = make_float4(drho, ux, uy, uz);
-    const float om = lv.omega;
-    const float src_w = 1.0f - 0.5f * om;
-    const float uF = ux * Fx + uy * Fy + uz * Fz;
-    // relaxation toward the shifted equilibrium w (drho + rho t); rho t is
-    // taken as rho_bar t + drho t, which keeps the small deviation exact in
-    // FP32; the Guo source with cu = c.u, cF = c.F
-    auto relax = [&](float fr, float w, float t, float cu, float cF) {
-      const float feq = w * (drho + fmaf(drho, t, lv.rho0 * t));
-      float fs = TAU1 ? feq : fr - om * (fr - feq);
-      if constexpr (FORCE) fs += src_w * w * (3.0f * (cF - uF) + 9.0f * cu * cF);
-      return fs;
-    };
-    // third-order equilibrium in pairs r, rbar = r + 1 (c_rbar = -c_r):
-    // t = E + O and E - O with the even part E = 4.5 cu^2 - 1.5 uu and the
-    // odd part O = cu (3 + 4.5 cu^2 - 4.5 uu)
-    const float a = 3.0f - 4.5f * uu, b = 1.5f * uu;
-    f[0] = relax(f[0], 12.0f / 36.0f, -b, 0.f, 0.f);
+    const float om = TAU1 ? 1.0f : lv.omega;
+    const Collide k = collide_coeffs<FORCE>(drho, rho, ux, uy, uz, uu, om, F[0], F[1], F[2], uF);
+    f[0] = relax_to<0, TAU1>(f[0], collide_rest(k), om);
     sfor<0, 9>([&](auto P) {
       constexpr int r = 2 * decltype(P)::value + 1, rb = r + 1;
-      constexpr float w = D::m(r) / 36.0f;
-      float cu = 0.f, cF = 0.f;
-      if constexpr (D::cx(r) != 0) cu += D::cx(r) * ux;
-      if constexpr (D::cy(r) != 0) cu += D::cy(r) * uy;
-      if constexpr (D::cz(r) != 0) cu += D::cz(r) * uz;
-      if constexpr (FORCE) cF = D::cx(r) * Fx + D::cy(r) * Fy + D::cz(r) * Fz;
-      const float q = 4.5f * cu * cu;
-      const float E = q - b, O = cu * (a + q);
-      f[r] = relax(f[r], w, E + O, cu, cF);
-      f[rb] = relax(f[rb], w, E - O, -cu, -cF);
+      float xr, xb;
+      collide_pair<r, FORCE>(k, xr, xb);
+      f[r] = relax_to<r, TAU1>(f[r], xr, om);
+      f[rb] = relax_to<rb, TAU1>(f[rb], xb, om);
     });
     Store<S>::st(pop + n, f[0]);
     // neighbour classes from the geometry pass: solid = any non-fluid node;
-    // next to a wall or a cell the owners of the solid neighbours give the
-    // walls and the cells (in direction order: the first and a second cell
-    // each get a record and a pending C; a third, rare, its links one by one)
+    // next to a wall or a cell its neighbours' owners come from the
+    // neighbour-cell word (one cell and nothing else, the common case) or the
+    // mixed word: the first and a second cell in direction order each get a
+    // record and a pending C; a third, rare, its links one by one
     if (nbw & (NB_WALL | NB_CELL)) {
       unsigned wall = 0, cmask = 0, cmask2 = 0, csec = 0;
       int p1 = -1, p2 = -1;
-      // one cell and nothing else next to the node (the common case): its
-      // index from the neighbour-cell word, no owner to read
-      const bool one_cell = !(nbc & NBC_MIXED);
-      if (one_cell) {
+      if (!CELLS || !(nbw & NB_CELL)) {
+        wall = solid;
+      } else if (!mixed) {
         p1 = (int)nbc;
         cmask = solid;
-      }
-      for (unsigned m = one_cell ? 0u : solid; m; m &= m - 1u) {
-        const int r = __ffs(m) - 1;
-        const int ow = lv.owner[neighbour_rt(r, xo, yo, zo)];
-        if (ow <= -2) {
-          wall |= 1u << r;
-        } else if (p1 < 0 || ow == p1) {
-          p1 = ow;
-          cmask |= 1u << r;
-        } else if (p2 < 0 || ow == p2) {
-          p2 = ow;
-          cmask2 |= 1u << r;
-        } else {
-          csec |= 1u << r;
-        }
+      } else {
+        p1 = (int)(xw.x & NBX_NONE);
+        p2 = (int)(xw.x >> 16);
+        cmask = xw.y;
+        cmask2 = xw.z;
+        wall = xw.w;
+        csec = solid & ~(cmask | cmask2 | wall);
       }
       if (wall) {
         // links into a wall: the moving-wall term C for the population
@@ -388,8 +335,7 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
           if (wall & (1u << r)) {
             const unsigned nb = xo[1 + D::cx(r)] + yo[1 + D::cy(r)] + zo[1 + D::cz(r)];
             const int w = -2 - lv.owner[nb];
-            const float C = -(D::m(r) / 6.0f) * rho *
-                            (D::cx(r) * lv.wall_vel[w][0] + D::cy(r) * lv.wall_vel[w][1] + D::cz(r) * lv.wall_vel[w][2]);
+            const float C = wall_term<r>(rho, lv.wall_vel[w]);
             const float dp = 2.0f * f[r] + C;
             if (wkey != w && wkey >= 0) {
               // a node touching two different walls: flush the first one directly
@@ -416,7 +362,7 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
       // for C in place after the solve.  At tau = 1 a record holds the
       // node's moments (the same for every cell of the node), else the sum
       // of 2 f~*_r c_r over its directions
-      if (cmask) {
+      if (CELLS && cmask) {
         cl.p = p1;
         cl.mask = cmask;
         cl.e[0] = drho;
@@ -458,7 +404,7 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
     }
     // a node whose C was pending and that has no first-cell record now: no
     // pending C for the next sweep (a record's pu is written after the solve)
-    if (pm && cl.p < 0) reinterpret_cast<float *>(lv.pu + n)[3] = 0.f;
+    if (CELLS && pm && cl.p < 0) reinterpret_cast<float *>(lv.pu + n)[3] = 0.f;
     // streaming, or bounce-back into the slot where the next step reads
     // direction rbar where the neighbour is solid: one store per direction,
     // its slot chosen without a branch (so that a warp mixing open and
@@ -476,15 +422,18 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
   }
 }
 
-template <class S, int PAR, bool FORCE, bool TAU1>
-__global__ void __launch_bounds__(128, BL_ONE_MINB) k_lb_step(LatticeView lv, WallAcc wa) {
+// One node per thread, the nodes of a z plane numbered through (x fastest), so
+// that rows of any length fill the warps: with a block per row segment, 150
+// nodes left 41 % of the threads without a node, 48 nodes 25 %.
+template <class S, int PAR, bool FORCE, bool TAU1, bool CELLS>
+__global__ void __launch_bounds__(128, TAU1 || !CELLS ? BL_ONE_MINB : BL_ONE_MINB_BGK) k_lb_step(LatticeView lv, WallAcc wa) {
   const int nx = lv.nx, ny = lv.ny;
-  const int x0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z;
-  const bool valid = x0 < nx;
-  const int x = valid ? x0 : nx - 1;
-  const unsigned nxy = (unsigned)nx * (unsigned)ny;
-  const unsigned n = (unsigned)x + (unsigned)nx * (unsigned)y + nxy * (unsigned)z;
+  const unsigned nxy = lv.dnxy.d;
+  const unsigned i0 = blockIdx.x * 128u + threadIdx.x;
+  const bool valid = i0 < nxy;
+  const unsigned i = valid ? i0 : nxy - 1u;
+  const int y = (int)fdiv(i, lv.dnx), x = (int)(i - (unsigned)y * (unsigned)nx), z = blockIdx.y;
+  const unsigned n = i + nxy * (unsigned)z;
   // coordinates of the 3 x 3 x 3 neighbourhood, periodic wrap on every axis
   // (a walled axis has wall layers at both ends, never crossed by a link)
   const unsigned xo[3] = {(unsigned)(x == 0 ? nx - 1 : x - 1), (unsigned)x, (unsigned)(x == nx - 1 ? 0 : x + 1)};
@@ -506,8 +455,10 @@ __global__ void __launch_bounds__(128, BL_ONE_MINB) k_lb_step(LatticeView lv, Wa
       constexpr int r = decltype(R)::value;
       fin[r] = Store<S>::ld(pop + src_slot<PAR>(r, lv.N, n, xo, yo, zo));
     });
-    nbcv = lv.nbc[n];
-    puv = lv.pu[n];
+    if constexpr (CELLS) {
+      nbcv = lv.nbc[n];
+      puv = lv.pu[n];
+    }
   }
   // wall momentum of this thread: wall id, variable part, constant-part integers
   int wkey = -1;
@@ -518,10 +469,10 @@ __global__ void __launch_bounds__(128, BL_ONE_MINB) k_lb_step(LatticeView lv, Wa
   cl.p2 = -1;
   if (nbw & NB_FLUID) {
     const int xyz[3] = {x, y, z};
-    node_update<S, PAR, FORCE, TAU1>(lv, wa, n, xyz, xo, yo, zo, nbw, nbcv, puv,
-                                     [&](int r, unsigned) { return fin[r]; }, wkey, wF, wK, cl);
+    node_update<S, PAR, FORCE, TAU1, CELLS>(lv, wa, n, xyz, xo, yo, zo, nbw, nbcv, puv,
+                                            [&](int r, unsigned) { return fin[r]; }, wkey, wF, wK, cl);
   }
-  emit_links<TAU1>(lv, cl, n);
+  if constexpr (CELLS) emit_links<TAU1>(lv, cl, n);
   flush_wall_momentum(wa, wkey, wF, wK);
 }
 
@@ -604,7 +555,7 @@ __global__ void __launch_bounds__(128, BL_LB_MINB) k_lb_step_pipe(LatticeView lv
     zoff(z, zo);
     if (w[0] & NB_FLUID) {
       const int xyz[3] = {x, y, z};
-      node_update<float, PAR, FORCE, TAU1>(lv, wa, rowb + zo[1], xyz, xo, yo, zo, w[0], lv.nbc[rowb + zo[1]],
+      node_update<float, PAR, FORCE, TAU1, true>(lv, wa, rowb + zo[1], xyz, xo, yo, zo, w[0], lv.nbc[rowb + zo[1]],
                                            lv.pu[rowb + zo[1]],
                                            [&](int r, unsigned) { return stage[b][r][tx]; }, wkey, wF, wK, cl);
     }
@@ -658,13 +609,14 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
                : "memory");
 }
 
-template <class S, int PAR, bool FORCE, bool TAU1, int ZC, int TS>
+template <class S, int PAR, bool FORCE, bool TAU1, bool CELLS, int ZC, int TS>
 __global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView lv, WallAcc wa) {
   using D = D3Q19;
   __shared__ alignas(128) S sb[TS][Q][128];        // [stage][array][x]
   __shared__ alignas(128) uint32_t sw[TS][128];    // [stage][x] neighbour words
-  __shared__ alignas(128) float4 spu[TS][128];     // [stage][x] pending velocities
-  __shared__ alignas(128) uint32_t sc[TS][128];    // [stage][x] neighbour-cell words
+  constexpr int CW = CELLS ? 128 : 1;
+  __shared__ alignas(128) float4 spu[TS][CW];      // [stage][x] pending velocities
+  __shared__ alignas(128) uint32_t sc[TS][CW];     // [stage][x] neighbour-cell words
   __shared__ alignas(8) unsigned long long bar[TS];
   __shared__ int s_ok;
   const int nx = lv.nx, ny = lv.ny, nz = lv.nz;
@@ -693,7 +645,7 @@ __global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView 
     unsigned zo[3];
     zoff(z, zo);
     const unsigned bytes = (unsigned)W * (unsigned)sizeof(S);
-    mbar_expect_tx(&bar[s], Q * bytes + (unsigned)W * 24u);
+    mbar_expect_tx(&bar[s], Q * bytes + (unsigned)W * (CELLS ? 24u : 4u));
     sfor<0, Q>([&](auto R) {
       constexpr int r = decltype(R)::value;
       unsigned row;
@@ -702,8 +654,10 @@ __global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView 
       bulk_g2s(&sb[s][r][0], pop + row + (unsigned)x0, bytes, &bar[s]);
     });
     bulk_g2s(&sw[s][0], lv.nbm + yo[1] + zo[1] + (unsigned)x0, (unsigned)W * 4u, &bar[s]);
-    bulk_g2s(&spu[s][0], lv.pu + yo[1] + zo[1] + (unsigned)x0, (unsigned)W * 16u, &bar[s]);
-    bulk_g2s(&sc[s][0], lv.nbc + yo[1] + zo[1] + (unsigned)x0, (unsigned)W * 4u, &bar[s]);
+    if constexpr (CELLS) {
+      bulk_g2s(&spu[s][0], lv.pu + yo[1] + zo[1] + (unsigned)x0, (unsigned)W * 16u, &bar[s]);
+      bulk_g2s(&sc[s][0], lv.nbc + yo[1] + zo[1] + (unsigned)x0, (unsigned)W * 4u, &bar[s]);
+    }
   };
   if (tx == 0) {
     for (int k = 0; k < TS; ++k) mbar_init(&bar[k], 1);
@@ -735,8 +689,8 @@ __global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView 
     cl.p2 = -1;
     if (w & NB_FLUID) {
       const int xyz[3] = {x, y, z};
-      node_update<S, PAR, FORCE, TAU1>(
-          lv, wa, n, xyz, xo, yo, zo, w, sc[s][tx], spu[s][tx],
+      node_update<S, PAR, FORCE, TAU1, CELLS>(
+          lv, wa, n, xyz, xo, yo, zo, w, CELLS ? sc[s][CELLS ? tx : 0] : NBC_MIXED, spu[s][CELLS ? tx : 0],
           [&](int r, unsigned slot) -> float {
             if (PAR == 0 || r == 0) return Store<S>::ld(&sb[s][r][tx]);
             int j = tx - D::cx(r);
@@ -745,11 +699,15 @@ __global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView 
           },
           wkey, wF, wK, cl);
     }
-    const LinkSlot sl = reserve_links(lv, cl);
-    const LinkSlot sl2 = reserve_slots(lv, cl.p2);
-    __syncthreads();  // stage s is read: free for refill (the atomics' round trip overlaps it)
-    write_links(lv, cl, n, sl);
-    write_second<TAU1>(lv, cl, n, sl2);
+    if constexpr (CELLS) {
+      const LinkSlot sl = reserve_links(lv, cl);
+      const LinkSlot sl2 = reserve_slots(lv, cl.p2);
+      __syncthreads();  // stage s is read: free for refill (the atomics' round trip overlaps it)
+      write_links(lv, cl, n, sl);
+      write_second<TAU1>(lv, cl, n, sl2);
+    } else {
+      __syncthreads();
+    }
   }
   if (z < ze && tx == 0) {
     // gave up: let the copies still in flight land before the block exits
@@ -770,7 +728,8 @@ static void launch_pipe(const LatticeView &lv, dim3 grid, dim3 block, const Wall
 template <class S, int PAR, bool FORCE, bool TAU1, int ZC, int TS>
 static void launch_bulk(const LatticeView &lv, dim3 grid, const WallAcc &wa, cudaStream_t st) {
   const dim3 gp((lv.nx + 127) / 128, grid.y, (grid.z + ZC - 1) / ZC);
-  k_lb_step_bulk<S, PAR, FORCE, TAU1, ZC, TS><<<gp, 128, 0, st>>>(lv, wa);
+  if (lv.rec) k_lb_step_bulk<S, PAR, FORCE, TAU1, true, ZC, TS><<<gp, 128, 0, st>>>(lv, wa);
+  else k_lb_step_bulk<S, PAR, FORCE, TAU1, false, ZC, TS><<<gp, 128, 0, st>>>(lv, wa);
 }
 
 // The persistent row sweep: a grid of as many blocks as the device holds at
@@ -898,7 +857,7 @@ __global__ void __launch_bounds__(128, BL_ROWS_MINB) k_lb_step_rows(LatticeView 
     if (w & NB_FLUID) {
       const int xyz[3] = {x, g.y, g.z};
       const int W = g.W;
-      node_update<S, PAR, FORCE, TAU1>(
+      node_update<S, PAR, FORCE, TAU1, true>(
           lv, wa, n, xyz, xo, yo, zo, w, sc[s][tx], spu[s][tx],
           [&](int r, unsigned slot) -> float {
             if (PAR == 0 || r == 0) return Store<S>::ld(&sb[s][r][tx]);
@@ -980,7 +939,9 @@ static void launch_lb_variant(const LatticeView &lv, dim3 grid, dim3 block, cons
     if (lv.sweep == 4) return launch_bulk<S, PAR, FORCE, TAU1, 4, BL_BULK_TS>(lv, grid, wa, st);
     if (lv.sweep == 5) return launch_rows<S, PAR, FORCE, TAU1>(lv, wa, st);
   }
-  k_lb_step<S, PAR, FORCE, TAU1><<<grid, block, 0, st>>>(lv, wa);
+  const dim3 g1((lv.dnxy.d + 127u) / 128u, lv.nz);
+  if (lv.rec) k_lb_step<S, PAR, FORCE, TAU1, true><<<g1, 128, 0, st>>>(lv, wa);
+  else k_lb_step<S, PAR, FORCE, TAU1, false><<<g1, 128, 0, st>>>(lv, wa);
 }
 
 template <class S, int PAR, bool FORCE>

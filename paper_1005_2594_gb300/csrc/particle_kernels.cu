@@ -695,13 +695,7 @@ constexpr int LT = 128;  // threads of a link-reduction block
 __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView lv, PartView pv) {
   __shared__ float shf[LT / 32][27];
   __shared__ int shi[LT / 32][6];
-  __shared__ float4 cw[Q];  // (c_x, c_y, c_z, w_r) of each direction, for the masks' bits
   const int p = blockIdx.x;
-  if (threadIdx.x < Q) {
-    const int r = threadIdx.x;
-    cw[r] = make_float4((float)D3::cx(r), (float)D3::cy(r), (float)D3::cz(r), (float)D3::m(r) / 36.0f);
-  }
-  __syncthreads();
   const int nrec = min(lv.rec_count[p], lv.rec_cap);
   const float4 k0 = pv.kin[3 * p], k1 = pv.kin[3 * p + 1], k2 = pv.kin[3 * p + 2];
   const int Xi[3] = {(int)k0.w, (int)k1.w, (int)k2.w};
@@ -733,19 +727,22 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
     // again from the node's moments (drho, u, uu, uF), else the sweep's sums
     float Fr[3];
     if (tau1) {
-      const float ux = r0.w, uy = r1.x, uz = r1.y, uu = r1.z, uF = r1.w;
       const float Fx = lv.has_force ? rho * lv.g[0] : 0.f, Fy = lv.has_force ? rho * lv.g[1] : 0.f,
                   Fz = lv.has_force ? rho * lv.g[2] : 0.f;
+      const Collide ck = collide_coeffs<true>(r0.z, rho, r0.w, r1.x, r1.y, r1.z, 1.0f, Fx, Fy, Fz, r1.w);
       Fr[0] = Fr[1] = Fr[2] = 0.f;
-      for (uint32_t mm = m; mm; mm &= mm - 1u) {
-        const float4 c = cw[__ffs(mm) - 1];
-        const float cu = c.x * ux + c.y * uy + c.z * uz;
-        const float cF = c.x * Fx + c.y * Fy + c.z * Fz;
-        const float fs2 = 2.0f * post_tau1(c.w, r0.z, lv.rho0, cu, uu, lv.has_force != 0, cF, uF, 0.5f);
-        Fr[0] += c.x * fs2;
-        Fr[1] += c.y * fs2;
-        Fr[2] += c.z * fs2;
-      }
+      sfor<0, 9>([&](auto P) {
+        constexpr int r = 2 * decltype(P)::value + 1;
+        float fr, fb;
+        collide_pair<r, true>(ck, fr, fb);
+        // 2 f~*_r c_r of r and of rbar (c_rbar = -c_r)
+        float v = (m >> r) & 1u ? fr : 0.f;
+        if ((m >> (r + 1)) & 1u) v -= fb;
+        v *= 2.0f * (float)D3::m(r) / 36.0f;
+        if constexpr (D3::cx(r) != 0) Fr[0] += D3::cx(r) > 0 ? v : -v;
+        if constexpr (D3::cy(r) != 0) Fr[1] += D3::cy(r) > 0 ? v : -v;
+        if constexpr (D3::cz(r) != 0) Fr[2] += D3::cz(r) > 0 ? v : -v;
+      });
     } else {
       Fr[0] = r0.w;
       Fr[1] = r1.x;
@@ -1512,7 +1509,9 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
 // bit r neighbour x + c_r solid, NB_WALL / NB_CELL some solid neighbour is a
 // wall / a cell; for a cell node its contact links (bit r: the neighbour is a
 // wall node or another cell's); zero for wall nodes
-__device__ __forceinline__ uint32_t node_word(const LatticeView &lv, int x, int y, int z, uint32_t &cellw) {
+// (the mixed word of a fluid node is written here, to node on_node)
+__device__ __forceinline__ uint32_t node_word(const LatticeView &lv, int x, int y, int z, unsigned on_node,
+                                              uint32_t &cellw) {
   using D = D3Q19;
   const unsigned nx = (unsigned)lv.nx, nxy = (unsigned)lv.nx * (unsigned)lv.ny;
   cellw = NBC_MIXED;
@@ -1550,6 +1549,7 @@ __device__ __forceinline__ uint32_t node_word(const LatticeView &lv, int x, int 
     }
   });
   if (first >= 0 && !mixed) cellw = (uint32_t)first;
+  if (mixed && (solid & ~wall)) lv.nbx[on_node] = mixed_word(on);
   return NB_FLUID | solid | (wall ? NB_WALL : 0u) | ((solid & ~wall) ? NB_CELL : 0u);
 }
 
@@ -1574,7 +1574,7 @@ __global__ void k_nbm_update(LatticeView lv, ChangeList chg) {
     }
     uint32_t cw;
     const unsigned nn = node_of(lv, xyz[0], xyz[1], xyz[2]);
-    lv.nbm[nn] = node_word(lv, xyz[0], xyz[1], xyz[2], cw);
+    lv.nbm[nn] = node_word(lv, xyz[0], xyz[1], xyz[2], nn, cw);
     lv.nbc[nn] = cw;
   }
 }
