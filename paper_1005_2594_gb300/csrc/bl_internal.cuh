@@ -175,6 +175,7 @@ struct PartView {
   int n;
   double *X, *q, *V, *L, *Om;
   double *o;         // exact FP64 symmetry axis of the current q, n x 3
+  float4 *axis;      // n: the current axis in FP32
   float *oprev;      // n x 3 axis before the last move (FP32): the claims' old ellipsoid
   float4 *kin;       // kinematics of the current step, 3 float4 per cell:
                      //   (f.x, f.y, f.z, Xi.x), (V, Xi.y), (W, Xi.z); X = Xi + f, Xi = rint(X)
@@ -198,6 +199,7 @@ struct PartView {
   int bfc, move;
   double le_dr;  // Lees-Edwards: reflect a cell within le_dr of the sheared plane (0: no shear)
   double inv_rpar2, inv_rperp2, R_par, R_perp;
+  float inv_rpar2_f, inv_rperp2_f, kk_f;  // 1 / R^2 in FP32, kk = 1 / R_par^2 - 1 / R_perp^2
   float sig_par, sig_perp, eps, eps_w, mu, nu, chi_prime, r_cut;
   float chi, sigbar, sigbar_w, chi_w, sigw_max;
   double chi_d, sigbar_d, sigbar_w_d, chi_w_d;  // the same in FP64 (contact geometry)

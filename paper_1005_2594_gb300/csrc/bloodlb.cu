@@ -347,7 +347,7 @@ extern "C" int bl_walls_set(bl_ctx *c, const uint8_t *mask) {
 
 static void free_particles(bl_ctx *c) {
   PartView &pv = c->pv;
-  void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
+  void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.axis, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
                   pv.touched, pv.touched_count, pv.lsum, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink, pv.Ftot,
                   pv.Ttot, pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
                   c->chg.count, c->chg.items, c->lv.rec, c->lv.rec_count};
@@ -377,6 +377,8 @@ static int alloc_particles(bl_ctx *c, int n) {
     CU(cudaMalloc(d, n3));
     CU(cudaMemsetAsync(*d, 0, n3, c->stream));
   }
+  CU(cudaMalloc(&pv.axis, sizeof(float4) * (size_t)n));
+  CU(cudaMemsetAsync(pv.axis, 0, sizeof(float4) * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.oprev, sizeof(float) * 3 * (size_t)n));
   CU(cudaMemsetAsync(pv.oprev, 0, sizeof(float) * 3 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.q, sizeof(double) * 4 * (size_t)n));
@@ -478,6 +480,9 @@ static void fill_particle_constants(bl_ctx *c) {
                                              : fmax(pp.sig_perp, fmax(pp.R_perp, pp.R_par) + 1.0));
   pv.inv_rpar2 = 1.0 / (pp.R_par * pp.R_par);
   pv.inv_rperp2 = 1.0 / (pp.R_perp * pp.R_perp);
+  pv.inv_rpar2_f = (float)pv.inv_rpar2;
+  pv.inv_rperp2_f = (float)pv.inv_rperp2;
+  pv.kk_f = (float)(pv.inv_rpar2 - pv.inv_rperp2);
   pv.R_par = pp.R_par;
   pv.R_perp = pp.R_perp;
   pv.sig_par = (float)pp.sig_par;

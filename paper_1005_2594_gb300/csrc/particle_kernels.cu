@@ -31,9 +31,11 @@
 //
 // FP64 is used only where the state needs it (positions, velocities, angular
 // momenta, the exact inside test near a surface, the contact geometry of the
-// potentials); on this GPU a one-lane FP64 instruction costs a full warp
-// slot of a narrow pipe, so sums, the 6 x 6 solve and the rotation increment
-// are FP32 around FP64 reference values.
+// potentials); on this GPU an FP64 instruction holds the SM's FP64 pipe for 16
+// cycles whatever number of lanes it has, so sums, the 6 x 6 solve and the
+// rotation increment are FP32 around FP64 reference values, and the kernels
+// that test nodes against ellipsoids read each cell's position (node + FP32
+// fraction) and axis in the FP32 form the solve leaves them.
 #include <climits>
 
 #include "bl_internal.cuh"
@@ -133,10 +135,38 @@ __global__ void k_cl_sort(CellListView cl) {
 // Contact geometry in FP64.  In contact the overlap h = 1 - r / sigma is a
 // small difference of O(1) numbers (h ~ 1e-2), and the force is
 // proportional to it: rounding r and sigma to FP32 (~1e-7) would put ~1e-5
-// into the force.  So r (from the FP64 positions), the angles a, b, c, the
-// shape function S, sigma and h are formed in FP64; the strength, its
+// into the force.  With sigma = sigma_bar / sqrt(S) and P = r^2 S,
+//   h = (sigma_bar^2 - P) / (sigma_bar (sigma_bar + sqrt(P))),
+// so the one difference is formed in FP64, from products of the positions and
+// axes without a root or a normalised vector, and its quotient in FP32.  Two
+// FP64 reciprocals (Newton from the FP32 one) replace six roots and divisions
+// of some 20 FP64 instructions each: the contact geometry was 170 FP64
+// instructions per warp, each holding the SM's FP64 pipe for 16 cycles, and
+// bound the kernel (104 us on 256^3 with 8446 cells).  The strength, its
 // derivatives and the force and torque, which multiply h without cancelling
-// it, in FP32.
+// it, are FP32.
+
+// 1 / x and 1 / sqrt(x) in FP64 to about an ulp, for x within FP32's range
+// (rsqrt64: the root and quotient themselves below it)
+__device__ __forceinline__ double rcp64(double x) {
+  double y = (double)(1.0f / (float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+  if (!(x > 1e-30)) return 1.0 / sqrt(x);
+  double y = (double)rsqrtf((float)x);
+  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+}
+__device__ __forceinline__ double dot64(const double a[3], const double b[3]) {
+  return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
+}
+
+// h from sigma_bar^2 - P (> 0) and P
+__device__ __forceinline__ float overlap(double D, double P, float sigbar) {
+  return (float)D / (sigbar * (sigbar + sqrtf((float)P)));
+}
 
 // FP32 test of a pair against its contact distance (Eq. sigma) with a
 // relative margin of 1e-4: false only for pairs certainly out of contact
@@ -155,26 +185,24 @@ __device__ __forceinline__ bool near_contact(const float r[3], float r2, const f
 // cell-cell pair, force and torque on i; r = X_j - X_i (Eqs. phi, epsilon,
 // sigma; the Gay-Berne factor eps2^mu of the variant)
 __device__ __forceinline__ void bp_pair(const double rd[3], const double oid[3], const double ojd[3],
-                                        const PartView &pv, float F[3], float T[3]) {
-  const double r2d = rd[0] * rd[0] + rd[1] * rd[1] + rd[2] * rd[2];
-  if (!(r2d > 0.0)) return;
-  const double rld = sqrt(r2d), ird = 1.0 / rld;
-  const double rhd[3] = {rd[0] * ird, rd[1] * ird, rd[2] * ird};
-  const double ad = rhd[0] * oid[0] + rhd[1] * oid[1] + rhd[2] * oid[2];
-  const double bd = rhd[0] * ojd[0] + rhd[1] * ojd[1] + rhd[2] * ojd[2];
-  const double cd = oid[0] * ojd[0] + oid[1] * ojd[1] + oid[2] * ojd[2];
-  const double apd = ad + bd, amd = ad - bd;
-  const double Sd = 1.0 - 0.5 * pv.chi_d * (apd * apd / (1.0 + pv.chi_d * cd) + amd * amd / (1.0 - pv.chi_d * cd));
-  const double sigd = pv.sigbar_d / sqrt(Sd);
-  if (rld >= sigd) return;
-  const float h = (float)(1.0 - rld / sigd);
-  const float rl = (float)rld, ir = (float)ird, sigma = (float)sigd, S = (float)Sd;
-  const float rh[3] = {(float)rhd[0], (float)rhd[1], (float)rhd[2]};
-  const float oi[3] = {(float)oid[0], (float)oid[1], (float)oid[2]};
-  const float oj[3] = {(float)ojd[0], (float)ojd[1], (float)ojd[2]};
-  const float a = (float)ad, b = (float)bd, c = (float)cd;
+                                        const float oi[3], const float oj[3], const PartView &pv, float F[3],
+                                        float T[3]) {
+  const double r2 = dot64(rd, rd);
+  if (!(r2 > 0.0)) return;
+  const double A = dot64(rd, oid), B = dot64(rd, ojd), cd = dot64(oid, ojd);
+  const double Ap = A + B, Am = A - B, qp = fma(pv.chi_d, cd, 1.0), qm = fma(-pv.chi_d, cd, 1.0);
+  // (A + B)^2 / (1 + chi c) + (A - B)^2 / (1 - chi c)
+  const double X = fma(Ap * Ap, qm, Am * Am * qp) * rcp64(qp * qm);
+  const double P = fma(-0.5 * pv.chi_d, X, r2), D = pv.sigbar_d * pv.sigbar_d - P;
+  if (!(D > 0.0)) return;
+  const double ird = rsqrt64(r2);
+  const float h = overlap(D, P, pv.sigbar);
+  const float rl = (float)(r2 * ird), ir = (float)ird, S = (float)(P * (ird * ird));
+  const float sigma = pv.sigbar / sqrtf(S);
+  const float rh[3] = {(float)(rd[0] * ird), (float)(rd[1] * ird), (float)(rd[2] * ird)};
+  const float a = (float)(A * ird), b = (float)(B * ird), c = (float)cd;
   const float chi = pv.chi;
-  const float ap = (float)apd, am = (float)amd;
+  const float ap = (float)(Ap * ird), am = (float)(Am * ird);
   const float dp = 1.0f + chi * c, dm = 1.0f - chi * c;
   const float e1 = 1.0f - chi * chi * c * c;
   float eps = pv.eps * (pv.nu == 1.0f ? rsqrtf(e1) : powf(e1, -0.5f * pv.nu));
@@ -210,22 +238,20 @@ __device__ __forceinline__ void bp_pair(const double rd[3], const double oid[3],
 }
 
 // cell-wall sphere (Eq. sigmaw), force and torque on the cell; r = x_wall - X
-__device__ __forceinline__ void bp_wall(const double rd[3], const double oid[3], const PartView &pv, float F[3],
-                                        float T[3]) {
-  const double r2d = rd[0] * rd[0] + rd[1] * rd[1] + rd[2] * rd[2];
-  if (!(r2d > 0.0)) return;
-  const double rld = sqrt(r2d), ird = 1.0 / rld;
-  const double rhd[3] = {rd[0] * ird, rd[1] * ird, rd[2] * ird};
-  const double ad = rhd[0] * oid[0] + rhd[1] * oid[1] + rhd[2] * oid[2];
-  const double Dd = 1.0 - pv.chi_w_d * ad * ad;
-  const double sigd = pv.sigbar_w_d / sqrt(Dd);
-  if (rld >= sigd) return;
-  const float h = (float)(1.0 - rld / sigd);
-  const float rl = (float)rld, ir = (float)ird, sigma = (float)sigd, D = (float)Dd, a = (float)ad;
-  const float rh[3] = {(float)rhd[0], (float)rhd[1], (float)rhd[2]};
-  const float oi[3] = {(float)oid[0], (float)oid[1], (float)oid[2]};
+__device__ __forceinline__ void bp_wall(const double rd[3], const double oid[3], const float oi[3],
+                                        const PartView &pv, float F[3], float T[3]) {
+  const double r2 = dot64(rd, rd);
+  if (!(r2 > 0.0)) return;
+  const double A = dot64(rd, oid);
+  const double P = fma(-pv.chi_w_d * A, A, r2), D = pv.sigbar_w_d * pv.sigbar_w_d - P;
+  if (!(D > 0.0)) return;
+  const double ird = rsqrt64(r2);
+  const float h = overlap(D, P, pv.sigbar_w);
+  const float rl = (float)(r2 * ird), ir = (float)ird, S = (float)(P * (ird * ird)), a = (float)(A * ird);
+  const float sigma = pv.sigbar_w / sqrtf(S);
+  const float rh[3] = {(float)(rd[0] * ird), (float)(rd[1] * ird), (float)(rd[2] * ird)};
   const float eps = pv.eps_w;
-  const float dsig_a = sigma * pv.chi_w * a / D;
+  const float dsig_a = sigma * pv.chi_w * a / S;
   const float phi_r = -2.0f * eps * h / sigma;
   const float phi_a = 2.0f * eps * h * rl / (sigma * sigma) * dsig_a;
   for (int m = 0; m < 3; ++m) F[m] += phi_r * rh[m] + phi_a * (oi[m] - a * rh[m]) * ir;
@@ -343,42 +369,6 @@ __device__ __forceinline__ unsigned node_of(const LatticeView &lv, int x, int y,
   return (unsigned)x + (unsigned)lv.nx * ((unsigned)y + (unsigned)lv.ny * z);
 }
 
-// walks the nodes of an inclusive box, CB threads at a time, without
-// dividing per node: thread t starts at node t and advances by CB
-struct BoxIter {
-  int bx, by, bz, total;
-  int ix, iy, iz, dx, dy, dz;
-  __device__ void init(const int lo[3], const int hi[3]) {
-    bx = hi[0] - lo[0] + 1;
-    by = hi[1] - lo[1] + 1;
-    bz = hi[2] - lo[2] + 1;
-    total = (bx > 0 && by > 0 && bz > 0) ? bx * by * bz : 0;
-    if (!total) return;
-    const int t = threadIdx.x;
-    iz = t / (bx * by);
-    iy = (t / bx) % by;
-    ix = t % bx;
-    dz = CB / (bx * by);
-    dy = (CB / bx) % by;
-    dx = CB % bx;
-  }
-  __device__ void advance() {
-    ix += dx;
-    int c = 0;
-    if (ix >= bx) {
-      ix -= bx;
-      c = 1;
-    }
-    iy += dy + c;
-    c = 0;
-    if (iy >= by) {
-      iy -= by;
-      c = 1;
-    }
-    iz += dz + c;
-  }
-};
-
 // slot where the sweep of parity par bounced direction r of fluid node y
 __device__ __forceinline__ unsigned bounce_slot(const LatticeView &lv, int par, unsigned y, const int yc[3], int r) {
   if (par == 0) {
@@ -420,24 +410,33 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
   const float4 a0 = pv.kin[3 * i], a1 = pv.kin[3 * i + 1], a2 = pv.kin[3 * i + 2];
   const int Xi[3] = {(int)a0.w, (int)a1.w, (int)a2.w};
   const float fi[3] = {a0.x, a0.y, a0.z};
-  // FP64 state of the step's start (the solve rewrites it only after the join)
-  const double Xd[3] = {pv.X[3 * i], pv.X[3 * i + 1], pv.X[3 * i + 2]};
-  const double oid[3] = {pv.o[3 * i], pv.o[3 * i + 1], pv.o[3 * i + 2]};
-  const double fd[3] = {Xd[0] - (double)Xi[0], Xd[1] - (double)Xi[1], Xd[2] - (double)Xi[2]};  // exact
-  const float oif[3] = {(float)oid[0], (float)oid[1], (float)oid[2]};
+  const float4 ax = pv.axis[i];
+  const float oif[3] = {ax.x, ax.y, ax.z};
   const int dims[3] = {lv.nx, lv.ny, lv.nz};
   float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
+  // the FP64 state (of the step's start: the solve rewrites it only after the
+  // join) is read where a contact is evaluated; the periodic image comes from
+  // the nearest nodes, in integers
   auto pair_force = [&](int j) {
+    const int Xj[3] = {(int)pv.kin[3 * j].w, (int)pv.kin[3 * j + 1].w, (int)pv.kin[3 * j + 2].w};
     double rd[3];
-    for (int m = 0; m < 3; ++m) rd[m] = min_image_exact(__dsub_rn(pv.X[3 * j + m], Xd[m]), dims[m], lv.per[m]);
+    for (int m = 0; m < 3; ++m) {
+      const int d = Xj[m] - Xi[m];
+      rd[m] = (pv.X[3 * j + m] - pv.X[3 * i + m]) + (double)(imin_image(d, dims[m], lv.per[m]) - d);
+    }
+    const double oid[3] = {pv.o[3 * i], pv.o[3 * i + 1], pv.o[3 * i + 2]};
     const double ojd[3] = {pv.o[3 * j], pv.o[3 * j + 1], pv.o[3 * j + 2]};
-    bp_pair(rd, oid, ojd, pv, F, T);
+    const float4 aj = pv.axis[j];
+    const float oj[3] = {aj.x, aj.y, aj.z};
+    bp_pair(rd, oid, ojd, oif, oj, pv, F, T);
   };
   // the wall node at offsets (dx, oy, oz) from rint(X); queued packed in
   // 3 x 10 bits (offsets within +-511, else evaluated where found)
   auto wall_force = [&](int dx, int oy, int oz) {
-    const double rd[3] = {(double)dx - fd[0], (double)oy - fd[1], (double)oz - fd[2]};
-    bp_wall(rd, oid, pv, F, T);
+    const double oid[3] = {pv.o[3 * i], pv.o[3 * i + 1], pv.o[3 * i + 2]};
+    const double rd[3] = {(double)(dx + Xi[0]) - pv.X[3 * i], (double)(oy + Xi[1]) - pv.X[3 * i + 1],
+                          (double)(oz + Xi[2]) - pv.X[3 * i + 2]};
+    bp_wall(rd, oid, oif, pv, F, T);
   };
   if (threadIdx.x < 27) {
     const int bin = cl.bin_of[i];
@@ -468,7 +467,8 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
         // relative, far inside the margin): only pairs at or within contact
         // take the FP64 geometry
         if (r2 >= rc2 || r2 > smax2) continue;
-        const float oj[3] = {(float)pv.o[3 * j], (float)pv.o[3 * j + 1], (float)pv.o[3 * j + 2]};
+        const float4 aj = pv.axis[j];
+        const float oj[3] = {aj.x, aj.y, aj.z};
         if (!near_contact(r, r2, oif, oj, pv)) continue;
         const int q = atomicAdd(&s_np, 1);
         if (q < FQ_PAIR) s_pair[q] = j;
@@ -624,33 +624,50 @@ __device__ void aabb(const PartView &pv, const double X[3], const double o[3], i
   }
 }
 
-// inside test: FP32 filter, exact FP64 re-evaluation near the surface
-__device__ __forceinline__ bool inside_cell(int x, int y, int z, const double *X, const double *o, const float *Xf,
-                                            const int *Xi, const float *of, const PartView &pv, const LatticeView &lv) {
-  const float d0 = (float)imin_image(x - Xi[0], lv.nx, lv.per[0]) - Xf[0];
-  const float d1 = (float)imin_image(y - Xi[1], lv.ny, lv.per[1]) - Xf[1];
-  const float d2 = (float)imin_image(z - Xi[2], lv.nz, lv.per[2]) - Xf[2];
-  const float dpar = d0 * of[0] + d1 * of[1] + d2 * of[2];
-  const float dd = d0 * d0 + d1 * d1 + d2 * d2;
-  const float s = dpar * dpar * (float)pv.inv_rpar2 + (dd - dpar * dpar) * (float)pv.inv_rperp2;
-  if (fabsf(s - 1.0f) >= INSIDE_MARGIN) return s < 1.0f;
-  return inside_exact(x, y, z, X, o, pv.inv_rpar2, pv.inv_rperp2, lv);
-}
-
+// position (nearest node + fraction) and axis of a cell in FP32, as the solve
+// leaves them (kin: the kinematics that belong to the position, axis).  Formed
+// from the FP64 state by every thread, they took 68 % of the FP64 pipe in the
+// claims and most of the owner search.
 struct CellGeo {
-  double X[3], o[3];
   float Xf[3], of[3];
   int Xi[3];
 };
 
-__device__ __forceinline__ void cell_geo(const PartView &pv, int p, CellGeo &g) {
-  for (int k = 0; k < 3; ++k) {
-    g.X[k] = pv.X[3 * p + k];
-    g.o[k] = pv.o[3 * p + k];
-    g.Xi[k] = (int)rint(g.X[k]);
-    g.Xf[k] = (float)(g.X[k] - (double)g.Xi[k]);
-    g.of[k] = (float)g.o[k];
-  }
+__device__ __forceinline__ void cell_geo(const PartView &pv, const float4 *kin, int p, CellGeo &g) {
+  const float4 a = kin[3 * p], o = pv.axis[p];
+  g.Xf[0] = a.x;
+  g.Xf[1] = a.y;
+  g.Xf[2] = a.z;
+  g.Xi[0] = (int)a.w;
+  g.Xi[1] = (int)kin[3 * p + 1].w;
+  g.Xi[2] = (int)kin[3 * p + 2].w;
+  g.of[0] = o.x;
+  g.of[1] = o.y;
+  g.of[2] = o.z;
+}
+
+// inside test of cell p: FP32 filter, exact FP64 re-evaluation near the surface
+__device__ __forceinline__ bool inside_cell(int x, int y, int z, int p, const CellGeo &g, const PartView &pv,
+                                            const LatticeView &lv) {
+  const float d0 = (float)imin_image(x - g.Xi[0], lv.nx, lv.per[0]) - g.Xf[0];
+  const float d1 = (float)imin_image(y - g.Xi[1], lv.ny, lv.per[1]) - g.Xf[1];
+  const float d2 = (float)imin_image(z - g.Xi[2], lv.nz, lv.per[2]) - g.Xf[2];
+  const float dpar = d0 * g.of[0] + d1 * g.of[1] + d2 * g.of[2];
+  const float dd = d0 * d0 + d1 * d1 + d2 * d2;
+  const float s = dpar * dpar * pv.inv_rpar2_f + (dd - dpar * dpar) * pv.inv_rperp2_f;
+  if (fabsf(s - 1.0f) >= INSIDE_MARGIN) return s < 1.0f;
+  return inside_exact(x, y, z, pv.X + 3 * p, pv.o + 3 * p, pv.inv_rpar2, pv.inv_rperp2, lv);
+}
+
+// lever arm of a node from the centre of cell p in FP64: the image of the node
+// nearest the cell chosen in integers, one conversion and one subtraction per
+// axis
+__device__ __forceinline__ void arm64(const LatticeView &lv, const PartView &pv, const float4 *kin, int p,
+                                      const int xyz[3], double a[3]) {
+  const int Xi[3] = {(int)kin[3 * p].w, (int)kin[3 * p + 1].w, (int)kin[3 * p + 2].w};
+  const int dims[3] = {lv.nx, lv.ny, lv.nz};
+  for (int k = 0; k < 3; ++k)
+    a[k] = __dsub_rn((double)(Xi[k] + imin_image(xyz[k] - Xi[k], dims[k], lv.per[k])), pv.X[3 * p + k]);
 }
 
 // ---------------------------------------------------------------------------
@@ -937,6 +954,7 @@ __global__ void k_solve(LatticeView lv, PartView pv) {
     double o_new[3];
     axis_exact(q, o_new);
     for (int k = 0; k < 3; ++k) pv.o[3 * p + k] = o_new[k];
+    pv.axis[p] = make_float4((float)o_new[0], (float)o_new[1], (float)o_new[2], 0.f);
     bool finite = true;
     for (int k = 0; k < 3; ++k) finite = finite && isfinite(X[k]) && isfinite(o_new[k]);
     // a cell faster than half a node per step is far outside the method's
@@ -1105,6 +1123,7 @@ __global__ void k_set_state(LatticeView lv, PartView pv, int mode) {
     pv.oprev[3 * p + k] = (float)(mode == 2 ? o_old[k] : o_new[k]);
     pv.o[3 * p + k] = o_new[k];
   }
+  pv.axis[p] = make_float4((float)o_new[0], (float)o_new[1], (float)o_new[2], 0.f);
   write_kin(pv, p, X, V, W);
   int lo[3], hi[3], lo2[3], hi2[3];
   aabb(pv, X, o_new, lo, hi);
@@ -1205,7 +1224,7 @@ __global__ void __launch_bounds__(PB, BL_CLAIMS_MINB) k_claims(LatticeView lv, P
   const int by = pv.box[6 * p + 4] - lo1 + 1, bz = pv.box[6 * p + 5] - lo2 + 1;
   const int rows = (by > 0 && bz > 0) ? by * bz : 0;
   CellGeo g;
-  cell_geo(pv, p, g);
+  cell_geo(pv, pv.kin_next, p, g);
   const bool has_old = mode != 1;
   int Xo[3] = {0, 0, 0};
   float xfo[3] = {0.f, 0.f, 0.f}, oo[3] = {0.f, 0.f, 0.f};
@@ -1219,7 +1238,7 @@ __global__ void __launch_bounds__(PB, BL_CLAIMS_MINB) k_claims(LatticeView lv, P
     xfo[2] = k0.z;
     for (int k = 0; k < 3; ++k) oo[k] = pv.oprev[3 * p + k];
   }
-  const float ip = (float)pv.inv_rperp2, kk = (float)(pv.inv_rpar2 - pv.inv_rperp2);
+  const float ip = pv.inv_rperp2_f, kk = pv.kk_f;
   const int shift = imin_image(Xo[0] - g.Xi[0], lv.nx, lv.per[0]);  // old rint(X_x) from the new one
   // offsets of one period (periodic x) or of the lattice (walled x)
   const int imin = lv.per[0] ? -(lv.nx / 2) : -g.Xi[0];
@@ -1278,12 +1297,12 @@ __global__ void __launch_bounds__(PB, BL_CLAIMS_MINB) k_claims(LatticeView lv, P
       const int ow = lv.owner[idx];
       int mark = 0;
       if (ow == p) {
-        if (!inside_cell(x, y, z, g.X, g.o, g.Xf, g.Xi, g.of, pv, lv)) {
+        if (!inside_cell(x, y, z, p, g, pv, lv)) {
           atomicMin(&claim[idx], CLAIM_TOUCHED);
           mark = 1;
         }
       } else if (ow == FLUID) {
-        if (inside_cell(x, y, z, g.X, g.o, g.Xf, g.Xi, g.of, pv, lv)) {
+        if (inside_cell(x, y, z, p, g, pv, lv)) {
           atomicMin(&claim[idx], p);
           mark = 1;
         }
@@ -1325,8 +1344,8 @@ __device__ int lowest_cover(const LatticeView &lv, const PartView &pv, const Cel
     for (int k = cl.start[b]; k < e; ++k) {
       const int j = cl.ids[k];
       CellGeo g;
-      cell_geo(pv, j, g);
-      if (inside_cell(x, y, z, g.X, g.o, g.Xf, g.Xi, g.of, pv, lv)) {
+      cell_geo(pv, pv.kin_next, j, g);
+      if (inside_cell(x, y, z, j, g, pv, lv)) {
         best = j;
         break;
       }
@@ -1345,6 +1364,12 @@ __device__ __forceinline__ void atomic_add3(double *a, const double v[3]) {
   atomicAdd(a + 2, v[2]);
 }
 
+// One block per cell over its touched nodes.  The new owners are decided first
+// and the changed nodes queued, covered ones (fluid to cell) from the front,
+// uncovered ones (a cell leaves) from the back; then each kind is worked off
+// by warps of its own, so that the FP64 of the momentum balance is issued once
+// for up to 32 nodes instead of for the few of one warp's nodes that take a
+// branch.
 template <class S>
 __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv, CellListView cl, int *claim,
                                                       ChangeList chg, int par_next, int impulses) {
@@ -1358,19 +1383,22 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
   const int nt = pv.touched_count[p];
   const int lane = threadIdx.x & 31;
   S *pop = reinterpret_cast<S *>(lv.pop);
-  const int dims[3] = {lv.nx, lv.ny, lv.nz};
   __shared__ int s_need[PB], s_res[PB];
-  __shared__ int s_ns;
+  __shared__ unsigned long long s_xyz[PB];
+  __shared__ int s_old[PB], s_new[PB];
+  __shared__ int s_ns, s_nc, s_nu;
   for (int t0 = 0; t0 < nt; t0 += PB) {
     const int t = t0 + threadIdx.x;
     int old = 0, nw = 0, xyz[3] = {0, 0, 0};
     bool changed = false, act = false, need = false;
     unsigned idx = 0;
-    if (threadIdx.x == 0) s_ns = 0;
+    unsigned long long tv = 0ull;
+    if (threadIdx.x == 0) s_ns = s_nc = s_nu = 0;
     __syncthreads();
     if (t < nt) {
       int r_unused;
-      unpack_xyzr(t0 == 0 ? tv0 : touched[t], xyz, r_unused);
+      tv = t0 == 0 ? tv0 : touched[t];
+      unpack_xyzr(tv, xyz, r_unused);
       idx = node_of(lv, xyz[0], xyz[1], xyz[2]);
       const int own = lv.owner[idx];  // requested beside the claim's exchange
       const int c = atomicExch(&claim[idx], CLAIM_FREE);
@@ -1401,96 +1429,115 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
     if (act) {
       if (need) nw = s_res[threadIdx.x];
       changed = nw != old;
-      if (changed) lv.owner[idx] = nw;
+      if (changed) {
+        lv.owner[idx] = nw;
+        const int k = old == FLUID ? atomicAdd(&s_nc, 1) : PB - 1 - atomicAdd(&s_nu, 1);
+        s_xyz[k] = tv;
+        s_old[k] = old;
+        s_new[k] = nw;
+      }
     }
     // warp-level compaction of the changed nodes into the diagnostic list
     const unsigned bal = __ballot_sync(0xffffffffu, changed);
     int wbase = 0;
     if (lane == 0 && bal) wbase = atomicAdd(chg.count, __popc(bal));
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
-    if (!changed) continue;
-    const int pos = wbase + __popc(bal & ((1u << lane) - 1u));
-    if (pos < chg.cap) {
-      chg.items[3 * pos] = (int32_t)idx;
-      chg.items[3 * pos + 1] = old;
-      chg.items[3 * pos + 2] = nw;
-    }
-    unsigned slot[Q];
-    for (int r = 0; r < Q; ++r) {
-      if (par_next == 0 || r == 0) {
-        slot[r] = (unsigned)r * lv.N + idx;
-      } else {
-        slot[r] = (unsigned)D::opp(r) * lv.N +
-                  node_of(lv, wrapi(xyz[0] - D::cx(r), lv.nx), wrapi(xyz[1] - D::cy(r), lv.ny),
-                          wrapi(xyz[2] - D::cz(r), lv.nz));
+    if (changed) {
+      const int pos = wbase + __popc(bal & ((1u << lane) - 1u));
+      if (pos < chg.cap) {
+        chg.items[3 * pos] = (int32_t)idx;
+        chg.items[3 * pos + 1] = old;
+        chg.items[3 * pos + 2] = nw;
       }
     }
-    double arm_o[3] = {0, 0, 0}, arm_n[3] = {0, 0, 0};
-    float u_o[3] = {0.f, 0.f, 0.f};
-    if (old >= 0) {
-      for (int k = 0; k < 3; ++k) arm_o[k] = min_image_exact((double)xyz[k] - pv.X[3 * old + k], dims[k], lv.per[k]);
-      const double *W = pv.Om + 3 * old;
-      u_o[0] = (float)(pv.V[3 * old + 0] + (W[1] * arm_o[2] - W[2] * arm_o[1]));
-      u_o[1] = (float)(pv.V[3 * old + 1] + (W[2] * arm_o[0] - W[0] * arm_o[2]));
-      u_o[2] = (float)(pv.V[3 * old + 2] + (W[0] * arm_o[1] - W[1] * arm_o[0]));
-    }
-    if (nw >= 0)
-      for (int k = 0; k < 3; ++k) arm_n[k] = min_image_exact((double)xyz[k] - pv.X[3 * nw + k], dims[k], lv.per[k]);
-    if (old == FLUID && nw >= 0) {
-      // covered: the fluid is deleted, its momentum goes to the new owner;
-      // its populations bounced off a cell in this step still owe their C
-      // (the next sweep would have added it): C_r enters direction rbar,
-      // momentum -C_r c_r, with the velocity of this step's half step at
-      // the link's cell at its position of this step
-      const float4 pu = lv.pu[idx];
-      const uint32_t pm = __float_as_uint(pu.w);
-      if (impulses) {
-        float mf[3] = {0.f, 0.f, 0.f};
-        for (int r = 0; r < Q; ++r) {
-          const float v = Store<S>::ld(pop + slot[r]);
-          mf[0] += v * D::cx(r);
-          mf[1] += v * D::cy(r);
-          mf[2] += v * D::cz(r);
+    __syncthreads();
+    // covered nodes first, then from a warp boundary on the uncovered ones
+    const int nc = s_nc, nc32 = (nc + 31) & ~31, ntot = nc32 + s_nu;
+    for (int k = threadIdx.x; k < ntot; k += PB) {
+      if (k >= nc && k < nc32) continue;
+      const bool cover = k < nc;
+      const int e = cover ? k : PB - 1 - (k - nc32);
+      int r_unused;
+      unpack_xyzr(s_xyz[e], xyz, r_unused);
+      idx = node_of(lv, xyz[0], xyz[1], xyz[2]);
+      old = s_old[e];
+      nw = s_new[e];
+      unsigned slot[Q];
+      for (int r = 0; r < Q; ++r) {
+        if (par_next == 0 || r == 0) {
+          slot[r] = (unsigned)r * lv.N + idx;
+        } else {
+          slot[r] = (unsigned)D::opp(r) * lv.N +
+                    node_of(lv, wrapi(xyz[0] - D::cx(r), lv.nx), wrapi(xyz[1] - D::cy(r), lv.ny),
+                            wrapi(xyz[2] - D::cz(r), lv.nz));
         }
-        // C_r owed to direction rbar: momentum -C_r c_r (the links to a second
-        // or third cell got theirs in place)
-        for (uint32_t m = pm; m; m &= m - 1u) {
-          const int r = __ffs(m) - 1;
-          const float cx = (float)rt_c<0>(r), cy = (float)rt_c<1>(r), cz = (float)rt_c<2>(r);
-          const float C = -((float)rt_m(r) / 6.0f) * (cx * pu.x + cy * pu.y + cz * pu.z);
-          mf[0] -= C * cx;
-          mf[1] -= C * cy;
-          mf[2] -= C * cz;
-        }
-        const double mom[3] = {mf[0], mf[1], mf[2]};
-        const double tq[3] = {arm_n[1] * mom[2] - arm_n[2] * mom[1], arm_n[2] * mom[0] - arm_n[0] * mom[2],
-                              arm_n[0] * mom[1] - arm_n[1] * mom[0]};
-        atomic_add3(pv.PF + 3 * nw, mom);
-        atomic_add3(pv.PT + 3 * nw, tq);
       }
-      if (pm) reinterpret_cast<float *>(lv.pu + idx)[3] = 0.f;
-    } else if (old >= 0) {
-      const double mom[3] = {pv.rho0 * u_o[0], pv.rho0 * u_o[1], pv.rho0 * u_o[2]};
-      const double tq[3] = {arm_o[1] * mom[2] - arm_o[2] * mom[1], arm_o[2] * mom[0] - arm_o[0] * mom[2],
-                            arm_o[0] * mom[1] - arm_o[1] * mom[0]};
-      const double mneg[3] = {-mom[0], -mom[1], -mom[2]}, tneg[3] = {-tq[0], -tq[1], -tq[2]};
-      atomic_add3(pv.PF + 3 * old, mneg);
-      atomic_add3(pv.PT + 3 * old, tneg);
-      if (nw == FLUID) {
-        // uncovered: new fluid at n^eq(rho_bar, u_rigid), stored shifted
-        const float rho0 = (float)pv.rho0;
-        const float uu = u_o[0] * u_o[0] + u_o[1] * u_o[1] + u_o[2] * u_o[2];
-        for (int r = 0; r < Q; ++r) {
-          const float cu = D::cx(r) * u_o[0] + D::cy(r) * u_o[1] + D::cz(r) * u_o[2];
-          const float w = D::m(r) / 36.0f;
-          Store<S>::st(pop + slot[r], rho0 * w * (cu * (3.0f + cu * (4.5f + 4.5f * cu)) - uu * (1.5f + 4.5f * cu)));
+      if (cover) {
+        // covered: the fluid is deleted, its momentum goes to the new owner;
+        // its populations bounced off a cell in this step still owe their C
+        // (the next sweep would have added it): C_r enters direction rbar,
+        // momentum -C_r c_r, with the velocity of this step's half step at
+        // the link's cell at its position of this step
+        const float4 pu = lv.pu[idx];
+        const uint32_t pm = __float_as_uint(pu.w);
+        if (impulses) {
+          float mf[3] = {0.f, 0.f, 0.f};
+          for (int r = 0; r < Q; ++r) {
+            const float v = Store<S>::ld(pop + slot[r]);
+            mf[0] += v * D::cx(r);
+            mf[1] += v * D::cy(r);
+            mf[2] += v * D::cz(r);
+          }
+          // C_r owed to direction rbar: momentum -C_r c_r (the links to a second
+          // or third cell got theirs in place)
+          for (uint32_t m = pm; m; m &= m - 1u) {
+            const int r = __ffs(m) - 1;
+            const float cx = (float)rt_c<0>(r), cy = (float)rt_c<1>(r), cz = (float)rt_c<2>(r);
+            const float C = -((float)rt_m(r) / 6.0f) * (cx * pu.x + cy * pu.y + cz * pu.z);
+            mf[0] -= C * cx;
+            mf[1] -= C * cy;
+            mf[2] -= C * cz;
+          }
+          double arm[3];
+          arm64(lv, pv, pv.kin_next, nw, xyz, arm);
+          const double mom[3] = {mf[0], mf[1], mf[2]};
+          const double tq[3] = {arm[1] * mom[2] - arm[2] * mom[1], arm[2] * mom[0] - arm[0] * mom[2],
+                                arm[0] * mom[1] - arm[1] * mom[0]};
+          atomic_add3(pv.PF + 3 * nw, mom);
+          atomic_add3(pv.PT + 3 * nw, tq);
         }
+        if (pm) reinterpret_cast<float *>(lv.pu + idx)[3] = 0.f;
       } else {
-        // direct change of owner: uncover by the old, cover by the new (reading Q6)
-        const double tq2[3] = {arm_n[1] * mom[2] - arm_n[2] * mom[1], arm_n[2] * mom[0] - arm_n[0] * mom[2],
-                               arm_n[0] * mom[1] - arm_n[1] * mom[0]};
-        atomic_add3(pv.PF + 3 * nw, mom);
-        atomic_add3(pv.PT + 3 * nw, tq2);
+        double arm[3];
+        arm64(lv, pv, pv.kin_next, old, xyz, arm);
+        const double *W = pv.Om + 3 * old, *V = pv.V + 3 * old;
+        const float u[3] = {(float)(V[0] + (W[1] * arm[2] - W[2] * arm[1])),
+                            (float)(V[1] + (W[2] * arm[0] - W[0] * arm[2])),
+                            (float)(V[2] + (W[0] * arm[1] - W[1] * arm[0]))};
+        const double mom[3] = {pv.rho0 * u[0], pv.rho0 * u[1], pv.rho0 * u[2]};
+        const double mneg[3] = {-mom[0], -mom[1], -mom[2]};
+        const double tneg[3] = {arm[2] * mom[1] - arm[1] * mom[2], arm[0] * mom[2] - arm[2] * mom[0],
+                                arm[1] * mom[0] - arm[0] * mom[1]};
+        atomic_add3(pv.PF + 3 * old, mneg);
+        atomic_add3(pv.PT + 3 * old, tneg);
+        if (nw == FLUID) {
+          // uncovered: new fluid at n^eq(rho_bar, u_rigid), stored shifted
+          const float rho0 = lv.rho0;
+          const float uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+          for (int r = 0; r < Q; ++r) {
+            const float cu = D::cx(r) * u[0] + D::cy(r) * u[1] + D::cz(r) * u[2];
+            const float w = D::m(r) / 36.0f;
+            Store<S>::st(pop + slot[r], rho0 * w * (cu * (3.0f + cu * (4.5f + 4.5f * cu)) - uu * (1.5f + 4.5f * cu)));
+          }
+        } else {
+          // direct change of owner: uncover by the old, cover by the new (reading Q6)
+          double an[3];
+          arm64(lv, pv, pv.kin_next, nw, xyz, an);
+          const double tq2[3] = {an[1] * mom[2] - an[2] * mom[1], an[2] * mom[0] - an[0] * mom[2],
+                                 an[0] * mom[1] - an[1] * mom[0]};
+          atomic_add3(pv.PF + 3 * nw, mom);
+          atomic_add3(pv.PT + 3 * nw, tq2);
+        }
       }
     }
   }
@@ -1596,12 +1643,10 @@ __global__ void __launch_bounds__(LB) k_contacts(LatticeView lv, PartView pv) {
   const int by = pv.box[6 * p + 4] - lo1 + 1, bz = pv.box[6 * p + 5] - lo2 + 1;
   const int rows = (by > 0 && bz > 0) ? by * bz : 0;
   CellGeo g;
-  cell_geo(pv, p, g);
-  const float ip = (float)pv.inv_rperp2, kk = (float)(pv.inv_rpar2 - pv.inv_rperp2);
+  cell_geo(pv, pv.kin, p, g);
+  const float ip = pv.inv_rperp2_f, kk = pv.kk_f;
   const int imin = lv.per[0] ? -(lv.nx / 2) : -g.Xi[0];
   const int imax = lv.per[0] ? imin + lv.nx - 1 : lv.nx - 1 - g.Xi[0];
-  const float4 k0 = pv.kin[3 * p], k1 = pv.kin[3 * p + 1], k2 = pv.kin[3 * p + 2];
-  const int Xk[3] = {(int)k0.w, (int)k1.w, (int)k2.w};
   const unsigned nx = (unsigned)lv.nx, nxy = (unsigned)lv.nx * (unsigned)lv.ny;
   int ci[6] = {0, 0, 0, 0, 0, 0};
   for (int r0 = 0; r0 < rows; r0 += LB) {
@@ -1643,8 +1688,8 @@ __global__ void __launch_bounds__(LB) k_contacts(LatticeView lv, PartView pv) {
       // the node's contact links, kept in its neighbour word by the geometry passes
       const unsigned cmask = lv.nbm[nn] & NB_SOLID;
       if (cmask) {
-        const int di[3] = {imin_image(x - Xk[0], lv.nx, lv.per[0]), imin_image(yy - Xk[1], lv.ny, lv.per[1]),
-                           imin_image(zz - Xk[2], lv.nz, lv.per[2])};
+        const int di[3] = {imin_image(x - g.Xi[0], lv.nx, lv.per[0]), imin_image(yy - g.Xi[1], lv.ny, lv.per[1]),
+                           imin_image(zz - g.Xi[2], lv.nz, lv.per[2])};
         sfor<1, Q>([&](auto R) {
           constexpr int r = decltype(R)::value;
           constexpr int m = D::m(r);
