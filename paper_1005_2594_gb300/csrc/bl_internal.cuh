@@ -123,7 +123,8 @@ struct LatticeView {
 // displaced by U t
 struct LeView {
   double U;
-  double *D;     // offset of the pass in flight: written by the gather, read by the scatter
+  float4 *D;     // offset of the pass in flight, written by the gather, read by the scatter: floor(D), D - floor(D)
+                 // and the same of -D (whole parts as the bits of .x, .z)
   long long *t;  // steps since the shear was set
   double *P;     // z-momentum moved along +x across the plane, summed over the steps
   long long *n;  // steps summed
@@ -183,7 +184,8 @@ struct PartView {
   int *rec_last;     // n: records of the last sweep (for the link read-out)
   int *cK, *cIT;     // n x 3 each: contact links, sum m_r c_r and sum m_r dI x c_r
   unsigned long long *touched;  // n x touched_cap nodes claimed or left in one re-discretisation (pack_xyzr)
-  double *lsum;      // n x 27 link sums of one step: F, T (variable part), Zff 6, Zft 9, Ztt 6
+  double *lsum;      // n x 6 link sums of one step: F, T (variable part)
+  float *lsum_f;     // n x 21: Zff 6, Zft 9, Ztt 6
   int *lsum_i;       // n x 6 integer link sums: K, IT
   float *vw;         // n x 6 velocities of the half step the bounced populations are given
   int *touched_count;
@@ -199,6 +201,7 @@ struct PartView {
   int bfc, move;
   double le_dr;  // Lees-Edwards: reflect a cell within le_dr of the sheared plane (0: no shear)
   double inv_rpar2, inv_rperp2, R_par, R_perp;
+  float Rpar2_f, Rperp2_f, Rmax_f;  // R^2 and the larger half-axis in FP32
   float inv_rpar2_f, inv_rperp2_f, kk_f;  // 1 / R^2 in FP32, kk = 1 / R_par^2 - 1 / R_perp^2
   float sig_par, sig_perp, eps, eps_w, mu, nu, chi_prime, r_cut;
   float chi, sigbar, sigbar_w, chi_w, sigw_max;
@@ -275,8 +278,10 @@ void launch_contacts(const LatticeView &lv, const PartView &pv, cudaStream_t st,
 // the pending C of the last step into the stored populations (layout par),
 // before read-outs and state changes between steps
 void launch_flush_pending(int dtype, const LatticeView &lv, int par, cudaStream_t st, int64_t *nl);
+// replaced: the cells were set anew (bl_particles_set), not moved by a step
 void launch_resolve_fill(int dtype, const LatticeView &lv, const PartView &pv, const CellListView &cl, int *claim,
-                         const ChangeList &chg, int par_next, int impulses, cudaStream_t st, int64_t *nl);
+                         const ChangeList &chg, int par_next, int impulses, int replaced, cudaStream_t st,
+                         int64_t *nl);
 void launch_clear_cells(int dtype, const LatticeView &lv, int par, cudaStream_t st, int64_t *nl);
 
 void launch_pair_features(const LatticeView &lv, const PartView &pv, const int2 *pairs, int n, float *out,

@@ -348,7 +348,7 @@ extern "C" int bl_walls_set(bl_ctx *c, const uint8_t *mask) {
 static void free_particles(bl_ctx *c) {
   PartView &pv = c->pv;
   void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.axis, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
-                  pv.touched, pv.touched_count, pv.lsum, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink, pv.Ftot,
+                  pv.touched, pv.touched_count, pv.lsum, pv.lsum_f, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink, pv.Ftot,
                   pv.Ttot, pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
                   c->chg.count, c->chg.items, c->lv.rec, c->lv.rec_count};
   for (void *p : ptrs)
@@ -390,8 +390,10 @@ static int alloc_particles(bl_ctx *c, int n) {
   CU(cudaMalloc(&pv.box, sizeof(int) * 6 * (size_t)n));
   CU(cudaMemsetAsync(pv.box, 0, sizeof(int) * 6 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.stage, sizeof(double) * 13 * (size_t)n));
-  CU(cudaMalloc(&pv.lsum, sizeof(double) * 27 * (size_t)n));
-  CU(cudaMemsetAsync(pv.lsum, 0, sizeof(double) * 27 * (size_t)n, c->stream));
+  CU(cudaMalloc(&pv.lsum, sizeof(double) * 6 * (size_t)n));
+  CU(cudaMemsetAsync(pv.lsum, 0, sizeof(double) * 6 * (size_t)n, c->stream));
+  CU(cudaMalloc(&pv.lsum_f, sizeof(float) * 21 * (size_t)n));
+  CU(cudaMemsetAsync(pv.lsum_f, 0, sizeof(float) * 21 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.lsum_i, sizeof(int) * 6 * (size_t)n));
   CU(cudaMemsetAsync(pv.lsum_i, 0, sizeof(int) * 6 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.vw, sizeof(float) * 6 * (size_t)n));
@@ -480,6 +482,9 @@ static void fill_particle_constants(bl_ctx *c) {
                                              : fmax(pp.sig_perp, fmax(pp.R_perp, pp.R_par) + 1.0));
   pv.inv_rpar2 = 1.0 / (pp.R_par * pp.R_par);
   pv.inv_rperp2 = 1.0 / (pp.R_perp * pp.R_perp);
+  pv.Rmax_f = (float)fmax(pp.R_par, pp.R_perp);
+  pv.Rpar2_f = (float)(pp.R_par * pp.R_par);
+  pv.Rperp2_f = (float)(pp.R_perp * pp.R_perp);
   pv.inv_rpar2_f = (float)pv.inv_rpar2;
   pv.inv_rperp2_f = (float)pv.inv_rperp2;
   pv.kk_f = (float)(pv.inv_rpar2 - pv.inv_rperp2);
@@ -576,7 +581,7 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
   // of the new positions
   if (!first) launch_cell_list(c->lv, c->pv, c->cl, c->stream, &c->launches);
   launch_claims(c->lv, c->pv, c->claim, c->chg, first ? 1 : 2, c->stream, &c->launches);
-  launch_resolve_fill(c->dtype, c->lv, c->pv, c->cl, c->claim, c->chg, c->parity, first ? 0 : 1, c->stream,
+  launch_resolve_fill(c->dtype, c->lv, c->pv, c->cl, c->claim, c->chg, c->parity, first ? 0 : 1, 1, c->stream,
                       &c->launches);
   // neighbour words: the whole lattice after a first placement; after a
   // re-placement only around the nodes resolve changed (every step starts by
@@ -654,7 +659,7 @@ static int enqueue_step(bl_ctx *c, cudaStream_t st) {
     group_end(c, slot, st);
     cudaStreamWaitEvent(st, c->ev_join2, 0);
     group_begin(c, 4, &slot, st);
-    launch_resolve_fill(c->dtype, c->lv, c->pv, c->cl, c->claim, c->chg, c->parity ^ 1, 1, st, &c->launches);
+    launch_resolve_fill(c->dtype, c->lv, c->pv, c->cl, c->claim, c->chg, c->parity ^ 1, 1, 0, st, &c->launches);
     launch_nbm_update(c->lv, c->pv, c->chg, st, &c->launches);
     group_end(c, slot, st);
     std::swap(c->pv.kin, c->pv.kin_next);
@@ -778,7 +783,7 @@ extern "C" int bl_lees_edwards_set(bl_ctx *c, double U, double d_reflect) {
   if (!c->le_on) {
     if (cudaMalloc(&c->lv.le_mom, sizeof(float4) * 2 * M) != cudaSuccess ||
         cudaMalloc(&c->le.T, sizeof(float) * 10 * M) != cudaSuccess ||
-        cudaMalloc(&c->le.D, sizeof(double)) != cudaSuccess || cudaMalloc(&c->le.t, sizeof(long long)) != cudaSuccess ||
+        cudaMalloc(&c->le.D, sizeof(float4)) != cudaSuccess || cudaMalloc(&c->le.t, sizeof(long long)) != cudaSuccess ||
         cudaMalloc(&c->le.P, sizeof(double)) != cudaSuccess || cudaMalloc(&c->le.n, sizeof(long long)) != cudaSuccess)
       return fail(c, BL_ENOMEM, "Lees-Edwards buffers");
   }

@@ -504,7 +504,9 @@ __global__ void __launch_bounds__(128) k_le_gather(LatticeView lv, LeView le) {
   const float ws = warp_sum(Pc);
   if ((threadIdx.x & 31) == 0 && ws != 0.f) atomicAdd(le.P, (double)ws);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *le.D = fmod(le.U * (double)*le.t, (double)lv.nz);
+    const double D = fmod(le.U * (double)*le.t, (double)lv.nz);
+    const double a = floor(D), b = floor(-D);
+    *le.D = make_float4(__int_as_float((int)a), (float)(D - a), __int_as_float((int)b), (float)(-D - b));
     *le.t += 1;
     *le.n += 1;
   }
@@ -523,15 +525,15 @@ __global__ void __launch_bounds__(128) k_le_scatter(LatticeView lv, LeView le) {
   const int yz = i - pl * M, y = yz % ny, z = yz / ny;
   const int x = pl ? lv.nx - 1 : 0;
   const unsigned n = (unsigned)x + (unsigned)lv.nx * (unsigned)yz;
-  const double Dz = pl ? -*le.D : *le.D;
+  // the offset splits into whole nodes and a fraction, the same for every node
+  const float4 Dz = *le.D;
+  const int iD = __float_as_int(pl ? Dz.z : Dz.x);
+  const float w = pl ? Dz.w : Dz.y;
   const float *T = le.T + (size_t)(pl ? 0 : 5) * M;  // sources: x = 0 for pl 1, x = nx - 1 for pl 0
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const int r = pl ? kLeDn[k] : kLeUp[k];
-    const double zs = (double)(z - D::cz(r)) + Dz;
-    const double z0 = floor(zs);
-    const float w = (float)(zs - z0);
-    int za = (int)z0 % nz;
+    int za = (z - D::cz(r) + iD) % nz;
     za = za < 0 ? za + nz : za;
     const int zb = za + 1 == nz ? 0 : za + 1;
     int ys = y - D::cy(r);

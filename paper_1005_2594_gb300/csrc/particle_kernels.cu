@@ -549,33 +549,6 @@ __device__ void inertia_f(const PartView &pv, const double q[4], float I[3][3], 
     }
 }
 
-// A x = b, A symmetric positive definite 6 x 6 (Cholesky, FP32)
-__device__ void solve_spd6f(float A[6][6], const float b[6], float x[6]) {
-  for (int j = 0; j < 6; ++j) {
-    float d = A[j][j];
-    for (int k = 0; k < j; ++k) d -= A[j][k] * A[j][k];
-    d = sqrtf(d);
-    A[j][j] = d;
-    const float id = 1.0f / d;
-    for (int i = j + 1; i < 6; ++i) {
-      float v = A[i][j];
-      for (int k = 0; k < j; ++k) v -= A[i][k] * A[j][k];
-      A[i][j] = v * id;
-    }
-  }
-  float y[6];
-  for (int i = 0; i < 6; ++i) {
-    float v = b[i];
-    for (int k = 0; k < i; ++k) v -= A[i][k] * y[k];
-    y[i] = v / A[i][i];
-  }
-  for (int i = 5; i >= 0; --i) {
-    float v = y[i];
-    for (int k = i + 1; k < 6; ++k) v -= A[k][i] * x[k];
-    x[i] = v / A[i][i];
-  }
-}
-
 __device__ void write_kin(const PartView &pv, int p, const double X[3], const double V[3], const double Om[3]) {
   double Xi[3], f[3];
   for (int k = 0; k < 3; ++k) {
@@ -587,40 +560,17 @@ __device__ void write_kin(const PartView &pv, int p, const double X[3], const do
   pv.kin_next[3 * p + 2] = make_float4((float)Om[0], (float)Om[1], (float)Om[2], (float)Xi[2]);
 }
 
-// X += V (wrapped), q <- exp(W / 2) (x) q with the rotation increment in FP32
-// and a first-order renormalisation (|q|^2 - 1 is O(1e-7))
-__device__ void rigid_advance(const LatticeView &lv, double X[3], double q[4], const double V[3], const double W[3]) {
-  const int dims[3] = {lv.nx, lv.ny, lv.nz};
-  for (int k = 0; k < 3; ++k) {
-    X[k] += V[k];
-    if (lv.per[k]) {
-      if (X[k] < 0.0) X[k] += (double)dims[k];
-      else if (X[k] >= (double)dims[k]) X[k] -= (double)dims[k];
-    }
-  }
-  const float wx = (float)W[0], wy = (float)W[1], wz = (float)W[2];
-  const float th = sqrtf(wx * wx + wy * wy + wz * wz);
-  if (!(th > 0.f)) return;
-  float sn, cs;
-  sincosf(0.5f * th, &sn, &cs);
-  const float sh = sn / th;
-  const double dq[4] = {cs, wx * sh, wy * sh, wz * sh};
-  double nq[4];
-  nq[0] = dq[0] * q[0] - dq[1] * q[1] - dq[2] * q[2] - dq[3] * q[3];
-  nq[1] = dq[0] * q[1] + dq[1] * q[0] + dq[2] * q[3] - dq[3] * q[2];
-  nq[2] = dq[0] * q[2] - dq[1] * q[3] + dq[2] * q[0] + dq[3] * q[1];
-  nq[3] = dq[0] * q[3] + dq[1] * q[2] - dq[2] * q[1] + dq[3] * q[0];
-  const double nn = nq[0] * nq[0] + nq[1] * nq[1] + nq[2] * nq[2] + nq[3] * nq[3];
-  const double c = 1.5 - 0.5 * nn;  // 1 / sqrt(nn) to second order in (nn - 1)
-  for (int k = 0; k < 4; ++k) q[k] = nq[k] * c;
+// node range of an ellipsoid along one axis (centre x, axis component o)
+__device__ __forceinline__ void aabb1(const PartView &pv, float x, float o, int &lo, int &hi) {
+  const float h = sqrtf(pv.Rperp2_f * (1.0f - o * o) + pv.Rpar2_f * o * o) + 0.01f;
+  lo = (int)floorf(x - h);
+  hi = (int)ceilf(x + h);
 }
 
 __device__ void aabb(const PartView &pv, const double X[3], const double o[3], int lo[3], int hi[3]) {
   for (int k = 0; k < 3; ++k) {
     const float ok = (float)o[k];
-    const float h = sqrtf((float)(pv.R_perp * pv.R_perp) * (1.0f - ok * ok) + (float)(pv.R_par * pv.R_par) * ok * ok) + 0.01f;
-    lo[k] = (int)floorf((float)X[k] - h);
-    hi[k] = (int)ceilf((float)X[k] + h);
+    aabb1(pv, (float)X[k], ok, lo[k], hi[k]);
   }
 }
 
@@ -703,12 +653,6 @@ constexpr int LT = 128;  // threads of a link-reduction block
 #ifndef BL_CLAIMS_MINB
 #define BL_CLAIMS_MINB 7
 #endif
-// threads of a block of the cell solve (one thread per cell): few, so that
-// the FP64 work of the cells spreads over many SMs
-#ifndef BL_SOLVE_TB
-#define BL_SOLVE_TB 32
-#endif
-
 __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView lv, PartView pv) {
   __shared__ float shf[LT / 32][27];
   __shared__ int shi[LT / 32][6];
@@ -826,7 +770,8 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
   if (threadIdx.x < 27) {
     double t = 0.0;
     for (int w2 = 0; w2 < LT / 32; ++w2) t += (double)shf[w2][threadIdx.x];
-    pv.lsum[27 * p + threadIdx.x] = t;
+    if (threadIdx.x < 6) pv.lsum[6 * p + threadIdx.x] = t;
+    else pv.lsum_f[21 * p + threadIdx.x - 6] = (float)t;
   } else if (threadIdx.x >= 32 && threadIdx.x < 38) {
     int t = 0;
     for (int w2 = 0; w2 < LT / 32; ++w2) t += shi[w2][threadIdx.x - 32];
@@ -838,154 +783,246 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
   }
 }
 
-// one thread per cell: link force at the predictor, 6 x 6 solve, leap-frog,
-// kinematics and claim box of the next step
-__global__ void k_solve(LatticeView lv, PartView pv) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= pv.n) return;
-  const float4 k1 = pv.kin[3 * p + 1], k2 = pv.kin[3 * p + 2];
-  double X[3], q[4], V[3], L[3], W[3], Xold[3], o_old[3];
-  for (int k = 0; k < 3; ++k) {
-    X[k] = pv.X[3 * p + k];
-    V[k] = pv.V[3 * p + k];
-    L[k] = pv.L[3 * p + k];
-    W[k] = pv.Om[3 * p + k];
-    Xold[k] = X[k];
-    o_old[k] = pv.o[3 * p + k];
-  }
-  for (int k = 0; k < 4; ++k) q[k] = pv.q[4 * p + k];
-  for (int k = 0; k < 3; ++k) pv.oprev[3 * p + k] = (float)o_old[k];  // the claims' old ellipsoid
-  double vd[6];
-  float v[27];
-  for (int k = 0; k < 27; ++k) {
-    v[k] = (float)pv.lsum[27 * p + k];
-    if (k < 6) vd[k] = pv.lsum[27 * p + k];
-  }
-  double K[3], IT[3];
-  for (int k = 0; k < 3; ++k) {
-    // (the link reduction and the contact kernel rewrite these every step)
-    K[k] = (double)(pv.lsum_i[6 * p + k] + pv.cK[3 * p + k]);
-    IT[k] = (double)(pv.lsum_i[6 * p + 3 + k] + pv.cIT[3 * p + k]);
-  }
+// Link force at the predictor, 6 x 6 solve, leap-frog, kinematics and claim
+// box of the next step.  Four lanes per cell, lane k holding component k of
+// its vectors (lane 3 component 0 again) and of its quaternion: every FP64
+// instruction holds the SM's FP64 pipe for 16 cycles, so a warp of 32 cells
+// with three components in a row took 14.4 us at any number of cells.  The
+// 6 x 6 system (FP32) is solved by all four lanes alike.
+constexpr int SOLVE_CELLS = 8;  // per block of one warp
+
+__device__ __forceinline__ float pick3f(int k, float a, float b, float c) { return k == 0 ? a : (k == 1 ? b : c); }
+
+__global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x, k4 = lane & 3, k = k4 < 3 ? k4 : 0, g0 = lane & ~3;
+  const int pr = blockIdx.x * SOLVE_CELLS + (lane >> 2);
+  const bool valid = pr < pv.n, wr = valid && k4 < 3;
+  const int p = valid ? pr : pv.n - 1, c = 3 * p + k;
+  // component j of the cell's vector
+  auto at = [&](auto v, int j) { return __shfl_sync(FULL, v, g0 + j); };
+  double X = pv.X[c], V = pv.V[c], L = pv.L[c], W = pv.Om[c], q = pv.q[4 * p + k4];
+  const double Xold = X, o_old = pv.o[c];
+  const float *kf = reinterpret_cast<const float *>(pv.kin + 3 * p);
+  const float Vpf = kf[4 + k], Wpf = kf[8 + k];
+  float Zs[21];
+#pragma unroll
+  for (int i = 0; i < 21; ++i) Zs[i] = pv.lsum_f[21 * p + i];
+  // (the link reduction and the contact kernel rewrite these every step)
+  const double K = (double)(pv.lsum_i[6 * p + k] + pv.cK[c]), IT = (double)(pv.lsum_i[6 * p + 3 + k] + pv.cIT[c]);
   // link force at the predictor: variable part + exact constant part, with
   // f = X - rint(X) the fraction the sweep's lever arms used
   const double cst = pv.rho0 / 18.0;
-  double f[3];
-  for (int k = 0; k < 3; ++k) f[k] = X[k] - rint(X[k]);
-  const double fxK[3] = {f[1] * K[2] - f[2] * K[1], f[2] * K[0] - f[0] * K[2], f[0] * K[1] - f[1] * K[0]};
-  double Fl[3], Tl[3], Ft[3], Tt[3];
-  for (int k = 0; k < 3; ++k) {
-    Fl[k] = vd[k] + cst * K[k];
-    Tl[k] = vd[3 + k] + cst * (IT[k] - fxK[k]);
-    Ft[k] = Fl[k] + pv.Fpot[3 * p + k] + pv.PF[3 * p + k] + (pv.bfc ? pv.m * pv.g[k] : 0.0);
-    Tt[k] = Tl[k] + pv.Tpot[3 * p + k] + pv.PT[3 * p + k];
-    pv.PF[3 * p + k] = 0.0;
-    pv.PT[3 * p + k] = 0.0;
+  const double f = X - rint(X);
+  const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+  const double fxK = at(f, k1) * at(K, k2) - at(f, k2) * at(K, k1);
+  double Fl = pv.lsum[6 * p + k] + cst * K, Tl = pv.lsum[6 * p + 3 + k] + cst * (IT - fxK);
+  double Ft = Fl + pv.Fpot[c] + pv.PF[c] + (pv.bfc ? pv.m * pv.g[k] : 0.0);
+  double Tt = Tl + pv.Tpot[c] + pv.PT[c];
+  const float oldf = (float)o_old;
+  if (wr) {
+    pv.PF[c] = 0.0;
+    pv.PT[c] = 0.0;
+    pv.oprev[c] = oldf;  // the claims' old ellipsoid
   }
-  const double Vp[3] = {k1.x, k1.y, k1.z}, Wp[3] = {k2.x, k2.y, k2.z};
   const bool move = pv.move != 0;
   if (pv.move == 1) {  // free cells; 2: prescribed, V and W stay as set
-    float Z[6][6];
+    float I[3][3];
     {
-      int k = 6;
-      for (int s = 0; s < 3; ++s)
-        for (int t = s; t < 3; ++t, ++k) Z[s][t] = Z[t][s] = v[k];
-      for (int s = 0; s < 3; ++s)
-        for (int t = 0; t < 3; ++t, ++k) Z[s][3 + t] = Z[3 + t][s] = v[k];
-      for (int s = 0; s < 3; ++s)
-        for (int t = s; t < 3; ++t, ++k) Z[3 + s][3 + t] = Z[3 + t][3 + s] = v[k];
+      const float qf = (float)q;
+      const float w = at(qf, 0), x = at(qf, 1), y = at(qf, 2), z = at(qf, 3);
+      const float R[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
+                             {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
+                             {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
+      const float d0 = (float)pv.Iperp, d2 = (float)pv.Ipar;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          I[a][b] = R[a][0] * d0 * R[b][0] + R[a][1] * d0 * R[b][1] + R[a][2] * d2 * R[b][2];
     }
-    float I[3][3], Iinv[3][3], A[6][6], rhs[6], d[6];
-    inertia_f(pv, q, I, Iinv);
-    for (int s = 0; s < 6; ++s)
-      for (int t = 0; t < 6; ++t) A[s][t] = Z[s][t];
-    for (int s = 0; s < 3; ++s) {
-      A[s][s] += (float)pv.m;
-      for (int t = 0; t < 3; ++t) A[3 + s][3 + t] += I[s][t];
+    float Z[6][6], A[6][6], rhs[6], d[6], inv[6];
+    {
+      int i = 0;
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int t = s; t < 3; ++t, ++i) Z[s][t] = Z[t][s] = Zs[i];
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int t = 0; t < 3; ++t, ++i) Z[s][3 + t] = Z[3 + t][s] = Zs[i];
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+#pragma unroll
+        for (int t = s; t < 3; ++t, ++i) Z[3 + s][3 + t] = Z[3 + t][3 + s] = Zs[i];
+    }
+    {
       // L(t-1/2) - I Wp: a small difference of O(I W) numbers, in FP64
-      const double IW = (double)I[s][0] * Wp[0] + (double)I[s][1] * Wp[1] + (double)I[s][2] * Wp[2];
-      rhs[s] = (float)(Ft[s] - pv.m * (Vp[s] - V[s]));
-      rhs[3 + s] = (float)(Tt[s] + (L[s] - IW));
-    }
-    solve_spd6f(A, rhs, d);
-    for (int s = 0; s < 3; ++s) {
-      float dF = 0.f, dT = 0.f;
-      for (int t = 0; t < 6; ++t) {
-        dF += Z[s][t] * d[t];
-        dT += Z[3 + s][t] * d[t];
+      double IW = 0.0;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) IW += (double)pick3f(k, I[0][t], I[1][t], I[2][t]) * (double)at(Wpf, t);
+      const float r0 = (float)(Ft - pv.m * ((double)Vpf - V)), r1 = (float)(Tt + (L - IW));
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        rhs[s] = at(r0, s);
+        rhs[3 + s] = at(r1, s);
       }
-      Fl[s] -= dF;
-      Tl[s] -= dT;
-      Ft[s] -= dF;
-      Tt[s] -= dT;
     }
+    // Cholesky with the reciprocals of the diagonal (a Newton step on rsqrt)
+    const float m = (float)pv.m;
+#pragma unroll
+    for (int s = 0; s < 6; ++s)
+#pragma unroll
+      for (int t = 0; t <= s; ++t) {
+        A[s][t] = Z[s][t];
+        if (s < 3 && s == t) A[s][t] += m;
+        if (s >= 3 && t >= 3) A[s][t] += I[s >= 3 ? s - 3 : 0][t >= 3 ? t - 3 : 0];
+      }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      float dj = A[j][j];
+#pragma unroll
+      for (int t = 0; t < j; ++t) dj -= A[j][t] * A[j][t];
+      const float y = rsqrtf(dj);
+      inv[j] = fmaf(0.5f * y, fmaf(-dj * y, y, 1.0f), y);
+#pragma unroll
+      for (int i = j + 1; i < 6; ++i) {
+        float v = A[i][j];
+#pragma unroll
+        for (int t = 0; t < j; ++t) v -= A[i][t] * A[j][t];
+        A[i][j] = v * inv[j];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      float v = rhs[i];
+#pragma unroll
+      for (int t = 0; t < i; ++t) v -= A[i][t] * d[t];
+      d[i] = v * inv[i];
+    }
+#pragma unroll
+    for (int i = 5; i >= 0; --i) {
+      float v = d[i];
+#pragma unroll
+      for (int t = i + 1; t < 6; ++t) v -= A[t][i] * d[t];
+      d[i] = v * inv[i];
+    }
+    float dF[3], dT[3];
+#pragma unroll
     for (int s = 0; s < 3; ++s) {
-      V[s] = Vp[s] + (double)d[s];
-      W[s] = Wp[s] + (double)d[3 + s];
-      L[s] += Tt[s];
+      dF[s] = dT[s] = 0.f;
+#pragma unroll
+      for (int t = 0; t < 6; ++t) {
+        dF[s] += Z[s][t] * d[t];
+        dT[s] += Z[3 + s][t] * d[t];
+      }
     }
+    const double dFk = pick3f(k, dF[0], dF[1], dF[2]), dTk = pick3f(k, dT[0], dT[1], dT[2]);
+    Fl -= dFk;
+    Tl -= dTk;
+    Ft -= dFk;
+    Tt -= dTk;
+    V = (double)Vpf + (double)pick3f(k, d[0], d[1], d[2]);
+    W = (double)Wpf + (double)pick3f(k, d[3], d[4], d[5]);
+    L += Tt;
   }
-  for (int s = 0; s < 3; ++s) {
-    pv.Flink[3 * p + s] = Fl[s];
-    pv.Tlink[3 * p + s] = Tl[s];
-    pv.Ftot[3 * p + s] = Ft[s];
-    pv.Ttot[3 * p + s] = Tt[s];
-    pv.vw[6 * p + s] = (float)V[s];
-    pv.vw[6 * p + 3 + s] = (float)W[s];
+  const float Wf = (float)W;
+  float Vf = (float)V;
+  if (wr) {
+    pv.Flink[c] = Fl;
+    pv.Tlink[c] = Tl;
+    pv.Ftot[c] = Ft;
+    pv.Ttot[c] = Tt;
+    pv.vw[6 * p + k] = Vf;
+    pv.vw[6 * p + 3 + k] = Wf;
   }
-  int lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
   if (move) {
+    const int dim = k == 0 ? lv.nx : (k == 1 ? lv.ny : lv.nz);
     // Sec. IV: a free cell closer than le_dr to the sheared plane (x = -1/2)
     // and moving toward it has its normal velocity negated; the step's
     // coupling above used the solve's velocity, the cell moves with the
     // reflected one (reading Q25)
-    if (pv.le_dr > 0.0 && pv.move == 1) {
-      const double dlo = X[0] + 0.5, dhi = (double)lv.nx - 0.5 - X[0];
-      if ((dlo < pv.le_dr && V[0] < 0.0) || (dhi < pv.le_dr && V[0] > 0.0)) V[0] = -V[0];
+    if (pv.le_dr > 0.0 && pv.move == 1 && k == 0) {
+      const double dlo = X + 0.5, dhi = (double)lv.nx - 0.5 - X;
+      if ((dlo < pv.le_dr && V < 0.0) || (dhi < pv.le_dr && V > 0.0)) {
+        V = -V;
+        Vf = -Vf;
+      }
     }
-    rigid_advance(lv, X, q, V, W);
-    for (int k = 0; k < 3; ++k) {
-      pv.X[3 * p + k] = X[k];
-      pv.V[3 * p + k] = V[k];
-      pv.L[3 * p + k] = L[k];
-      pv.Om[3 * p + k] = W[k];
+    // X += V (wrapped), q <- exp(W / 2) (x) q with the rotation increment in
+    // FP32 and a first-order renormalisation (|q|^2 - 1 is O(1e-7))
+    X += V;
+    if (lv.per[k]) {
+      if (X < 0.0) X += (double)dim;
+      else if (X >= (double)dim) X -= (double)dim;
     }
-    for (int k = 0; k < 4; ++k) pv.q[4 * p + k] = q[k];
-    double o_new[3];
-    axis_exact(q, o_new);
-    for (int k = 0; k < 3; ++k) pv.o[3 * p + k] = o_new[k];
-    pv.axis[p] = make_float4((float)o_new[0], (float)o_new[1], (float)o_new[2], 0.f);
-    bool finite = true;
-    for (int k = 0; k < 3; ++k) finite = finite && isfinite(X[k]) && isfinite(o_new[k]);
+    const float wx = at(Wf, 0), wy = at(Wf, 1), wz = at(Wf, 2);
+    const float th = sqrtf(wx * wx + wy * wy + wz * wz);
+    float sn, cs;
+    sincosf(0.5f * th, &sn, &cs);
+    const float sh = sn / th;
+    // component l = k4 of the product: sum over m of +- dq[m] q[l xor m]
+    const float dx = (k4 & 1) ? wx * sh : -(wx * sh);
+    const float dy = (k4 == 1 || k4 == 2) ? wy * sh : -(wy * sh);
+    const float dz = (k4 & 2) ? wz * sh : -(wz * sh);
+    double nq = (double)cs * q;
+    nq += (double)dx * __shfl_xor_sync(FULL, q, 1);
+    nq += (double)dy * __shfl_xor_sync(FULL, q, 2);
+    nq += (double)dz * __shfl_xor_sync(FULL, q, 3);
+    double nn = nq * nq;
+    nn += __shfl_xor_sync(FULL, nn, 1);
+    nn += __shfl_xor_sync(FULL, nn, 2);
+    if (th > 0.f) q = nq * (1.5 - 0.5 * nn);  // 1 / sqrt(nn) to second order in (nn - 1)
+    // the exact axis (axis_exact), component by component
+    const double a1 = at(q, k == 1 ? 2 : 1), b1 = at(q, k == 2 ? 1 : 3), a2 = at(q, k == 2 ? 2 : 0),
+                 b2 = at(q, k == 1 ? 1 : 2);
+    const double pa = __dmul_rn(a1, b1), pb = __dmul_rn(a2, b2);
+    const double o2 = __dmul_rn(2.0, __dadd_rn(pa, k == 1 ? -pb : pb));
+    const double o = k == 2 ? __dsub_rn(1.0, o2) : o2;
+    const float of = (float)o, Xf = (float)X;
     // a cell faster than half a node per step is far outside the method's
     // low-Mach range (and would outrun the cell list of the step's start)
-    if (!(V[0] * V[0] + V[1] * V[1] + V[2] * V[2] < 0.25)) finite = false;
+    const double vv = V * V, v2 = at(vv, 0) + at(vv, 1) + at(vv, 2);
+    const bool ok = isfinite(X) && isfinite(o) && v2 < 0.25;
+    const bool finite = ((__ballot_sync(FULL, ok) >> g0) & 7u) == 7u;
+    int lo = 0, hi = -1;
     if (finite) {
-      int lo2[3], hi2[3];
-      aabb(pv, X, o_new, lo, hi);
-      aabb(pv, Xold, o_old, lo2, hi2);
-      const int dims[3] = {lv.nx, lv.ny, lv.nz};
-      for (int k = 0; k < 3; ++k) {
-        lo[k] = min(lo[k], lo2[k]);
-        hi[k] = max(hi[k], hi2[k]);
-        if (!lv.per[k]) {
-          lo[k] = max(lo[k], 0);
-          hi[k] = min(hi[k], dims[k] - 1);
-        } else if (hi[k] - lo[k] + 1 > dims[k]) {
-          lo[k] = 0;
-          hi[k] = dims[k] - 1;
-        }
+      int lo2, hi2;
+      aabb1(pv, Xf, of, lo, hi);
+      aabb1(pv, (float)Xold, oldf, lo2, hi2);
+      lo = min(lo, lo2);
+      hi = max(hi, hi2);
+      if (!lv.per[k]) {
+        lo = max(lo, 0);
+        hi = min(hi, dim - 1);
+      } else if (hi - lo + 1 > dim) {
+        lo = 0;
+        hi = dim - 1;
       }
-    } else {
+    } else if (valid) {
       atomicOr(pv.status, ST_UNSTABLE);
     }
-  }
-  if (move)  // fixed cells keep the box of their last set: the geometry pass still needs it
-    for (int k = 0; k < 3; ++k) {
-      pv.box[6 * p + k] = lo[k];
-      pv.box[6 * p + 3 + k] = hi[k];
+    if (valid) pv.q[4 * p + k4] = q;
+    if (wr) {
+      pv.X[c] = X;
+      pv.V[c] = V;
+      pv.L[c] = L;
+      pv.Om[c] = W;
+      pv.o[c] = o;
+      reinterpret_cast<float *>(pv.axis + p)[k] = of;
+      pv.box[6 * p + k] = lo;  // fixed cells keep the box of their last set: the geometry pass still needs it
+      pv.box[6 * p + 3 + k] = hi;
     }
-  write_kin(pv, p, X, V, W);
+  }
+  if (wr) {
+    const double Xi = rint(X);
+    float *kn = reinterpret_cast<float *>(pv.kin_next + 3 * p);
+    kn[k] = (float)(X - Xi);
+    kn[4 + k] = Vf;
+    kn[8 + k] = Wf;
+    kn[4 * k + 3] = (float)Xi;
+  }
 }
 
 // The pending moving-boundary term of each record, right after the solve
@@ -997,7 +1034,7 @@ __global__ void k_solve(LatticeView lv, PartView pv) {
 // velocities of the solve; d: node minus the cell's position of this step.
 // Every link is one cell's, so no two blocks touch the same slot.
 template <class S>
-__global__ void __launch_bounds__(LT) k_link_pending(LatticeView lv, PartView pv, int par) {
+__global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView pv, int par) {
   constexpr int PQ = 512;  // queue of a block's second- and third-cell records
   __shared__ int s_nq;
   __shared__ int s_q[PQ];
@@ -1011,12 +1048,9 @@ __global__ void __launch_bounds__(LT) k_link_pending(LatticeView lv, PartView pv
   const float V[3] = {vw[0], vw[1], vw[2]}, W[3] = {vw[3], vw[4], vw[5]};
   S *pop = reinterpret_cast<S *>(lv.pop);
   const float4 *rec = lv.rec + 2 * (size_t)p * lv.rec_cap;
-  // rho (V + W x d) of record i's node, its coordinates and its mask word
-  auto node_u = [&](int i, unsigned &n, uint32_t &mb, int yc[3], float u[3]) {
-    const float4 r0 = rec[2 * i];
-    n = __float_as_uint(r0.x);
-    mb = __float_as_uint(r0.y);
-    node_xyz(lv, n, yc);
+  // rho (V + W x d) of a record's node and its coordinates
+  auto node_u = [&](const float4 &r0, int yc[3], float u[3]) {
+    node_xyz(lv, __float_as_uint(r0.x), yc);
     const float d[3] = {(float)imin_image(yc[0] - Xi[0], lv.nx, lv.per[0]) - k0.x,
                         (float)imin_image(yc[1] - Xi[1], lv.ny, lv.per[1]) - k0.y,
                         (float)imin_image(yc[2] - Xi[2], lv.nz, lv.per[2]) - k0.z};
@@ -1025,41 +1059,69 @@ __global__ void __launch_bounds__(LT) k_link_pending(LatticeView lv, PartView pv
     u[1] = rho * (V[1] + (W[2] * d[0] - W[0] * d[2]));
     u[2] = rho * (V[2] + (W[0] * d[1] - W[1] * d[0]));
   };
-  // C in place for the directions of a second- or third-cell record
+  // C in place for the directions of a second- or third-cell record: all its
+  // populations requested together, then written
   auto direct = [&](int i) {
-    unsigned n;
-    uint32_t mb;
+    const float4 r0 = rec[2 * i];
+    const unsigned n = __float_as_uint(r0.x);
+    const uint32_t m = __float_as_uint(r0.y) & NB_SOLID;
     int yc[3];
-    float u[3];
-    node_u(i, n, mb, yc, u);
-    for (uint32_t m = mb & NB_SOLID; m; m &= m - 1u) {
-      const int r = __ffs(m) - 1;
-      const float C = -((float)rt_m(r) / 6.0f) * ((float)rt_c<0>(r) * u[0] + (float)rt_c<1>(r) * u[1] +
-                                                  (float)rt_c<2>(r) * u[2]);
-      const unsigned slot = bounce_slot(lv, par, n, yc, r);
-      Store<S>::st(pop + slot, Store<S>::ld(pop + slot) + C);
-    }
+    float u[3], v[Q];
+    node_u(r0, yc, u);
+    unsigned slot[Q];
+    const unsigned nx = (unsigned)lv.nx, nxy = nx * (unsigned)lv.ny;
+    const unsigned xo[3] = {(unsigned)(yc[0] == 0 ? lv.nx - 1 : yc[0] - 1), (unsigned)yc[0],
+                            (unsigned)(yc[0] == lv.nx - 1 ? 0 : yc[0] + 1)};
+    const unsigned yo[3] = {(unsigned)(yc[1] == 0 ? lv.ny - 1 : yc[1] - 1) * nx, (unsigned)yc[1] * nx,
+                            (unsigned)(yc[1] == lv.ny - 1 ? 0 : yc[1] + 1) * nx};
+    const unsigned zo[3] = {(unsigned)(yc[2] == 0 ? lv.nz - 1 : yc[2] - 1) * nxy, (unsigned)yc[2] * nxy,
+                            (unsigned)(yc[2] == lv.nz - 1 ? 0 : yc[2] + 1) * nxy};
+    sfor<1, Q>([&](auto R) {
+      constexpr int r = decltype(R)::value;
+      // the slot the sweep of parity par bounced direction r into
+      slot[r] = par == 0 ? (unsigned)r * lv.N + xo[1 + D3::cx(r)] + yo[1 + D3::cy(r)] + zo[1 + D3::cz(r)]
+                         : (unsigned)D3::opp(r) * lv.N + n;
+      if ((m >> r) & 1u) v[r] = Store<S>::ld(pop + slot[r]);
+    });
+    sfor<1, Q>([&](auto R) {
+      constexpr int r = decltype(R)::value;
+      const float C = -(D3::m(r) / 6.0f) * (D3::cx(r) * u[0] + D3::cy(r) * u[1] + D3::cz(r) * u[2]);
+      if ((m >> r) & 1u) Store<S>::st(pop + slot[r], v[r] + C);
+    });
   };
-  for (int i = threadIdx.x; i < nrec; i += LT) {
-    const uint32_t mb = __float_as_uint(rec[2 * i].y);
-    if (mb & REC_DIRECT) {
-      const int k = atomicAdd(&s_nq, 1);
-      if (k < PQ) s_q[k] = i;
-      else direct(i);
-      continue;
+  // four records per thread requested together: one memory round trip each
+  // took most of the kernel's time
+  constexpr int PU = 4;
+  for (int i0 = threadIdx.x; i0 < nrec; i0 += PU * LT) {
+    float4 r0[PU];
+#pragma unroll
+    for (int j = 0; j < PU; ++j)
+      if (i0 + j * LT < nrec) r0[j] = rec[2 * (i0 + j * LT)];
+#pragma unroll
+    for (int j = 0; j < PU; ++j) {
+      const int i = i0 + j * LT;
+      if (i >= nrec) break;
+      const uint32_t mb = __float_as_uint(r0[j].y);
+      if (mb & REC_DIRECT) {
+        const int k = atomicAdd(&s_nq, 1);
+        if (k < PQ) s_q[k] = i;
+        continue;
+      }
+      int yc[3];
+      float u[3];
+      node_u(r0[j], yc, u);
+      lv.pu[__float_as_uint(r0[j].x)] = make_float4(u[0], u[1], u[2], __uint_as_float(mb & NB_SOLID));
     }
-    unsigned n;
-    uint32_t mb2;
-    int yc[3];
-    float u[3];
-    node_u(i, n, mb2, yc, u);
-    lv.pu[n] = make_float4(u[0], u[1], u[2], __uint_as_float(mb2 & NB_SOLID));
   }
   // the records of a node's second or third cell, gathered so that the
   // warps take their per-direction loops with full lanes
   __syncthreads();
-  const int nq = min(s_nq, PQ);
-  for (int k = threadIdx.x; k < nq; k += LT) direct(s_q[k]);
+  const bool full = s_nq > PQ;  // more than the queue holds: found again among all records
+  const int nq = full ? nrec : s_nq;
+  for (int k = threadIdx.x; k < nq; k += LT) {
+    const int i = full ? k : s_q[k];
+    if (!full || (__float_as_uint(rec[2 * i].y) & REC_DIRECT)) direct(i);
+  }
 }
 
 // The pending C of the last step given to the stored populations, for
@@ -1364,6 +1426,65 @@ __device__ __forceinline__ void atomic_add3(double *a, const double v[3]) {
   atomicAdd(a + 2, v[2]);
 }
 
+// cells that can cover a node cell p leaves: within 2 max(R) + 2 of it after
+// the move (the node is within max(R) + 1 of p's centre, a cell covers it
+// within max(R)).  Gathered once per block into shared memory from the bins
+// within reach (the list is of the step's start; a cell moves less than half a
+// node), so that a node's search reads no memory: a search of its own per
+// node, three dependent loads deep, was the longest chain of the kernel.
+constexpr int NCAND = 64;
+
+struct Cands {
+  int n;
+  int id[NCAND];
+  CellGeo g[NCAND];
+};
+
+__device__ __forceinline__ void gather_cands(const LatticeView &lv, const PartView &pv, const CellListView &cl, int p,
+                                             Cands &cd) {
+  CellGeo g;
+  cell_geo(pv, pv.kin_next, p, g);
+  const float reach = 2.0f * pv.Rmax_f + 2.0f;
+  const int dims[3] = {lv.nx, lv.ny, lv.nz};
+  int b0[3], cnt[3];
+  for (int k = 0; k < 3; ++k) {
+    const float x = (float)g.Xi[k] + g.Xf[k], s = (float)cl.nb[k] / (float)dims[k];
+    int lo = (int)floorf((x - reach - 0.6f) * s - 1e-3f), hi = (int)floorf((x + reach + 0.6f) * s + 1e-3f);
+    if (!lv.per[k]) {
+      lo = max(lo, 0);
+      hi = min(hi, cl.nb[k] - 1);
+    } else if (hi - lo + 1 >= cl.nb[k]) {
+      lo = 0;
+      hi = cl.nb[k] - 1;
+    }
+    b0[k] = lo;
+    cnt[k] = hi - lo + 1;
+  }
+  const int total = cnt[0] * cnt[1] * cnt[2];
+  for (int t = threadIdx.x; t < total; t += PB) {
+    const int bx = wrapi(b0[0] + t % cnt[0], cl.nb[0]), by = wrapi(b0[1] + (t / cnt[0]) % cnt[1], cl.nb[1]),
+              bz = wrapi(b0[2] + t / (cnt[0] * cnt[1]), cl.nb[2]);
+    const int b = bx + cl.nb[0] * (by + cl.nb[1] * bz);
+    const int e = cl.start[b + 1];
+    for (int k = cl.start[b]; k < e; ++k) {
+      const int j = cl.ids[k];
+      CellGeo h;
+      cell_geo(pv, pv.kin_next, j, h);
+      float d2 = 0.f;
+      for (int m = 0; m < 3; ++m) {
+        const float d = (float)imin_image(h.Xi[m] - g.Xi[m], dims[m], lv.per[m]) + (h.Xf[m] - g.Xf[m]);
+        d2 += d * d;
+      }
+      if (d2 > reach * reach) continue;
+      const int i = atomicAdd(&cd.n, 1);
+      if (i < NCAND) {
+        cd.id[i] = j;
+        cd.g[i] = h;
+      }
+    }
+  }
+}
+
 // One block per cell over its touched nodes.  The new owners are decided first
 // and the changed nodes queued, covered ones (fluid to cell) from the front,
 // uncovered ones (a cell leaves) from the back; then each kind is worked off
@@ -1372,7 +1493,7 @@ __device__ __forceinline__ void atomic_add3(double *a, const double v[3]) {
 // branch.
 template <class S>
 __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv, CellListView cl, int *claim,
-                                                      ChangeList chg, int par_next, int impulses) {
+                                                      ChangeList chg, int par_next, int impulses, int replaced) {
   using D = D3Q19;
   const int p = blockIdx.x;
   const unsigned long long *touched = pv.touched + (size_t)p * pv.touched_cap;
@@ -1386,7 +1507,13 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
   __shared__ int s_need[PB], s_res[PB];
   __shared__ unsigned long long s_xyz[PB];
   __shared__ int s_old[PB], s_new[PB];
-  __shared__ int s_ns, s_nc, s_nu;
+  __shared__ int s_ns, s_nc, s_nu, s_base;
+  __shared__ Cands s_cd;
+  if (nt == 0) return;
+  // (a re-placement can put cells anywhere: its nodes are searched one by one)
+  if (threadIdx.x == 0) s_cd.n = replaced ? NCAND + 1 : 0;
+  __syncthreads();
+  if (!replaced) gather_cands(lv, pv, cl, p, s_cd);
   for (int t0 = 0; t0 < nt; t0 += PB) {
     const int t = t0 + threadIdx.x;
     int old = 0, nw = 0, xyz[3] = {0, 0, 0};
@@ -1422,7 +1549,17 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
       const int tt = s_need[k];
       int cc[3], r_unused;
       unpack_xyzr(touched[t0 + tt], cc, r_unused);
-      const int best = lowest_cover(lv, pv, cl, cc[0], cc[1], cc[2]);
+      const int ncd = s_cd.n;
+      int best;
+      if (ncd <= NCAND) {
+        best = INT_MAX;
+        for (int i = lane; i < ncd; i += 32)
+          if (s_cd.id[i] < best && inside_cell(cc[0], cc[1], cc[2], s_cd.id[i], s_cd.g[i], pv, lv)) best = s_cd.id[i];
+        best = __reduce_min_sync(0xffffffffu, best);
+        if (best == INT_MAX) best = FLUID;
+      } else {
+        best = lowest_cover(lv, pv, cl, cc[0], cc[1], cc[2]);
+      }
       if (lane == 0) s_res[tt] = best;
     }
     __syncthreads();
@@ -1437,20 +1574,10 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
         s_new[k] = nw;
       }
     }
-    // warp-level compaction of the changed nodes into the diagnostic list
-    const unsigned bal = __ballot_sync(0xffffffffu, changed);
-    int wbase = 0;
-    if (lane == 0 && bal) wbase = atomicAdd(chg.count, __popc(bal));
-    wbase = __shfl_sync(0xffffffffu, wbase, 0);
-    if (changed) {
-      const int pos = wbase + __popc(bal & ((1u << lane) - 1u));
-      if (pos < chg.cap) {
-        chg.items[3 * pos] = (int32_t)idx;
-        chg.items[3 * pos + 1] = old;
-        chg.items[3 * pos + 2] = nw;
-      }
-    }
     __syncthreads();
+    // room in the change list, asked for before the momentum balance and used
+    // after it
+    if (threadIdx.x == PB - 1) s_base = s_nc + s_nu ? atomicAdd(chg.count, s_nc + s_nu) : 0;
     // covered nodes first, then from a warp boundary on the uncovered ones
     const int nc = s_nc, nc32 = (nc + 31) & ~31, ntot = nc32 + s_nu;
     for (int k = threadIdx.x; k < ntot; k += PB) {
@@ -1540,6 +1667,17 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
         }
       }
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nc + s_nu; k += PB) {
+      const int e = k < nc ? k : PB - 1 - (k - nc), pos = s_base + k;
+      if (pos >= chg.cap) break;
+      int r_unused;
+      unpack_xyzr(s_xyz[e], xyz, r_unused);
+      chg.items[3 * pos] = (int32_t)node_of(lv, xyz[0], xyz[1], xyz[2]);
+      chg.items[3 * pos + 1] = s_old[e];
+      chg.items[3 * pos + 2] = s_new[e];
+    }
+    __syncthreads();  // the queues are refilled by the next chunk
   }
 }
 
@@ -1866,7 +2004,7 @@ void launch_sums_solve(int dtype, const LatticeView &lv, const PartView &pv, int
   (void)par;
   if (pv.n == 0) return;
   k_link_reduce<<<pv.n, LT, 0, st>>>(lv, pv);
-  k_solve<<<nblk(pv.n, BL_SOLVE_TB), BL_SOLVE_TB, 0, st>>>(lv, pv);
+  k_solve<<<nblk(pv.n, SOLVE_CELLS), 32, 0, st>>>(lv, pv);
   *nl += 2;
 }
 
@@ -1932,11 +2070,12 @@ void launch_contacts(const LatticeView &lv, const PartView &pv, cudaStream_t st,
 }
 
 void launch_resolve_fill(int dtype, const LatticeView &lv, const PartView &pv, const CellListView &cl, int *claim,
-                         const ChangeList &chg, int par_next, int impulses, cudaStream_t st, int64_t *nl) {
+                         const ChangeList &chg, int par_next, int impulses, int replaced, cudaStream_t st,
+                         int64_t *nl) {
   if (pv.n == 0) return;
-  if (dtype == 0) k_resolve_fill<float><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses);
-  else if (dtype == 1) k_resolve_fill<__nv_bfloat16><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses);
-  else k_resolve_fill<__half><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses);
+  if (dtype == 0) k_resolve_fill<float><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
+  else if (dtype == 1) k_resolve_fill<__nv_bfloat16><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
+  else k_resolve_fill<__half><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
   *nl += 1;
 }
 
