@@ -109,7 +109,7 @@ struct LatticeView {
   // with the populations and adds as C = -(m_r / 6) c_r . u; the links to a
   // second or third cell of one node get C in place right after the solve.
   float4 *pu;              // N
-  float4 *rec;             // ncells x rec_cap records of 2 float4
+  float4 *rec;             // ncells x 2 x rec_cap: the first, then the second float4 of a cell's records
   int *rec_count;          // ncells
   int rec_cap;
   int *status;

@@ -982,7 +982,7 @@ extern "C" int bl_cell_links_get(bl_ctx *c, int32_t *out, int64_t cap, int64_t *
   std::vector<Link> links;
   for (int p = 0; p < n; ++p) {
     for (int i = 0; i < cnt[p] && i < capr; ++i) {
-      const float4 r0 = rec[2 * ((size_t)p * capr + i)];
+      const float4 r0 = rec[2 * (size_t)p * capr + i];
       uint32_t node, mask;
       memcpy(&node, &r0.x, 4);
       memcpy(&mask, &r0.y, 4);

@@ -143,9 +143,9 @@ __device__ __forceinline__ void write_links(const LatticeView &lv, const CellLin
   const int base = __shfl_sync(sl.grp, sl.base, __ffs(sl.grp) - 1);
   const int pos = base + __popc(sl.grp & ((1u << lane) - 1u));
   if (pos < lv.rec_cap) {
-    float4 *r = lv.rec + 2 * ((size_t)cl.p * lv.rec_cap + pos);
+    float4 *r = lv.rec + (2 * (size_t)cl.p * lv.rec_cap + pos);
     r[0] = make_float4(__uint_as_float(n), __uint_as_float(cl.mask), cl.e[0], cl.e[1]);
-    r[1] = make_float4(cl.e[2], cl.e[3], cl.e[4], cl.e[5]);
+    r[lv.rec_cap] = make_float4(cl.e[2], cl.e[3], cl.e[4], cl.e[5]);
   } else {
     atomicOr(lv.status, ST_OVERFLOW);
   }
@@ -161,13 +161,13 @@ __device__ __forceinline__ void write_second(const LatticeView &lv, const CellLi
   const int base = __shfl_sync(sl.grp, sl.base, __ffs(sl.grp) - 1);
   const int pos = base + __popc(sl.grp & ((1u << lane) - 1u));
   if (pos < lv.rec_cap) {
-    float4 *r = lv.rec + 2 * ((size_t)cl.p2 * lv.rec_cap + pos);
+    float4 *r = lv.rec + (2 * (size_t)cl.p2 * lv.rec_cap + pos);
     if constexpr (TAU1) {
       r[0] = make_float4(__uint_as_float(n), __uint_as_float(cl.mask2 | REC_DIRECT), cl.e[0], cl.e[1]);
-      r[1] = make_float4(cl.e[2], cl.e[3], cl.e[4], cl.e[5]);
+      r[lv.rec_cap] = make_float4(cl.e[2], cl.e[3], cl.e[4], cl.e[5]);
     } else {
       r[0] = make_float4(__uint_as_float(n), __uint_as_float(cl.mask2 | REC_DIRECT), cl.e[0], cl.f2[0]);
-      r[1] = make_float4(cl.f2[1], cl.f2[2], 0.f, 0.f);
+      r[lv.rec_cap] = make_float4(cl.f2[1], cl.f2[2], 0.f, 0.f);
     }
   } else {
     atomicOr(lv.status, ST_OVERFLOW);
@@ -231,9 +231,9 @@ __device__ __forceinline__ void append_link(const LatticeView &lv, unsigned n, i
                                             const float (&e)[6]) {
   const int pos = atomicAdd(&lv.rec_count[q], 1);
   if (pos < lv.rec_cap) {
-    float4 *rr = lv.rec + 2 * ((size_t)q * lv.rec_cap + pos);
+    float4 *rr = lv.rec + (2 * (size_t)q * lv.rec_cap + pos);
     rr[0] = make_float4(__uint_as_float(n), __uint_as_float(mask), e[0], e[1]);
-    rr[1] = make_float4(e[2], e[3], e[4], e[5]);
+    rr[lv.rec_cap] = make_float4(e[2], e[3], e[4], e[5]);
   } else {
     atomicOr(lv.status, ST_OVERFLOW);
   }
@@ -759,9 +759,9 @@ __device__ __forceinline__ void write_staged(const LatticeView &lv, int p, unsig
   const int base = __shfl_sync(grp, base0, __ffs(grp) - 1);
   const int pos = base + __popc(grp & ((1u << lane) - 1u));
   if (pos < lv.rec_cap) {
-    float4 *r = lv.rec + 2 * ((size_t)p * lv.rec_cap + pos);
+    float4 *r = lv.rec + (2 * (size_t)p * lv.rec_cap + pos);
     r[0] = r0;
-    r[1] = r1;
+    r[lv.rec_cap] = r1;
   } else {
     atomicOr(lv.status, ST_OVERFLOW);
   }

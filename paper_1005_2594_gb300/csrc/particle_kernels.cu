@@ -281,6 +281,50 @@ __device__ __forceinline__ int bin_offsets(int nb, int per, int b, int out[3]) {
   return k;
 }
 
+// the cells of the bins around bin bc, numbered through: off[b] is the number
+// of the first cell of neighbouring bin b, start[b] its place in the cell list.
+// A thread per bin that walks its cells alone takes as many dependent reads as
+// the fullest bin holds; numbered through, the cells are read one per thread.
+struct NearBins {
+  int off[28], start[27];
+};
+
+// (one whole warp)
+__device__ __forceinline__ void near_bins(const LatticeView &lv, const CellListView &cl, int bin, NearBins &nbs) {
+  const int lane = threadIdx.x & 31;
+  const int bc[3] = {bin % cl.nb[0], (bin / cl.nb[0]) % cl.nb[1], bin / (cl.nb[0] * cl.nb[1])};
+  int off[3][3], noff[3];
+  for (int k = 0; k < 3; ++k) noff[k] = bin_offsets(cl.nb[k], lv.per[k], bc[k], off[k]);
+  const int ix = lane % 3, iy = (lane / 3) % 3, iz = lane / 9;
+  int s = 0, n = 0;
+  if (lane < 27 && ix < noff[0] && iy < noff[1] && iz < noff[2]) {
+    const int b = wrapi(bc[0] + off[0][ix], cl.nb[0]) +
+                  cl.nb[0] * (wrapi(bc[1] + off[1][iy], cl.nb[1]) + cl.nb[1] * wrapi(bc[2] + off[2][iz], cl.nb[2]));
+    s = cl.start[b];
+    n = cl.start[b + 1] - s;
+  }
+  int inc = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane < 27) {
+    nbs.off[lane] = inc - n;
+    nbs.start[lane] = s;
+    if (lane == 26) nbs.off[27] = inc;
+  }
+}
+
+// cell number t (0 <= t < off[27])
+__device__ __forceinline__ int near_cell(const CellListView &cl, const NearBins &nbs, int t) {
+  int b = 0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    if (b + o < 27 && nbs.off[b + o] <= t) b += o;
+  return cl.ids[nbs.start[b] + t - nbs.off[b]];
+}
+
 // ---------------------------------------------------------------------------
 // block-wide helpers (blockDim.x == 256)
 
@@ -380,9 +424,8 @@ __device__ __forceinline__ unsigned bounce_slot(const LatticeView &lv, int par, 
 }
 
 // ---------------------------------------------------------------------------
-// potentials: one block per cell.  Warp 0 takes the pairs (one lane per
-// neighbouring bin), all threads take the rows (y, z) of the wall-sphere
-// range around the cell.
+// potentials: one block per cell; all threads take the rows (y, z) of the
+// wall-sphere range around the cell, then the cells around it.
 
 constexpr int FB = 128;        // threads of a potentials block
 constexpr int FQ_PAIR = 128;   // per-cell queue of pairs within contact reach
@@ -390,7 +433,7 @@ constexpr int FQ_WALL = 1024;  // per-cell queue of surface wall nodes within re
 
 // One block per cell.  The search runs in FP32 and queues what can be in
 // contact: the cells j of the 27 bins around cell i within the largest
-// contact distance (one thread per bin), and the surface wall nodes within
+// contact distance (one thread per cell), and the surface wall nodes within
 // the wall sphere's radius (rows without a surface wall node skipped by
 // their row bit).  The queued pairs and wall nodes then get the FP64 contact
 // geometry with one queue entry per thread, so that the few contacts of a
@@ -401,6 +444,7 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
   __shared__ int s_np, s_nw;
   __shared__ int s_pair[FQ_PAIR];
   __shared__ unsigned s_wall[FQ_WALL];
+  __shared__ NearBins s_nb;
   const int i = blockIdx.x;
   if (threadIdx.x == 0) {
     s_np = 0;
@@ -438,44 +482,7 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
                           (double)(oz + Xi[2]) - pv.X[3 * i + 2]};
     bp_wall(rd, oid, oif, pv, F, T);
   };
-  if (threadIdx.x < 27) {
-    const int bin = cl.bin_of[i];
-    const int bc[3] = {bin % cl.nb[0], (bin / cl.nb[0]) % cl.nb[1], bin / (cl.nb[0] * cl.nb[1])};
-    int off[3][3], noff[3];
-    for (int k = 0; k < 3; ++k) noff[k] = bin_offsets(cl.nb[k], lv.per[k], bc[k], off[k]);
-    const int ix = threadIdx.x % 3, iy = (threadIdx.x / 3) % 3, iz = threadIdx.x / 9;
-    if (ix < noff[0] && iy < noff[1] && iz < noff[2]) {
-      const int bx = wrapi(bc[0] + off[0][ix], cl.nb[0]);
-      const int by = wrapi(bc[1] + off[1][iy], cl.nb[1]);
-      const int bz = wrapi(bc[2] + off[2][iz], cl.nb[2]);
-      const int b = bx + cl.nb[0] * (by + cl.nb[1] * bz);
-      const float rc2 = pv.r_cut * pv.r_cut;
-      const float smax = 2.0f * fmaxf(pv.sig_par, pv.sig_perp);
-      const float smax2 = smax * smax * 1.0001f;
-      const int e = cl.start[b + 1];
-      for (int k = cl.start[b]; k < e; ++k) {
-        const int j = cl.ids[k];
-        if (j == i) continue;
-        const float4 b0 = pv.kin[3 * j], b1 = pv.kin[3 * j + 1], b2 = pv.kin[3 * j + 2];
-        const int Xj[3] = {(int)b0.w, (int)b1.w, (int)b2.w};
-        const float fj[3] = {b0.x, b0.y, b0.z};
-        float r[3];
-        for (int m = 0; m < 3; ++m) r[m] = (float)imin_image(Xj[m] - Xi[m], dims[m], lv.per[m]) + (fj[m] - fi[m]);
-        const float r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-        // no contact distance exceeds 2 max(sigma_perp, sigma_par); nearer
-        // pairs first get the contact distance in FP32 (its error is ~1e-6
-        // relative, far inside the margin): only pairs at or within contact
-        // take the FP64 geometry
-        if (r2 >= rc2 || r2 > smax2) continue;
-        const float4 aj = pv.axis[j];
-        const float oj[3] = {aj.x, aj.y, aj.z};
-        if (!near_contact(r, r2, oif, oj, pv)) continue;
-        const int q = atomicAdd(&s_np, 1);
-        if (q < FQ_PAIR) s_pair[q] = j;
-        else pair_force(j);
-      }
-    }
-  }
+  if (threadIdx.x < 32) near_bins(lv, cl, cl.bin_of[i], s_nb);
   if (sb.bits) {
     const int R = (int)ceilf(pv.sigw_max) + 1;
     const int side = 2 * R + 1;
@@ -508,6 +515,30 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
         else wall_force(dx, oy, oz);
       }
     }
+  }
+  __syncthreads();
+  const float rc2 = pv.r_cut * pv.r_cut;
+  const float smax = 2.0f * fmaxf(pv.sig_par, pv.sig_perp);
+  const float smax2 = smax * smax * 1.0001f;
+  for (int t = threadIdx.x; t < s_nb.off[27]; t += FB) {
+    const int j = near_cell(cl, s_nb, t);
+    if (j == i) continue;
+    const float4 b0 = pv.kin[3 * j], b1 = pv.kin[3 * j + 1], b2 = pv.kin[3 * j + 2], aj = pv.axis[j];
+    const int Xj[3] = {(int)b0.w, (int)b1.w, (int)b2.w};
+    const float fj[3] = {b0.x, b0.y, b0.z};
+    float r[3];
+    for (int m = 0; m < 3; ++m) r[m] = (float)imin_image(Xj[m] - Xi[m], dims[m], lv.per[m]) + (fj[m] - fi[m]);
+    const float r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
+    // no contact distance exceeds 2 max(sigma_perp, sigma_par); nearer
+    // pairs first get the contact distance in FP32 (its error is ~1e-6
+    // relative, far inside the margin): only pairs at or within contact
+    // take the FP64 geometry
+    if (r2 >= rc2 || r2 > smax2) continue;
+    const float oj[3] = {aj.x, aj.y, aj.z};
+    if (!near_contact(r, r2, oif, oj, pv)) continue;
+    const int q = atomicAdd(&s_np, 1);
+    if (q < FQ_PAIR) s_pair[q] = j;
+    else pair_force(j);
   }
   __syncthreads();
   // the queued contacts, one per thread
@@ -562,7 +593,8 @@ __device__ void write_kin(const PartView &pv, int p, const double X[3], const do
 
 // node range of an ellipsoid along one axis (centre x, axis component o)
 __device__ __forceinline__ void aabb1(const PartView &pv, float x, float o, int &lo, int &hi) {
-  const float h = sqrtf(pv.Rperp2_f * (1.0f - o * o) + pv.Rpar2_f * o * o) + 0.01f;
+  const float h2 = pv.Rperp2_f * (1.0f - o * o) + pv.Rpar2_f * o * o;
+  const float h = h2 * rsqrtf(h2) + 0.01f;  // the root to 2 ulp
   lo = (int)floorf(x - h);
   hi = (int)ceilf(x + h);
 }
@@ -653,6 +685,7 @@ constexpr int LT = 128;  // threads of a link-reduction block
 #ifndef BL_CLAIMS_MINB
 #define BL_CLAIMS_MINB 7
 #endif
+template <bool FORCE>
 __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView lv, PartView pv) {
   __shared__ float shf[LT / 32][27];
   __shared__ int shi[LT / 32][6];
@@ -669,7 +702,7 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
   const float4 *rec = lv.rec + 2 * (size_t)p * lv.rec_cap;
   const bool tau1 = lv.omega == 1.0f;  // the sweep's records hold moments (tau = 1) or link sums
   for (int i = threadIdx.x; i < nrec; i += LT) {
-    const float4 r0 = rec[2 * i], r1 = rec[2 * i + 1];
+    const float4 r0 = rec[i], r1 = rec[lv.rec_cap + i];
     const unsigned n = __float_as_uint(r0.x);
     const uint32_t m = __float_as_uint(r0.y) & NB_SOLID;
     const float rho = lv.rho0 + r0.z;
@@ -688,14 +721,13 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
     // again from the node's moments (drho, u, uu, uF), else the sweep's sums
     float Fr[3];
     if (tau1) {
-      const float Fx = lv.has_force ? rho * lv.g[0] : 0.f, Fy = lv.has_force ? rho * lv.g[1] : 0.f,
-                  Fz = lv.has_force ? rho * lv.g[2] : 0.f;
-      const Collide ck = collide_coeffs<true>(r0.z, rho, r0.w, r1.x, r1.y, r1.z, 1.0f, Fx, Fy, Fz, r1.w);
+      const float Fx = FORCE ? rho * lv.g[0] : 0.f, Fy = FORCE ? rho * lv.g[1] : 0.f, Fz = FORCE ? rho * lv.g[2] : 0.f;
+      const Collide ck = collide_coeffs<FORCE>(r0.z, rho, r0.w, r1.x, r1.y, r1.z, 1.0f, Fx, Fy, Fz, r1.w);
       Fr[0] = Fr[1] = Fr[2] = 0.f;
       sfor<0, 9>([&](auto P) {
         constexpr int r = 2 * decltype(P)::value + 1;
         float fr, fb;
-        collide_pair<r, true>(ck, fr, fb);
+        collide_pair<r, FORCE>(ck, fr, fb);
         // 2 f~*_r c_r of r and of rbar (c_rbar = -c_r)
         float v = (m >> r) & 1u ? fr : 0.f;
         if ((m >> (r + 1)) & 1u) v -= fb;
@@ -958,10 +990,20 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
       else if (X >= (double)dim) X -= (double)dim;
     }
     const float wx = at(Wf, 0), wy = at(Wf, 1), wz = at(Wf, 2);
-    const float th = sqrtf(wx * wx + wy * wy + wz * wz);
-    float sn, cs;
-    sincosf(0.5f * th, &sn, &cs);
-    const float sh = sn / th;
+    const float t2 = wx * wx + wy * wy + wz * wz;
+    // cos(|W| / 2) and sin(|W| / 2) / |W| as their Taylor series in |W|^2 (for
+    // |W| <= 1, a fast cell, the first term left out is below 3e-9 of each)
+    float cs, sh;
+    if (t2 <= 1.0f) {
+      const float h2 = 0.25f * t2;
+      cs = fmaf(h2, fmaf(h2, fmaf(h2, fmaf(h2, 1.0f / 40320.0f, -1.0f / 720.0f), 1.0f / 24.0f), -0.5f), 1.0f);
+      sh = 0.5f * fmaf(h2, fmaf(h2, fmaf(h2, fmaf(h2, 1.0f / 362880.0f, -1.0f / 5040.0f), 1.0f / 120.0f), -1.0f / 6.0f), 1.0f);
+    } else {
+      const float th = sqrtf(t2);
+      float sn;
+      sincosf(0.5f * th, &sn, &cs);
+      sh = sn / th;
+    }
     // component l = k4 of the product: sum over m of +- dq[m] q[l xor m]
     const float dx = (k4 & 1) ? wx * sh : -(wx * sh);
     const float dy = (k4 == 1 || k4 == 2) ? wy * sh : -(wy * sh);
@@ -973,7 +1015,7 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
     double nn = nq * nq;
     nn += __shfl_xor_sync(FULL, nn, 1);
     nn += __shfl_xor_sync(FULL, nn, 2);
-    if (th > 0.f) q = nq * (1.5 - 0.5 * nn);  // 1 / sqrt(nn) to second order in (nn - 1)
+    if (t2 > 0.f) q = nq * (1.5 - 0.5 * nn);  // 1 / sqrt(nn) to second order in (nn - 1)
     // the exact axis (axis_exact), component by component
     const double a1 = at(q, k == 1 ? 2 : 1), b1 = at(q, k == 2 ? 1 : 3), a2 = at(q, k == 2 ? 2 : 0),
                  b2 = at(q, k == 1 ? 1 : 2);
@@ -1062,7 +1104,7 @@ __global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView
   // C in place for the directions of a second- or third-cell record: all its
   // populations requested together, then written
   auto direct = [&](int i) {
-    const float4 r0 = rec[2 * i];
+    const float4 r0 = rec[i];
     const unsigned n = __float_as_uint(r0.x);
     const uint32_t m = __float_as_uint(r0.y) & NB_SOLID;
     int yc[3];
@@ -1096,7 +1138,7 @@ __global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView
     float4 r0[PU];
 #pragma unroll
     for (int j = 0; j < PU; ++j)
-      if (i0 + j * LT < nrec) r0[j] = rec[2 * (i0 + j * LT)];
+      if (i0 + j * LT < nrec) r0[j] = rec[i0 + j * LT];
 #pragma unroll
     for (int j = 0; j < PU; ++j) {
       const int i = i0 + j * LT;
@@ -1120,7 +1162,7 @@ __global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView
   const int nq = full ? nrec : s_nq;
   for (int k = threadIdx.x; k < nq; k += LT) {
     const int i = full ? k : s_q[k];
-    if (!full || (__float_as_uint(rec[2 * i].y) & REC_DIRECT)) direct(i);
+    if (!full || (__float_as_uint(rec[i].y) & REC_DIRECT)) direct(i);
   }
 }
 
@@ -1768,13 +1810,19 @@ __global__ void k_nbm_update(LatticeView lv, ChangeList chg) {
 // deltapppm): the rows of the cell's box, each cut to the outer interval of
 // its ellipsoid at its current position, flattened over the block; every
 // node the cell owns adds its links into another cell or a wall to exact
-// integer sums (the cell's bounce links come from the sweep's records)
-constexpr int LB = 128;  // threads of a contact block (8 blocks fit an SM)
+// integer sums (the cell's bounce links come from the sweep's records).  Each
+// row writes its nodes into a list in shared memory, so that a node costs one
+// shared read instead of a search of the row table (67 -> 48 us on 256^3
+// beside the sweep, whose issue slots it shares), and only a node with
+// contact links has its owner read.
+constexpr int LB = 128;       // threads of a contact block (8 blocks fit an SM)
+constexpr int CLIST = 4096;   // nodes listed at once: row (7 bits), place in the row (9 bits)
 
 __global__ void __launch_bounds__(LB) k_contacts(LatticeView lv, PartView pv) {
   using D = D3Q19;
   __shared__ int sh_w[LB / 32 + 1];
   __shared__ int s_off[LB + 1], s_x0[LB], s_y[LB], s_z[LB];
+  __shared__ uint16_t s_node[CLIST];
   __shared__ int s_ci[LB / 32][6];
   const int p = blockIdx.x;
   const int lo1 = pv.box[6 * p + 1], lo2 = pv.box[6 * p + 2];
@@ -1805,27 +1853,37 @@ __global__ void __launch_bounds__(LB) k_contacts(LatticeView lv, PartView pv) {
     }
     int tot;
     const int off = block_scan<LB>(len, sh_w, &tot);
+    const bool listed = !__syncthreads_or(len > 511) && tot <= CLIST;
     s_off[threadIdx.x] = off;
     s_x0[threadIdx.x] = ao;
     s_y[threadIdx.x] = y;
     s_z[threadIdx.x] = z;
+    if (listed)
+      for (int j = 0; j < len; ++j) s_node[off + j] = (uint16_t)(threadIdx.x | (j << 7));
     __syncthreads();
     for (int k = threadIdx.x; k < tot; k += LB) {
-      // the row holding flattened node k: the last row starting at or before k
-      int lo = 0, hi = LB - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_off[mid] <= k) lo = mid;
-        else hi = mid - 1;
+      int lo = 0, j;
+      if (listed) {
+        lo = s_node[k] & 127;
+        j = s_node[k] >> 7;
+      } else {
+        // the row holding flattened node k: the last row starting at or before k
+        int hi = LB - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (s_off[mid] <= k) lo = mid;
+          else hi = mid - 1;
+        }
+        j = k - s_off[lo];
       }
-      int x = g.Xi[0] + s_x0[lo] + (k - s_off[lo]);
+      int x = g.Xi[0] + s_x0[lo] + j;
       if (lv.per[0]) x = wrapi(x, lv.nx);
       const int yy = s_y[lo], zz = s_z[lo];
       const unsigned nn = (unsigned)x + nx * (unsigned)yy + nxy * (unsigned)zz;
-      if (lv.owner[nn] != p) continue;
       // the node's contact links, kept in its neighbour word by the geometry passes
-      const unsigned cmask = lv.nbm[nn] & NB_SOLID;
-      if (cmask) {
+      const uint32_t w = lv.nbm[nn];
+      const unsigned cmask = (w & NB_FLUID) ? 0u : w & NB_SOLID;
+      if (cmask && lv.owner[nn] == p) {
         const int di[3] = {imin_image(x - g.Xi[0], lv.nx, lv.per[0]), imin_image(yy - g.Xi[1], lv.ny, lv.per[1]),
                            imin_image(zz - g.Xi[2], lv.nz, lv.per[2])};
         sfor<1, Q>([&](auto R) {
@@ -1929,24 +1987,30 @@ __global__ void k_pair_features(LatticeView lv, PartView pv, const int2 *pairs, 
 }
 
 // close pairs (gap_lo <= gap < gap_cut, relative speed |V_j - V_i| in
-// [speed_lo, speed_hi]) from the cell list, one block per cell
-// (lane b < 27 scans bin b), with their features
-__global__ void k_mlp_pairs(LatticeView lv, PartView pv, CellListView cl, PairBuf pb, float gap_lo, float gap_cut,
-                            float speed_lo, float speed_hi) {
+// [speed_lo, speed_hi]) from the cell list, one warp per cell, with their
+// features; a pair whose centres are farther apart than the largest contact
+// distance and the cut-off is left before its features are formed
+__global__ void __launch_bounds__(32) k_mlp_pairs(LatticeView lv, PartView pv, CellListView cl, PairBuf pb,
+                                                  float gap_lo, float gap_cut, float speed_lo, float speed_hi) {
+  __shared__ NearBins s_nb;
   const int i = blockIdx.x;
-  if (threadIdx.x >= 27) return;
-  const int bin = cl.bin_of[i];
-  const int bc[3] = {bin % cl.nb[0], (bin / cl.nb[0]) % cl.nb[1], bin / (cl.nb[0] * cl.nb[1])};
-  int off[3][3], noff[3];
-  for (int k = 0; k < 3; ++k) noff[k] = bin_offsets(cl.nb[k], lv.per[k], bc[k], off[k]);
-  const int ix = threadIdx.x % 3, iy = (threadIdx.x / 3) % 3, iz = threadIdx.x / 9;
-  if (ix >= noff[0] || iy >= noff[1] || iz >= noff[2]) return;
-  const int b = wrapi(bc[0] + off[0][ix], cl.nb[0]) +
-                cl.nb[0] * (wrapi(bc[1] + off[1][iy], cl.nb[1]) + cl.nb[1] * wrapi(bc[2] + off[2][iz], cl.nb[2]));
-  const int e = cl.start[b + 1];
-  for (int k = cl.start[b]; k < e; ++k) {
-    const int j = cl.ids[k];
+  near_bins(lv, cl, cl.bin_of[i], s_nb);
+  __syncwarp();
+  CellGeo g;
+  cell_geo(pv, pv.kin, i, g);
+  const int dims[3] = {lv.nx, lv.ny, lv.nz};
+  const float far = (2.0f * pv.Rmax_f + gap_cut) * 1.0001f + 1e-3f;
+  for (int t = threadIdx.x; t < s_nb.off[27]; t += 32) {
+    const int j = near_cell(cl, s_nb, t);
     if (j == i) continue;
+    CellGeo h;
+    cell_geo(pv, pv.kin, j, h);
+    float r2 = 0.f;
+    for (int m = 0; m < 3; ++m) {
+      const float d = (float)imin_image(h.Xi[m] - g.Xi[m], dims[m], lv.per[m]) + (h.Xf[m] - g.Xf[m]);
+      r2 += d * d;
+    }
+    if (!(far > 0.f) || r2 > far * far) continue;
     float f[14], R[3][3];
     pair_features(lv, pv, i, j, f, R);
     if (!(f[7] >= gap_lo && f[7] < gap_cut)) continue;  // outside the range: the plain method
@@ -2003,7 +2067,8 @@ void launch_sums_solve(int dtype, const LatticeView &lv, const PartView &pv, int
   (void)dtype;
   (void)par;
   if (pv.n == 0) return;
-  k_link_reduce<<<pv.n, LT, 0, st>>>(lv, pv);
+  if (lv.has_force) k_link_reduce<true><<<pv.n, LT, 0, st>>>(lv, pv);
+  else k_link_reduce<false><<<pv.n, LT, 0, st>>>(lv, pv);
   k_solve<<<nblk(pv.n, SOLVE_CELLS), 32, 0, st>>>(lv, pv);
   *nl += 2;
 }
