@@ -162,12 +162,20 @@ __device__ __forceinline__ void load_x(const float *x, int B, int r0, const floa
   }
 }
 
+// the first n packed operands into shared memory, 16 bytes a thread (n is a
+// multiple of 8; both arrays are 16-byte aligned)
+__device__ __forceinline__ void load_operands(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int n) {
+  for (int i = threadIdx.x; i < n / 8; i += blockDim.x)
+    reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(src)[i];
+}
+static_assert(P_W2T % 8 == 0 && P_TOTAL % 8 == 0, "operand copies in 16-byte words");
+
 // inference on raw features: y = network(x) in raw output units (B x 6);
 // with Bdev the row count is min(*Bdev, B), read on the device
 __global__ void __launch_bounds__(128) k_mlp_forward(MlpDev m, const float *x, int B, const int *Bdev, float *y) {
   __shared__ __align__(16) __nv_bfloat16 wp[P_TOTAL];
   if (Bdev) B = min(*Bdev, B);
-  for (int i = threadIdx.x; i < P_W2T; i += blockDim.x) wp[i] = m.wp[i];
+  load_operands(wp, m.wp, P_W2T);
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   for (int r0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 16; r0 < B; r0 += gridDim.x * 64) {
@@ -185,195 +193,226 @@ __global__ void __launch_bounds__(128) k_mlp_forward(MlpDev m, const float *x, i
 }
 
 // Loss and gradient of the mean squared error of the standardised outputs
-// over B samples (targets in raw units).  Each block adds its tiles into
-// shared FP32 sums and writes one partial row of NPAR + 1 values (gradient,
-// then the loss sum); k_mlp_reduce adds the partial rows in block order.
-constexpr int DS = 24;  // row stride of the transposed [unit][sample] BF16 stages
+// over B samples (targets in raw units).  A block of eight warps takes 128
+// samples at a time: each warp runs forward and backward over 16 of them and
+// stages its activations and deltas, transposed, in shared memory; then the
+// block forms the weight gradients over all 128, each warp its own rows and
+// columns, in accumulators that stay in registers over the block's samples.
+// (With each warp adding every product of its 16 samples into shared FP32 sums
+// by atomics, 5510 of them per tile, the kernel took 115 us for 39400 samples;
+// its arithmetic takes about 5.)  Each block writes one partial row of NPAR +
+// 1 values (gradient, then the loss sum); k_mlp_reduce adds the rows in block
+// order.
+constexpr int DS = 24;   // row stride of the transposed [unit][sample] BF16 stages
+constexpr int GW = 8;    // warps of a gradient block
+// rows of a warp's stage: xT 16, h1T 64, h2T 64, d1T 64, d2T 64, d3T 16 (rows >= 6 zero)
+constexpr int R_X = 0, R_H1 = 16, R_H2 = R_H1 + NH, R_D1 = R_H2 + NH, R_D2 = R_D1 + NH, R_D3 = R_D2 + NH,
+              R_ALL = R_D3 + 16;
+constexpr int NBIAS = 2 * NH + 8;  // bias sums of a warp: b1, b2, b3 (6, padded)
 
-__global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float *x, const float *yt, int B,
-                                                  float *partial) {
+__global__ void __launch_bounds__(32 * GW, 1) k_mlp_grad(MlpDev m, const float *x, const float *yt, int B,
+                                                         float *partial) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __nv_bfloat16 *wp = reinterpret_cast<__nv_bfloat16 *>(smem_raw);
-  float *gs = reinterpret_cast<float *>(smem_raw + sizeof(__nv_bfloat16) * P_TOTAL);  // NPAR + 1 sums
-  __nv_bfloat16 *stg = reinterpret_cast<__nv_bfloat16 *>(gs + NPAR + 2);              // per warp stages
-  for (int i = threadIdx.x; i < P_TOTAL; i += blockDim.x) wp[i] = m.wp[i];
-  for (int i = threadIdx.x; i < NPAR + 1; i += blockDim.x) gs[i] = 0.f;
-  __syncthreads();
+  __nv_bfloat16 *stg = wp + P_TOTAL;                                     // GW stages
+  float *sb = reinterpret_cast<float *>(stg + (size_t)GW * R_ALL * DS);  // GW x NBIAS, then GW losses
+  load_operands(wp, m.wp, P_TOTAL);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, wid = threadIdx.x >> 5;
-  // per-warp transposed stages, [unit][sample]: xT 16 rows, h1T 64, h2T 64,
-  // d1T 64, d2T 64, d3T 16 (rows >= 6 zero)
-  __nv_bfloat16 *st = stg + (size_t)wid * (16 + 64 * 4 + 16) * DS;
-  __nv_bfloat16 *xT = st, *h1T = xT + 16 * DS, *h2T = h1T + 64 * DS, *d1T = h2T + 64 * DS, *d2T = d1T + 64 * DS,
-                *d3T = d2T + 64 * DS;
+  __nv_bfloat16 *st = stg + (size_t)wid * R_ALL * DS;
   const float inv_b = 1.0f / (float)B;
   const float *my = m.norm + 2 * NI, *sy = m.norm + 2 * NI + NO;
+  // this warp's share of the weight gradients: rows 16 mi.. of W1 and W2,
+  // columns 8 half.. of W1 and 32 half.. of W2, columns 8 wid.. of W3
+  const int mi = wid & 3, half = wid >> 2;
+  float c1[4] = {0.f, 0.f, 0.f, 0.f}, c2[4][4], c3[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) c2[j][0] = c2[j][1] = c2[j][2] = c2[j][3] = 0.f;
+  float b1[8][2], b2[8][2], b3[2] = {0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < 8; ++j) b1[j][0] = b1[j][1] = b2[j][0] = b2[j][1] = 0.f;
   float loss = 0.f;
-  for (int r0 = (blockIdx.x * 4 + wid) * 16; r0 < B; r0 += gridDim.x * 64) {
-    float xs[8];
-    load_x(x, B, r0, m.norm, xs);
-    Tile T;
-    tile_forward(wp, m.theta, xs, T);
-    // d3 = 2 (y~ - t~) / B on valid rows and outputs
-    float d3[4];
+  __syncthreads();
+  const int ntiles = (B + 15) / 16;
+  for (int t0 = blockIdx.x * GW; t0 < ntiles; t0 += gridDim.x * GW) {
+    const int r0 = (t0 + wid) * 16;  // (rows >= B give zero deltas)
+    {
+      float xs[8];
+      load_x(x, B, r0, m.norm, xs);
+      Tile T;
+      tile_forward(wp, m.theta, xs, T);
+      // d3 = 2 (y~ - t~) / B on valid rows and outputs
+      float d3[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int r = r0 + g + (e >= 2 ? 8 : 0), c = 2 * t + (e & 1);
-      float d = 0.f;
-      if (r < B && c < NO) {
-        const float res = T.y[e] - (yt[(size_t)r * NO + c] - my[c]) / sy[c];
-        loss += res * res;
-        d = 2.0f * res * inv_b;
+      for (int e = 0; e < 4; ++e) {
+        const int r = r0 + g + (e >= 2 ? 8 : 0), c = 2 * t + (e & 1);
+        float d = 0.f;
+        if (r < B && c < NO) {
+          const float res = T.y[e] - (yt[(size_t)r * NO + c] - my[c]) / sy[c];
+          loss += res * res;
+          d = 2.0f * res * inv_b;
+        }
+        d3[e] = d;
       }
-      d3[e] = d;
-    }
-    // d2 = (d3 W3) * (1 - h2^2): A = d3 (k = outputs, 8..15 zero), B = W3t
-    const uint32_t a3[4] = {pack_bf16(d3[0], d3[1]), pack_bf16(d3[2], d3[3]), 0u, 0u};
-    float d2[8][4];
+      // d2 = (d3 W3) * (1 - h2^2): A = d3 (k = outputs, 8..15 zero), B = W3t
+      const uint32_t a3[4] = {pack_bf16(d3[0], d3[1]), pack_bf16(d3[2], d3[3]), 0u, 0u};
+      float d2[8][4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      d2[j][0] = d2[j][1] = d2[j][2] = d2[j][3] = 0.f;
-      mma16816(d2[j], a3, ld2(wp + P_W3T, S3T, 8 * j + g, 2 * t), 0u);
+      for (int j = 0; j < 8; ++j) {
+        d2[j][0] = d2[j][1] = d2[j][2] = d2[j][3] = 0.f;
+        mma16816(d2[j], a3, ld2(wp + P_W3T, S3T, 8 * j + g, 2 * t), 0u);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) d2[j][e] *= 1.0f - T.h2[j][e] * T.h2[j][e];
-    }
-    // d1 = (d2 W2) * (1 - h1^2): B = W2t
-    float d1[8][4];
+        for (int e = 0; e < 4; ++e) d2[j][e] *= 1.0f - T.h2[j][e] * T.h2[j][e];
+      }
+      // d1 = (d2 W2) * (1 - h1^2): B = W2t
+      float d1[8][4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) d1[j][0] = d1[j][1] = d1[j][2] = d1[j][3] = 0.f;
+      for (int j = 0; j < 8; ++j) d1[j][0] = d1[j][1] = d1[j][2] = d1[j][3] = 0.f;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const uint32_t ak[4] = {pack_bf16(d2[2 * kk][0], d2[2 * kk][1]), pack_bf16(d2[2 * kk][2], d2[2 * kk][3]),
-                              pack_bf16(d2[2 * kk + 1][0], d2[2 * kk + 1][1]),
-                              pack_bf16(d2[2 * kk + 1][2], d2[2 * kk + 1][3])};
+      for (int kk = 0; kk < 4; ++kk) {
+        const uint32_t ak[4] = {pack_bf16(d2[2 * kk][0], d2[2 * kk][1]), pack_bf16(d2[2 * kk][2], d2[2 * kk][3]),
+                                pack_bf16(d2[2 * kk + 1][0], d2[2 * kk + 1][1]),
+                                pack_bf16(d2[2 * kk + 1][2], d2[2 * kk + 1][3])};
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          mma16816(d1[j], ak, ld2(wp + P_W2T, S2T, 8 * j + g, 16 * kk + 2 * t),
+                   ld2(wp + P_W2T, S2T, 8 * j + g, 16 * kk + 2 * t + 8));
+      }
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        mma16816(d1[j], ak, ld2(wp + P_W2T, S2T, 8 * j + g, 16 * kk + 2 * t),
-                 ld2(wp + P_W2T, S2T, 8 * j + g, 16 * kk + 2 * t + 8));
-    }
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+        for (int e = 0; e < 4; ++e) d1[j][e] *= 1.0f - T.h1[j][e] * T.h1[j][e];
+      // bias gradients: sums over the samples (FP32 deltas)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) d1[j][e] *= 1.0f - T.h1[j][e] * T.h1[j][e];
-    // stage the transposed operands: element (sample s, unit u) -> [u][s]
-    __syncwarp();
-    {
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          b1[j][e] += d1[j][e] + d1[j][e + 2];
+          b2[j][e] += d2[j][e] + d2[j][e + 2];
+        }
+      b3[0] += d3[0] + d3[2];
+      b3[1] += d3[1] + d3[3];
+      // stage the transposed operands: element (sample s, unit u) -> [u][s]
       const int sr[2] = {g, g + 8};
-      const float xv[8] = {xs[0], xs[1], xs[2], xs[3], xs[4], xs[5], xs[6], xs[7]};
       const int rsel[8] = {0, 0, 1, 1, 0, 0, 1, 1}, cols[8] = {2 * t, 2 * t + 1, 2 * t, 2 * t + 1,
                                                                 2 * t + 8, 2 * t + 9, 2 * t + 8, 2 * t + 9};
 #pragma unroll
-      for (int e = 0; e < 8; ++e) xT[cols[e] * DS + sr[rsel[e]]] = __float2bfloat16_rn(xv[e]);
+      for (int e = 0; e < 8; ++e) st[(R_X + cols[e]) * DS + sr[rsel[e]]] = __float2bfloat16_rn(xs[e]);
 #pragma unroll
       for (int j = 0; j < 8; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int s = sr[e >> 1], u = 8 * j + 2 * t + (e & 1);
-          h1T[u * DS + s] = __float2bfloat16_rn(T.h1[j][e]);
-          h2T[u * DS + s] = __float2bfloat16_rn(T.h2[j][e]);
-          d1T[u * DS + s] = __float2bfloat16_rn(d1[j][e]);
-          d2T[u * DS + s] = __float2bfloat16_rn(d2[j][e]);
+          const int o = (8 * j + 2 * t + (e & 1)) * DS + sr[e >> 1];
+          st[R_H1 * DS + o] = __float2bfloat16_rn(T.h1[j][e]);
+          st[R_H2 * DS + o] = __float2bfloat16_rn(T.h2[j][e]);
+          st[R_D1 * DS + o] = __float2bfloat16_rn(d1[j][e]);
+          st[R_D2 * DS + o] = __float2bfloat16_rn(d2[j][e]);
         }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) d3T[(2 * t + (e & 1)) * DS + sr[e >> 1]] = __float2bfloat16_rn(d3[e]);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) d3T[(8 + 2 * t + (e & 1)) * DS + sr[e >> 1]] = __float2bfloat16_rn(0.f);
+      for (int e = 0; e < 4; ++e) {
+        st[(R_D3 + 2 * t + (e & 1)) * DS + sr[e >> 1]] = __float2bfloat16_rn(d3[e]);
+        st[(R_D3 + 8 + 2 * t + (e & 1)) * DS + sr[e >> 1]] = __float2bfloat16_rn(0.f);
+      }
     }
-    __syncwarp();
-    // weight gradients dW = dT^T-products over the 16 samples: A = dT [unit][sample]
-    // (16 x 16 per m tile), B = hT [unit][sample] read as (k = sample, n = unit)
+    __syncthreads();
+    // weight gradients dT^T-products over the 128 samples, 16 (one stage) at a
+    // time: A = dT [unit][sample] (16 x 16), B = hT [unit][sample] read as
+    // (k = sample, n = unit)
     auto afrag = [&](const __nv_bfloat16 *src, int m0, uint32_t (&a)[4]) {
       a[0] = ld2(src, DS, m0 + g, 2 * t);
       a[1] = ld2(src, DS, m0 + g + 8, 2 * t);
       a[2] = ld2(src, DS, m0 + g, 2 * t + 8);
       a[3] = ld2(src, DS, m0 + g + 8, 2 * t + 8);
     };
-    auto acc = [&](int off, int ncols, int m0, int n0, const float (&c)[4], int mrows) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int r = m0 + g + (e >= 2 ? 8 : 0), col = n0 + 2 * t + (e & 1);
-        if (r < mrows && col < ncols) atomicAdd(&gs[off + r * ncols + col], c[e]);
-      }
+    auto bmma = [&](float (&c)[4], const uint32_t (&a)[4], const __nv_bfloat16 *src, int n0) {
+      mma16816(c, a, ld2(src, DS, n0 + g, 2 * t), ld2(src, DS, n0 + g, 2 * t + 8));
     };
-    // dW1 (64 x 14): m tiles of d1T, n tiles of xT (2 tiles, 16 columns)
-#pragma unroll
-    for (int mi = 0; mi < 4; ++mi) {
+#pragma unroll 2
+    for (int w = 0; w < GW; ++w) {
+      const __nv_bfloat16 *sw = stg + (size_t)w * R_ALL * DS;
       uint32_t a[4];
-      afrag(d1T, 16 * mi, a);
+      afrag(sw + R_D2 * DS, 16 * mi, a);
 #pragma unroll
-      for (int nj = 0; nj < 2; ++nj) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma16816(c, a, ld2(xT, DS, 8 * nj + g, 2 * t), ld2(xT, DS, 8 * nj + g, 2 * t + 8));
-        acc(OFF_W1, NI, 16 * mi, 8 * nj, c, NH);
-      }
+      for (int j = 0; j < 4; ++j) bmma(c2[j], a, sw + R_H1 * DS, 32 * half + 8 * j);
+      afrag(sw + R_D1 * DS, 16 * mi, a);
+      bmma(c1, a, sw + R_X * DS, 8 * half);
+      afrag(sw + R_D3 * DS, 0, a);
+      bmma(c3, a, sw + R_H2 * DS, 8 * wid);
     }
-    // dW2 (64 x 64): d2T x h1T
+    __syncthreads();  // the stages are read: free for the next samples
+  }
+  float *row = partial + (size_t)blockIdx.x * (NPAR + 1);
 #pragma unroll
-    for (int mi = 0; mi < 4; ++mi) {
-      uint32_t a[4];
-      afrag(d2T, 16 * mi, a);
+  for (int e = 0; e < 4; ++e) {
+    const int r = g + (e >= 2 ? 8 : 0), c = 2 * t + (e & 1);
+    if (8 * half + c < NI) row[OFF_W1 + (16 * mi + r) * NI + 8 * half + c] = c1[e];
 #pragma unroll
-      for (int nj = 0; nj < 8; ++nj) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma16816(c, a, ld2(h1T, DS, 8 * nj + g, 2 * t), ld2(h1T, DS, 8 * nj + g, 2 * t + 8));
-        acc(OFF_W2, NH, 16 * mi, 8 * nj, c, NH);
-      }
-    }
-    // dW3 (6 x 64): d3T x h2T
-    {
-      uint32_t a[4];
-      afrag(d3T, 0, a);
+    for (int j = 0; j < 4; ++j) row[OFF_W2 + (16 * mi + r) * NH + 32 * half + 8 * j + c] = c2[j][e];
+    if (r < NO) row[OFF_W3 + r * NH + 8 * wid + c] = c3[e];
+  }
+  // the biases and the loss: over the lanes of a warp, then over the warps in order
+  float *wb = sb + wid * NBIAS;
 #pragma unroll
-      for (int nj = 0; nj < 8; ++nj) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma16816(c, a, ld2(h2T, DS, 8 * nj + g, 2 * t), ld2(h2T, DS, 8 * nj + g, 2 * t + 8));
-        acc(OFF_W3, NH, 0, 8 * nj, c, NO);
-      }
-    }
-    // bias gradients: sums over the samples (FP32 deltas)
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        float s1 = d1[j][e] + d1[j][e + 2], s2 = d2[j][e] + d2[j][e + 2];
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if (g == 0) {
-          atomicAdd(&gs[OFF_B1 + 8 * j + 2 * t + e], s1);
-          atomicAdd(&gs[OFF_B2 + 8 * j + 2 * t + e], s2);
-        }
-      }
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      float s3 = d3[e] + d3[e + 2];
+      float s1 = b1[j][e], s2 = b2[j][e];
 #pragma unroll
-      for (int o = 4; o < 32; o <<= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-      if (g == 0 && 2 * t + e < NO) atomicAdd(&gs[OFF_B3 + 2 * t + e], s3);
+      for (int o = 4; o < 32; o <<= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      }
+      if (g == 0) {
+        wb[8 * j + 2 * t + e] = s1;
+        wb[NH + 8 * j + 2 * t + e] = s2;
+      }
     }
-    __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    float s3 = b3[e];
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+    if (g == 0) wb[2 * NH + 2 * t + e] = s3;
   }
-  // the block's loss sum, then its partial row
   loss = warp_sum(loss);
-  if (lane == 0) atomicAdd(&gs[NPAR], loss * inv_b);
+  if (lane == 0) sb[GW * NBIAS + wid] = loss * inv_b;
   __syncthreads();
-  for (int i = threadIdx.x; i < NPAR + 1; i += blockDim.x) partial[(size_t)blockIdx.x * (NPAR + 1) + i] = gs[i];
+  for (int i = threadIdx.x; i < NBIAS; i += blockDim.x) {
+    float s = 0.f;
+    for (int w = 0; w < GW; ++w) s += sb[w * NBIAS + i];
+    if (i < NH) row[OFF_B1 + i] = s;
+    else if (i < 2 * NH) row[OFF_B2 + i - NH] = s;
+    else if (i < 2 * NH + NO) row[OFF_B3 + i - 2 * NH] = s;
+  }
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int w = 0; w < GW; ++w) s += sb[GW * NBIAS + w];
+    row[NPAR] = s;
+  }
 }
 
-// sums the partial rows in block order (a fixed order: the same data give
-// the same gradient bit for bit)
-__global__ void k_mlp_reduce(const float *partial, int nblocks, float *grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPAR + 1) return;
+// sums the partial rows in a fixed order (the same data give the same
+// gradient bit for bit): a block takes 32 values, its eight warps a share of
+// the rows each, added in warp order
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float *partial, int nblocks, float *grad) {
+  __shared__ float sh[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  const int per = (nblocks + 7) / 8, b0 = w * per, b1 = min(b0 + per, nblocks);
   float s = 0.f;
-  for (int b = 0; b < nblocks; ++b) s += partial[(size_t)b * (NPAR + 1) + i];
-  grad[i] = s;
+  if (i < NPAR + 1)
+    for (int b = b0; b < b1; ++b) s += partial[(size_t)b * (NPAR + 1) + i];
+  sh[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && i < NPAR + 1) {
+    for (int k = 1; k < 8; ++k) s += sh[k][lane];
+    grad[i] = s;
+  }
 }
 
-// Adam on the FP32 master parameters (step count k >= 1)
-__global__ void k_mlp_adam(float *theta, const float *grad, float *m1, float *m2, float lr, float b1, float b2,
-                           float eps, int k) {
+// Adam on the FP32 master parameters (step count k >= 1), and the BF16 operand
+// copies of each (k_mlp_pack has set their padding)
+__global__ void k_mlp_adam(float *theta, const float *grad, float *m1, float *m2, __nv_bfloat16 *wp, float lr,
+                           float b1, float b2, float eps, int k) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= NPAR) return;
   const float gi = grad[i];
@@ -381,7 +420,20 @@ __global__ void k_mlp_adam(float *theta, const float *grad, float *m1, float *m2
   m1[i] = a;
   m2[i] = v;
   const float ah = a / (1.0f - powf(b1, (float)k)), vh = v / (1.0f - powf(b2, (float)k));
-  theta[i] -= lr * ah / (sqrtf(vh) + eps);
+  const float th = theta[i] - lr * ah / (sqrtf(vh) + eps);
+  theta[i] = th;
+  const __nv_bfloat16 v16 = __float2bfloat16_rn(th);
+  if (i < OFF_B1) {
+    wp[P_W1 + (i / NI) * S1 + i % NI] = v16;
+  } else if (i >= OFF_W2 && i < OFF_B2) {
+    const int j = i - OFF_W2, n = j / NH, kk = j % NH;
+    wp[P_W2 + n * S2 + kk] = v16;
+    wp[P_W2T + kk * S2T + n] = v16;
+  } else if (i >= OFF_W3 && i < OFF_B3) {
+    const int j = i - OFF_W3, n = j / NH, kk = j % NH;
+    wp[P_W3 + n * S3 + kk] = v16;
+    wp[P_W3T + kk * S3T + n] = v16;
+  }
 }
 
 }  // namespace bl
@@ -403,8 +455,7 @@ struct bl_mlp {
 static const int MLP_BLOCKS = 152;
 
 static size_t grad_smem() {
-  return sizeof(__nv_bfloat16) * P_TOTAL + sizeof(float) * (NPAR + 2) +
-         sizeof(__nv_bfloat16) * 4 * (16 + 64 * 4 + 16) * DS;
+  return sizeof(__nv_bfloat16) * (P_TOTAL + (size_t)GW * R_ALL * DS) + sizeof(float) * (GW * NBIAS + GW);
 }
 
 static int mlp_pack(bl_mlp *m) {
@@ -486,8 +537,10 @@ extern "C" int bl_mlp_forward(bl_mlp *m, const float *x, int B, float *y) {
 
 extern "C" int bl_mlp_grad(bl_mlp *m, const float *x, const float *y, int B, float *loss, float *grad) {
   if (!m || B < 1 || !x || !y) return BL_EINVAL;
-  k_mlp_grad<<<m->nblocks, 128, grad_smem(), m->stream>>>(mlp_dev(m), x, y, B, m->partial);
-  k_mlp_reduce<<<(NPAR + 1 + 255) / 256, 256, 0, m->stream>>>(m->partial, m->nblocks, m->grad);
+  // one block per SM, fewer where the samples fill fewer
+  const int nb = (int)min((long long)m->nblocks, ((long long)B + 16 * GW - 1) / (16 * GW));
+  k_mlp_grad<<<nb, 32 * GW, grad_smem(), m->stream>>>(mlp_dev(m), x, y, B, m->partial);
+  k_mlp_reduce<<<(NPAR + 1 + 31) / 32, 256, 0, m->stream>>>(m->partial, nb, m->grad);
   if (cudaGetLastError() != cudaSuccess) return BL_ECUDA;
   if (loss && cudaMemcpyAsync(loss, m->grad + NPAR, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return BL_ECUDA;
@@ -501,9 +554,9 @@ extern "C" int bl_mlp_adam(bl_mlp *m, float lr, float beta1, float beta2, float 
   if (!m || !(lr > 0.f) || !(beta1 >= 0.f && beta1 < 1.f) || !(beta2 >= 0.f && beta2 < 1.f) || !(eps > 0.f))
     return BL_EINVAL;
   m->k++;
-  k_mlp_adam<<<(NPAR + 255) / 256, 256, 0, m->stream>>>(m->theta, m->grad, m->m1, m->m2, lr, beta1, beta2, eps, m->k);
-  if (cudaGetLastError() != cudaSuccess) return BL_ECUDA;
-  return mlp_pack(m);
+  k_mlp_adam<<<(NPAR + 63) / 64, 64, 0, m->stream>>>(m->theta, m->grad, m->m1, m->m2, m->wp, lr, beta1, beta2, eps,
+                                                     m->k);
+  return cudaGetLastError() == cudaSuccess ? BL_OK : BL_ECUDA;
 }
 
 namespace bl {
