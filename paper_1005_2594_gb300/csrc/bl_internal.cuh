@@ -164,11 +164,36 @@ constexpr uint32_t NBC_CELL = 0x7FFFFFFFu;
 constexpr uint32_t NBX_NONE = 0xFFFFu;
 
 // momentum given to each wall id by its bounce-back links: variable part in
-// FP64, constant part 2 alpha_r rho_bar c_r as exact integer sums of m_r c_r
+// FP64, constant part 2 alpha_r rho_bar c_r as exact integer sums of m_r c_r.
+// WALL_COPIES sets of sums, a block adding to one of them: every warp beside a
+// wall adds to its wall's six words, and on one set those additions stood in
+// line at one L2 slice (the indexed sweep of a 2.2 M node vessel loop took 132
+// us in the even step, 85 of them for this).  The read-out adds the sets up.
+constexpr int WALL_COPIES = 128;
+constexpr int WALL_SUMS = NWALL * 3;
 struct WallAcc {
-  double *F;     // 8 x 3
-  long long *K;  // 8 x 3
+  double *F;     // WALL_COPIES x 8 x 3
+  long long *K;  // WALL_COPIES x 8 x 3
 };
+
+// the set of sums this block adds to
+__device__ __forceinline__ WallAcc wall_copy(const WallAcc &wa) {
+  const unsigned c = (blockIdx.x + 31u * blockIdx.y + 57u * blockIdx.z) % (unsigned)WALL_COPIES;
+  return WallAcc{wa.F + c * WALL_SUMS, wa.K + c * WALL_SUMS};
+}
+
+// the sets' sums as momentum per wall and component (host)
+inline void wall_total(const double *F, const long long *K, double rho0, double *out) {
+  for (int i = 0; i < WALL_SUMS; ++i) {
+    double f = 0.0;
+    long long k = 0;
+    for (int c = 0; c < WALL_COPIES; ++c) {
+      f += F[c * WALL_SUMS + i];
+      k += K[c * WALL_SUMS + i];
+    }
+    out[i] = f + rho0 / 18.0 * (double)k;
+  }
+}
 
 // Cells.  Their bounce links come from the sweep's link records
 // (LatticeView::rec); contact links enter as exact integer sums cK, cIT.

@@ -294,11 +294,11 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
       rc = fail(c, BL_ECUDA, "streams");
       break;
     }
-    if (cudaMalloc(&c->wacc.F, sizeof(double) * bl::NWALL * 3) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "wall"); break; }
-    if (cudaMalloc(&c->wacc.K, sizeof(long long) * bl::NWALL * 3) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "wall"); break; }
+    if (cudaMalloc(&c->wacc.F, sizeof(double) * bl::WALL_COPIES * bl::WALL_SUMS) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "wall"); break; }
+    if (cudaMalloc(&c->wacc.K, sizeof(long long) * bl::WALL_COPIES * bl::WALL_SUMS) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "wall"); break; }
     cudaMemsetAsync(c->status, 0, sizeof(int), c->stream);
-    cudaMemsetAsync(c->wacc.F, 0, sizeof(double) * bl::NWALL * 3, c->stream);
-    cudaMemsetAsync(c->wacc.K, 0, sizeof(long long) * bl::NWALL * 3, c->stream);
+    cudaMemsetAsync(c->wacc.F, 0, sizeof(double) * bl::WALL_COPIES * bl::WALL_SUMS, c->stream);
+    cudaMemsetAsync(c->wacc.K, 0, sizeof(long long) * bl::WALL_COPIES * bl::WALL_SUMS, c->stream);
     launch_init(c->dtype, lv, c->stream);
     launch_fill_int(c->claim, lv.N, INT_MAX, c->stream);
     c->launches += 2;
@@ -882,14 +882,14 @@ extern "C" int bl_force_parts_get(bl_ctx *c, double *Fh, double *Th, double *Fp,
 extern "C" int bl_wall_momentum_get(bl_ctx *c, double *wallmom) {
   if (!c || !wallmom) return BL_EINVAL;
   if (c->sticky) return c->sticky;
-  double F[bl::NWALL * 3];
-  long long K[bl::NWALL * 3];
+  double F[bl::WALL_COPIES * bl::WALL_SUMS];
+  long long K[bl::WALL_COPIES * bl::WALL_SUMS];
   CU(cudaMemcpyAsync(F, c->wacc.F, sizeof(F), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaMemcpyAsync(K, c->wacc.K, sizeof(K), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
   CU(cudaMemsetAsync(c->wacc.F, 0, sizeof(F), c->stream));
   CU(cudaMemsetAsync(c->wacc.K, 0, sizeof(K), c->stream));
-  for (int i = 0; i < bl::NWALL * 3; ++i) wallmom[i] = F[i] + c->lp.rho0 / 18.0 * (double)K[i];
+  wall_total(F, K, c->lp.rho0, wallmom);
   return BL_OK;
 }
 

@@ -6,9 +6,22 @@
 // a few per cent of its bounding box.  Here the fluid nodes of a lattice with
 // walls (face walls and a wall mask, as for the dense lattice) get compact
 // indices in dense node order (x fastest, so that runs along x stay
-// contiguous and a warp's reads coalesce), and a table gives each fluid
-// node's 18 neighbours: a fluid index, or -1 - w for a wall of id w.  Memory
-// and traffic scale with the lumen, not the box.
+// contiguous and a warp's reads coalesce).  Memory and traffic scale with the
+// lumen, not the box.
+//
+// Neighbours.  A node's neighbours along x are the indices beside its own, and
+// in each of the eight other lattice rows (dy, dz) around it they are b - 1, b
+// and b + 1 where they are fluid, with b the number of fluid nodes before the
+// node's x in that row's order; along a run of nodes b grows by one with each
+// node whose (dy, dz) neighbour is fluid.  So a node stores one word, with a
+// bit per open direction, and each segment (a run of nodes consecutive in x
+// within one warp's 32 nodes) stores the eight b of its first node, from which
+// the lanes count their own with a warp vote per row.  That is 5 to 6 bytes per
+// node where a table of 18 neighbours took 72, and the even step reads the
+// word alone.  Nodes for which this does not hold, the ends of a periodic row
+// and nodes between walls of different ids, are segments of their own that
+// point to an explicit table; the builder checks every node against the
+// neighbour table.
 //
 // The sweep is the dense lattice's plasma update (Sec. II: moments, Guo
 // forcing, BGK toward the third-order equilibrium, mid-link bounce-back with
@@ -26,6 +39,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/bloodlb.h"
@@ -37,44 +51,138 @@ namespace {
 
 inline unsigned nblk(unsigned n, unsigned b) { return (n + b - 1) / b; }
 
+// word of a node: bit 0 starts a segment, bits 1..18 open directions, bits
+// 20..22 the wall id of its closed ones, SP_TABLE neighbours in the table
+constexpr uint32_t SP_START = 1u;
+constexpr int SP_WALL = 20;
+constexpr uint32_t SP_TABLE = 1u << 24;
+
+// the rows (dy, dz) in the order of a segment's eight b, by their dx = 0
+// direction
+__host__ __device__ constexpr int row_dir(int j) {
+  return j < 4 ? 3 + j : 11 + j;  // +y, -y, +z, -z, (y,z) diagonals 15..18
+}
+__host__ __device__ constexpr int row_of(int r) {  // row of direction r (r = 1, 2: the node's own)
+  for (int j = 0; j < 8; ++j)
+    if (D3Q19::cy(row_dir(j)) == D3Q19::cy(r) && D3Q19::cz(row_dir(j)) == D3Q19::cz(r)) return j;
+  return -1;
+}
+
 struct SparseView {
-  unsigned Nf;          // fluid nodes
-  void *pop;            // 19 x Nf storage elements, slot r of node i at r Nf + i
-  const int32_t *nbr;   // 18 x Nf: neighbour i + c_r at (r - 1) Nf + i, fluid index or -1 - wall id
-  const int32_t *dense; // Nf: dense node index of each fluid node
+  unsigned Nf;            // fluid nodes
+  void *pop;              // 19 x Nf storage elements, slot r of node i at r Nf + i
+  const uint32_t *word;   // Nf
+  const int32_t *seg0;    // first segment of each 32 nodes
+  const int4 *seg;        // 2 per segment: its eight b, or the table entry of an SP_TABLE node
+  const int32_t *table;   // ntable x 18: neighbour index or -1 - wall id
+  const int32_t *dense;   // Nf: dense node index of each fluid node
   float wall_vel[NWALL][3];
   float omega, rho0, g[3];
   int *status;
 };
 
+// what a lane knows of its node's neighbours (all 32 lanes call rows_of)
+struct SparseRows {
+  uint32_t w;
+  int b[8];           // b of each row; b[0] the table entry of an SP_TABLE node
+};
+
+__device__ __forceinline__ void rows_of(const SparseView &sv, unsigned i, uint32_t w, SparseRows &q) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  q.w = w;
+  const unsigned le = FULL >> (31 - lane);
+  const unsigned starts = __ballot_sync(FULL, w & SP_START) & le;
+  const int first = 31 - __clz(starts | 1u);
+  // (a warp past the last node has no start of its own: any segment will do)
+  const int s = max(sv.seg0[i >> 5] + __popc(starts) - 1, 0);
+  const int4 lo = sv.seg[2 * s], hi = sv.seg[2 * s + 1];
+  q.b[0] = lo.x;
+  q.b[1] = lo.y;
+  q.b[2] = lo.z;
+  q.b[3] = lo.w;
+  q.b[4] = hi.x;
+  q.b[5] = hi.y;
+  q.b[6] = hi.z;
+  q.b[7] = hi.w;
+  const unsigned before = (le >> 1) & (FULL << first);  // the lanes of this segment before this one
+  sfor<0, 8>([&](auto J) {
+    constexpr int j = decltype(J)::value;
+    const unsigned m = __ballot_sync(FULL, (w >> row_dir(j)) & 1u);
+    q.b[j] += __popc(m & before);
+  });
+}
+
+// indices of the open neighbours i + c_r (what stands at a closed direction is
+// not used).  One branch for the table nodes: a choice per direction cost the
+// odd step 36 branches, more than half its instructions.
+__device__ __forceinline__ void open_nbrs(const SparseView &sv, const SparseRows &q, unsigned i, unsigned (&nb)[Q]) {
+  sfor<1, Q>([&](auto R) {
+    constexpr int r = decltype(R)::value, j = row_of(r), dx = D3Q19::cx(r);
+    if constexpr (j < 0) nb[r] = i + (unsigned)dx;
+    else nb[r] = (unsigned)(q.b[j] + (dx < 0 ? -1 : (dx > 0 ? (int)((q.w >> row_dir(j)) & 1u) : 0)));
+  });
+  if (q.w & SP_TABLE) {
+    const int32_t *t = sv.table + 18 * (size_t)q.b[0];
+    sfor<1, Q>([&](auto R) { nb[decltype(R)::value] = (unsigned)t[decltype(R)::value - 1]; });
+  }
+}
+
+// wall id behind the closed direction R
+template <int R>
+__device__ __forceinline__ int wall_of(const SparseView &sv, const SparseRows &q) {
+  if (q.w & SP_TABLE) return -1 - sv.table[18 * (size_t)q.b[0] + (R - 1)];
+  return (int)(q.w >> SP_WALL) & 7;
+}
+
+// slot from which node i reads direction R in a step of parity par (nb: its
+// open neighbours where par = 1)
+template <int R>
+__device__ __forceinline__ unsigned sparse_src(const SparseView &sv, uint32_t w, int par, unsigned i,
+                                               const unsigned (&nb)[Q]) {
+  constexpr int rb = D3Q19::opp(R);
+  if (par == 0 || R == 0) return (unsigned)R * sv.Nf + i;
+  return (w >> rb) & 1u ? (unsigned)rb * sv.Nf + nb[rb] : (unsigned)R * sv.Nf + i;
+}
+
+// One fluid node per thread.  Bound: HBM, 2 x 19 populations and about 5 bytes
+// of words and segments per node; BL_SPARSE_MINB blocks of 128 threads keep
+// enough loads in flight.
 #ifndef BL_SPARSE_MINB
-#define BL_SPARSE_MINB 3
+#define BL_SPARSE_MINB 8
 #endif
 
 template <class S, int PAR, bool FORCE, bool TAU1>
-__global__ void __launch_bounds__(256, BL_SPARSE_MINB) k_sparse_step(SparseView sv, WallAcc wa) {
+__global__ void __launch_bounds__(128, BL_SPARSE_MINB) k_sparse_step(SparseView sv, WallAcc wa0) {
+  const WallAcc wa = wall_copy(wa0);
   using D = D3Q19;
   const unsigned Nf = sv.Nf;
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned i0 = blockIdx.x * 128u + threadIdx.x;
+  const bool valid = i0 < Nf;
+  const unsigned i = valid ? i0 : Nf - 1u;
   S *pop = reinterpret_cast<S *>(sv.pop);
   int wkey = -1;
   float wF[3] = {0.f, 0.f, 0.f};
   int wK[3] = {0, 0, 0};
-  if (i < Nf) {
-    // the neighbour table is read twice, here and for the writes (the second
-    // time from L1), so that its 18 entries do not stay live through the
-    // collision
+  SparseRows q;
+  q.w = valid ? sv.word[i] : 0u;
+  if constexpr (PAR == 1) {
+    rows_of(sv, i, q.w, q);
+  } else {
+    // in place: the segments are needed for a table node's walls alone
+    const unsigned starts = __ballot_sync(0xffffffffu, q.w & SP_START) & (0xffffffffu >> (31 - (threadIdx.x & 31)));
+    if (q.w & SP_TABLE) q.b[0] = sv.seg[2 * (sv.seg0[i >> 5] + __popc(starts) - 1)].x;
+  }
+  if (valid) {
     float f[Q];
-    f[0] = Store<S>::ld(pop + i);
-    sfor<1, Q>([&](auto R) {
-      constexpr int r = decltype(R)::value;
-      if constexpr (PAR == 0) {
-        f[r] = Store<S>::ld(pop + (size_t)r * Nf + i);
-      } else {
-        const int s = sv.nbr[(size_t)(D::opp(r) - 1) * Nf + i];  // the node i - c_r
-        f[r] = Store<S>::ld(pop + (s >= 0 ? (size_t)D::opp(r) * Nf + (unsigned)s : (size_t)r * Nf + i));
-      }
-    });
+    {
+      unsigned nb[Q];
+      if constexpr (PAR == 1) open_nbrs(sv, q, i, nb);
+      sfor<0, Q>([&](auto R) {
+        constexpr int r = decltype(R)::value;
+        f[r] = Store<S>::ld(pop + sparse_src<r>(sv, q.w, PAR, i, nb));
+      });
+    }
     // moments of the shifted populations: rho = rho_bar + sum f~, j = sum f~ c
     float drho = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
     sfor<0, 9>([&](auto P) {
@@ -101,59 +209,66 @@ __global__ void __launch_bounds__(256, BL_SPARSE_MINB) k_sparse_step(SparseView 
       f[rb] = relax_to<rb, TAU1>(f[rb], xb, om);
     });
     Store<S>::st(pop + i, f[0]);
+    const uint32_t closed = ~q.w & NB_SOLID;
+    if (closed) {
+      // links into walls: the population returns along rbar with the
+      // moving-wall term C (Eq. c), the wall receives (2 f*_r + C) c_r
+      sfor<1, Q>([&](auto R) {
+        constexpr int r = decltype(R)::value;
+        if ((closed >> r) & 1u) {
+          const int w = wall_of<r>(sv, q);
+          const float C = wall_term<r>(rho, sv.wall_vel[w]);
+          const float dp = 2.0f * f[r] + C;
+          if (wkey != w && wkey >= 0) {
+            for (int kk = 0; kk < 3; ++kk) {
+              atomicAdd(&wa.F[3 * wkey + kk], (double)wF[kk]);
+              atomicAdd((unsigned long long *)&wa.K[3 * wkey + kk], (unsigned long long)(long long)wK[kk]);
+              wF[kk] = 0.f;
+              wK[kk] = 0;
+            }
+          }
+          wkey = w;
+          wF[0] += dp * D::cx(r);
+          wF[1] += dp * D::cy(r);
+          wF[2] += dp * D::cz(r);
+          wK[0] += D::m(r) * D::cx(r);
+          wK[1] += D::m(r) * D::cy(r);
+          wK[2] += D::m(r) * D::cz(r);
+          f[r] += C;
+        }
+      });
+    }
+    unsigned nb[Q];  // (again: they do not stay live through the collision)
+    if constexpr (PAR == 1) open_nbrs(sv, q, i, nb);
     sfor<1, Q>([&](auto R) {
       constexpr int r = decltype(R)::value;
       constexpr int rb = D::opp(r);
-      const int t = sv.nbr[(size_t)(r - 1) * Nf + i];
-      float v = f[r];
-      if (t < 0) {
-        // a link into wall w: the population returns along rbar with the
-        // moving-wall term C (Eq. c), the wall receives (2 f*_r + C) c_r
-        const int w = -1 - t;
-        const float C = wall_term<r>(rho, sv.wall_vel[w]);
-        const float dp = 2.0f * f[r] + C;
-        if (wkey != w && wkey >= 0) {
-          for (int k = 0; k < 3; ++k) {
-            atomicAdd(&wa.F[3 * wkey + k], (double)wF[k]);
-            atomicAdd((unsigned long long *)&wa.K[3 * wkey + k], (unsigned long long)(long long)wK[k]);
-            wF[k] = 0.f;
-            wK[k] = 0;
-          }
-        }
-        wkey = w;
-        wF[0] += dp * D::cx(r);
-        wF[1] += dp * D::cy(r);
-        wF[2] += dp * D::cz(r);
-        wK[0] += D::m(r) * D::cx(r);
-        wK[1] += D::m(r) * D::cy(r);
-        wK[2] += D::m(r) * D::cz(r);
-        v += C;
-      }
-      const size_t dst = (t >= 0 && PAR == 1) ? (size_t)r * Nf + (unsigned)t : (size_t)rb * Nf + i;
-      Store<S>::st(pop + dst, v);
+      unsigned dst = (unsigned)rb * Nf + i;
+      if constexpr (PAR == 1)
+        if ((q.w >> r) & 1u) dst = (unsigned)r * Nf + nb[r];
+      Store<S>::st(pop + dst, f[r]);
     });
   }
   flush_wall_momentum(wa, wkey, wF, wK);
-}
-
-// slot from which fluid node i reads direction r in a step of parity par
-__device__ __forceinline__ size_t sparse_src(const SparseView &sv, int par, unsigned i, int r) {
-  if (par == 0 || r == 0) return (size_t)r * sv.Nf + i;
-  const int s = sv.nbr[(size_t)(D3Q19::opp(r) - 1) * sv.Nf + i];
-  return s >= 0 ? (size_t)D3Q19::opp(r) * sv.Nf + (unsigned)s : (size_t)r * sv.Nf + i;
 }
 
 // moments on the dense grid (zero at walls): rho and u = j / rho + g / 2
 template <class S>
 __global__ void __launch_bounds__(256) k_sparse_fields(SparseView sv, int par, double rho0, double hg0, double hg1,
                                                        double hg2, double *rho, double *u) {
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sv.Nf) return;
+  const unsigned i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = i0 < sv.Nf;
+  const unsigned i = valid ? i0 : sv.Nf - 1u;
   const S *pop = reinterpret_cast<const S *>(sv.pop);
+  SparseRows q;
+  rows_of(sv, i, valid ? sv.word[i] : 0u, q);
+  if (!valid) return;
   float f[Q];
+  unsigned nb[Q];
+  open_nbrs(sv, q, i, nb);
   sfor<0, Q>([&](auto R) {
     constexpr int r = decltype(R)::value;
-    f[r] = Store<S>::ld(pop + sparse_src(sv, par, i, r));
+    f[r] = Store<S>::ld(pop + sparse_src<r>(sv, q.w, par, i, nb));
   });
   const double hg[3] = {hg0, hg1, hg2};
   double rh, uu[3];
@@ -167,16 +282,23 @@ __global__ void __launch_bounds__(256) k_sparse_fields(SparseView sv, int par, d
 // populations n_r (unshifted) on the dense grid, N x 19, to (0) or from (1) storage
 template <class S>
 __global__ void k_sparse_pop_io(SparseView sv, int par, double *buf, int to_storage) {
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sv.Nf) return;
+  const unsigned i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = i0 < sv.Nf;
+  const unsigned i = valid ? i0 : sv.Nf - 1u;
   S *pop = reinterpret_cast<S *>(sv.pop);
+  SparseRows q;
+  rows_of(sv, i, valid ? sv.word[i] : 0u, q);
+  if (!valid) return;
   const size_t n = (size_t)sv.dense[i];
-  for (int r = 0; r < Q; ++r) {
+  unsigned nb[Q];
+  open_nbrs(sv, q, i, nb);
+  sfor<0, Q>([&](auto R) {
+    constexpr int r = decltype(R)::value;
     const double shift = (double)sv.rho0 * D3Q19::m(r) / 36.0;
-    const size_t s = sparse_src(sv, par, i, r);
+    const unsigned s = sparse_src<r>(sv, q.w, par, i, nb);
     if (to_storage) Store<S>::st(pop + s, (float)(buf[n * Q + r] - shift));
     else buf[n * Q + r] = (double)Store<S>::ld(pop + s) + shift;
-  }
+  });
 }
 
 template <class S>
@@ -189,7 +311,7 @@ __global__ void k_sparse_rest(SparseView sv) {
 
 template <class S>
 void launch_sparse_typed(const SparseView &sv, int par, bool force, bool tau1, const WallAcc &wa, cudaStream_t st) {
-  const unsigned b = 256, g = nblk(sv.Nf, b);
+  const unsigned b = 128, g = nblk(sv.Nf, b);
 #define BL_SP(P_, F_, T_) k_sparse_step<S, P_, F_, T_><<<g, b, 0, st>>>(sv, wa)
   if (par == 0) {
     if (force) { if (tau1) BL_SP(0, true, true); else BL_SP(0, true, false); }
@@ -299,6 +421,94 @@ extern "C" int bl_sparse_index_build(const bl_lb_params *p, const uint8_t *mask,
   return BL_OK;
 }
 
+// words, segments and the explicit table of an index (see the head of this
+// file).  A node is a table node where its row wraps (an end of a periodic row)
+// or where its walls have different ids; the segments of the others are then
+// checked against the neighbour table, and a node they do not reproduce becomes
+// a table node too.
+struct RowIndex {
+  std::vector<uint32_t> word;
+  std::vector<int32_t> seg0, seg, table;
+};
+
+static void build_rows(int nx, bool per_x, const std::vector<int32_t> &dense, const std::vector<int32_t> &nbr,
+                       RowIndex &out) {
+  const size_t nf = dense.size();
+  out.word.assign(nf, 0u);
+  for (int r = 1; r < Q; ++r) {
+    const int32_t *nb = nbr.data() + (size_t)(r - 1) * nf;
+    for (size_t i = 0; i < nf; ++i) {
+      uint32_t &w = out.word[i];
+      if (nb[i] >= 0) {
+        w |= 1u << r;
+      } else {
+        const uint32_t id = (uint32_t)(-1 - nb[i]);
+        if (!(w & (1u << 19))) w |= (1u << 19) | (id << SP_WALL);  // bit 19: a wall id is noted (cleared below)
+        else if (((w >> SP_WALL) & 7u) != id) w |= SP_TABLE;
+      }
+    }
+  }
+  for (size_t i = 0; i < nf; ++i) {
+    const int x = dense[i] % nx;
+    if (per_x && (x == 0 || x == nx - 1)) out.word[i] |= SP_TABLE;
+    out.word[i] &= ~(1u << 19);
+  }
+  for (bool again = true; again;) {
+    again = false;
+    out.seg0.assign((nf + 31) / 32, 0);
+    out.seg.clear();
+    out.table.clear();
+    for (size_t i = 0; i < nf;) {
+      if (i % 32 == 0) out.seg0[i / 32] = (int32_t)(out.seg.size() / 8);
+      size_t e = i + 1;  // end of the segment
+      const bool tab = out.word[i] & SP_TABLE;
+      while (!tab && e < nf && e % 32 != 0 && dense[e] == dense[e - 1] + 1 && dense[e] % nx != 0 &&
+             !(out.word[e] & SP_TABLE))
+        ++e;
+      int32_t b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      if (tab) {
+        b[0] = (int32_t)(out.table.size() / 18);
+        for (int r = 1; r < Q; ++r) out.table.push_back(nbr[(size_t)(r - 1) * nf + i]);
+      } else {
+        auto at = [&](int r, size_t k) { return nbr[(size_t)(r - 1) * nf + k]; };
+        for (int j = 0; j < 8; ++j) {
+          // the first node of the segment with a fluid neighbour in row j gives b
+          const int r0 = row_dir(j);
+          int rp = 0, rm = 0;
+          for (int r = 7; r < 15; ++r)
+            if (row_of(r) == j) (D3Q19::cx(r) > 0 ? rp : rm) = r;
+          for (size_t k = i; k < e; ++k) {
+            if (at(r0, k) >= 0) b[j] = at(r0, k);
+            else if (rp && at(rp, k) >= 0) b[j] = at(rp, k);
+            else if (rm && at(rm, k) >= 0) b[j] = at(rm, k) + 1;
+            else continue;
+            break;
+          }
+          int32_t bb = b[j];
+          for (size_t k = i; k < e; ++k) {
+            const bool mid = at(r0, k) >= 0;
+            if ((mid && at(r0, k) != bb) || (rp && at(rp, k) >= 0 && at(rp, k) != bb + (mid ? 1 : 0)) ||
+                (rm && at(rm, k) >= 0 && at(rm, k) != bb - 1)) {
+              out.word[k] |= SP_TABLE;
+              again = true;
+            }
+            bb += mid ? 1 : 0;
+          }
+        }
+        for (size_t k = i; k < e; ++k)
+          if ((at(1, k) >= 0 && at(1, k) != (int32_t)k + 1) || (at(2, k) >= 0 && at(2, k) != (int32_t)k - 1)) {
+            out.word[k] |= SP_TABLE;
+            again = true;
+          }
+      }
+      out.word[i] |= SP_START;
+      for (size_t k = i + 1; k < e; ++k) out.word[k] &= ~SP_START;
+      out.seg.insert(out.seg.end(), b, b + 8);
+      i = e;
+    }
+  }
+}
+
 extern "C" void bl_sparse_destroy(bl_sparse *s) {
   if (!s) return;
   if (s->stream) cudaStreamSynchronize(s->stream);
@@ -306,7 +516,8 @@ extern "C" void bl_sparse_destroy(bl_sparse *s) {
   if (s->gstream) cudaStreamDestroy(s->gstream);
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
   if (s->ev_join) cudaEventDestroy(s->ev_join);
-  void *ptrs[] = {s->sv.pop, (void *)s->sv.nbr, (void *)s->sv.dense, s->sv.status, s->wa.F, s->wa.K, s->scratch};
+  void *ptrs[] = {s->sv.pop, (void *)s->sv.word, (void *)s->sv.seg0, (void *)s->sv.seg, (void *)s->sv.table,
+                  (void *)s->sv.dense, s->sv.status, s->wa.F, s->wa.K, s->scratch};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   delete s;
@@ -339,6 +550,8 @@ extern "C" int bl_sparse_init(bl_sparse **out, const bl_lb_params *p, const uint
   std::vector<int32_t> dense((size_t)nf), nbr((size_t)nf * 18);
   rc = bl_sparse_index_build(p, mask, &nf, dense.data(), nbr.data());
   if (rc != BL_OK) return rc;
+  RowIndex rows;
+  build_rows(p->nx, p->periodic[0] != 0, dense, nbr, rows);
   bl_sparse *s = new bl_sparse();
   s->lp = *p;
   s->stream = (cudaStream_t)cuda_stream;
@@ -352,32 +565,34 @@ extern "C" int bl_sparse_init(bl_sparse **out, const bl_lb_params *p, const uint
   sv.rho0 = (float)p->rho0;
   for (int k = 0; k < 3; ++k) sv.g[k] = (float)p->g[k];
   do {
-    void *pop = nullptr, *nb = nullptr, *dn = nullptr;
-    if (cudaMalloc(&pop, sp_elem(p->store_dtype) * Q * (size_t)nf) != cudaSuccess ||
-        cudaMalloc(&nb, sizeof(int32_t) * 18 * (size_t)nf) != cudaSuccess ||
-        cudaMalloc(&dn, sizeof(int32_t) * (size_t)nf) != cudaSuccess || cudaMalloc(&sv.status, sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&s->wa.F, sizeof(double) * NWALL * 3) != cudaSuccess ||
-        cudaMalloc(&s->wa.K, sizeof(long long) * NWALL * 3) != cudaSuccess) {
-      sv.pop = pop;
-      sv.nbr = (const int32_t *)nb;
-      sv.dense = (const int32_t *)dn;
+    // every array is handed to the context as it is made, so that destroy frees it
+    auto put = [&](auto *&dst, const void *src, size_t bytes) {
+      void *q = nullptr;
+      if (cudaMalloc(&q, bytes > 0 ? bytes : 1) != cudaSuccess) return false;
+      dst = static_cast<std::remove_reference_t<decltype(dst)>>(q);
+      return !src || bytes == 0 ||
+             cudaMemcpyAsync(q, src, bytes, cudaMemcpyHostToDevice, s->stream) == cudaSuccess;
+    };
+    if (!put(sv.pop, nullptr, sp_elem(p->store_dtype) * Q * (size_t)nf) ||
+        !put(sv.word, rows.word.data(), sizeof(uint32_t) * rows.word.size()) ||
+        !put(sv.seg0, rows.seg0.data(), sizeof(int32_t) * rows.seg0.size()) ||
+        !put(sv.seg, rows.seg.data(), sizeof(int32_t) * rows.seg.size()) ||
+        !put(sv.table, rows.table.data(), sizeof(int32_t) * rows.table.size()) ||
+        !put(sv.dense, dense.data(), sizeof(int32_t) * (size_t)nf) || !put(sv.status, nullptr, sizeof(int)) ||
+        !put(s->wa.F, nullptr, sizeof(double) * WALL_COPIES * WALL_SUMS) ||
+        !put(s->wa.K, nullptr, sizeof(long long) * WALL_COPIES * WALL_SUMS)) {
       rc = sp_fail(s, BL_ENOMEM, "indexed lattice");
       break;
     }
-    sv.pop = pop;
-    sv.nbr = (const int32_t *)nb;
-    sv.dense = (const int32_t *)dn;
     if (cudaStreamCreateWithFlags(&s->gstream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess) {
       rc = sp_fail(s, BL_ECUDA, "streams");
       break;
     }
-    if (cudaMemcpyAsync(nb, nbr.data(), sizeof(int32_t) * nbr.size(), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
-        cudaMemcpyAsync(dn, dense.data(), sizeof(int32_t) * dense.size(), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
-        cudaMemsetAsync(sv.status, 0, sizeof(int), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->wa.F, 0, sizeof(double) * NWALL * 3, s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->wa.K, 0, sizeof(long long) * NWALL * 3, s->stream) != cudaSuccess) {
+    if (cudaMemsetAsync(sv.status, 0, sizeof(int), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->wa.F, 0, sizeof(double) * WALL_COPIES * WALL_SUMS, s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->wa.K, 0, sizeof(long long) * WALL_COPIES * WALL_SUMS, s->stream) != cudaSuccess) {
       rc = sp_fail(s, BL_ECUDA, "upload");
       break;
     }
@@ -514,14 +729,14 @@ extern "C" int bl_sparse_populations_set(bl_sparse *s, const double *pop) {
 extern "C" int bl_sparse_wall_momentum_get(bl_sparse *s, double *wallmom) {
   if (!s || !wallmom) return BL_EINVAL;
   if (s->sticky) return s->sticky;
-  double F[NWALL * 3];
-  long long K[NWALL * 3];
+  double F[WALL_COPIES * WALL_SUMS];
+  long long K[WALL_COPIES * WALL_SUMS];
   SPCU(cudaMemcpyAsync(F, s->wa.F, sizeof(F), cudaMemcpyDeviceToHost, s->stream));
   SPCU(cudaMemcpyAsync(K, s->wa.K, sizeof(K), cudaMemcpyDeviceToHost, s->stream));
   SPCU(cudaStreamSynchronize(s->stream));
   SPCU(cudaMemsetAsync(s->wa.F, 0, sizeof(F), s->stream));
   SPCU(cudaMemsetAsync(s->wa.K, 0, sizeof(K), s->stream));
-  for (int i = 0; i < NWALL * 3; ++i) wallmom[i] = F[i] + s->lp.rho0 / 18.0 * (double)K[i];
+  wall_total(F, K, s->lp.rho0, wallmom);
   return BL_OK;
 }
 

@@ -426,7 +426,8 @@ __device__ __forceinline__ void node_update(const LatticeView &lv, const WallAcc
 // that rows of any length fill the warps: with a block per row segment, 150
 // nodes left 41 % of the threads without a node, 48 nodes 25 %.
 template <class S, int PAR, bool FORCE, bool TAU1, bool CELLS>
-__global__ void __launch_bounds__(128, TAU1 || !CELLS ? BL_ONE_MINB : BL_ONE_MINB_BGK) k_lb_step(LatticeView lv, WallAcc wa) {
+__global__ void __launch_bounds__(128, TAU1 || !CELLS ? BL_ONE_MINB : BL_ONE_MINB_BGK) k_lb_step(LatticeView lv, WallAcc wa0) {
+  const WallAcc wa = wall_copy(wa0);
   const int nx = lv.nx, ny = lv.ny;
   const unsigned nxy = lv.dnxy.d;
   const unsigned i0 = blockIdx.x * 128u + threadIdx.x;
@@ -498,7 +499,8 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 template <int PAR, bool FORCE, bool TAU1, int ZC>
-__global__ void __launch_bounds__(128, BL_LB_MINB) k_lb_step_pipe(LatticeView lv, WallAcc wa) {
+__global__ void __launch_bounds__(128, BL_LB_MINB) k_lb_step_pipe(LatticeView lv, WallAcc wa0) {
+  const WallAcc wa = wall_copy(wa0);
   __shared__ float stage[PIPE_ST][Q][128];
   const int nx = lv.nx, ny = lv.ny, nz = lv.nz;
   const int tx = threadIdx.x;
@@ -610,7 +612,8 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
 }
 
 template <class S, int PAR, bool FORCE, bool TAU1, bool CELLS, int ZC, int TS>
-__global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView lv, WallAcc wa) {
+__global__ void __launch_bounds__(128, BL_BULK_MINB) k_lb_step_bulk(LatticeView lv, WallAcc wa0) {
+  const WallAcc wa = wall_copy(wa0);
   using D = D3Q19;
   __shared__ alignas(128) S sb[TS][Q][128];        // [stage][array][x]
   __shared__ alignas(128) uint32_t sw[TS][128];    // [stage][x] neighbour words
@@ -768,7 +771,8 @@ __device__ __forceinline__ void write_staged(const LatticeView &lv, int p, unsig
 }
 
 template <class S, int PAR, bool FORCE, bool TAU1, int TS>
-__global__ void __launch_bounds__(128, BL_ROWS_MINB) k_lb_step_rows(LatticeView lv, WallAcc wa) {
+__global__ void __launch_bounds__(128, BL_ROWS_MINB) k_lb_step_rows(LatticeView lv, WallAcc wa0) {
+  const WallAcc wa = wall_copy(wa0);
   using D = D3Q19;
   __shared__ alignas(128) S sb[TS][Q][128];      // [stage][array][x]
   __shared__ alignas(128) uint32_t sw[TS][128];  // [stage][x] neighbour words
