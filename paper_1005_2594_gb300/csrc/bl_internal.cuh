@@ -202,6 +202,7 @@ struct PartView {
   double *X, *q, *V, *L, *Om;
   double *o;         // exact FP64 symmetry axis of the current q, n x 3
   float4 *axis;      // n: the current axis in FP32
+  float4 *qf;        // n: the current quaternion in FP32
   float *oprev;      // n x 3 axis before the last move (FP32): the claims' old ellipsoid
   float4 *kin;       // kinematics of the current step, 3 float4 per cell:
                      //   (f.x, f.y, f.z, Xi.x), (V, Xi.y), (W, Xi.z); X = Xi + f, Xi = rint(X)
@@ -311,9 +312,12 @@ void launch_clear_cells(int dtype, const LatticeView &lv, int par, cudaStream_t 
 
 void launch_pair_features(const LatticeView &lv, const PartView &pv, const int2 *pairs, int n, float *out,
                           cudaStream_t st);
-void launch_mlp_correction(const LatticeView &lv, const PartView &pv, const CellListView &cl, const PairBuf &pb,
-                           float gap_lo, float gap_cut, float speed_lo, float speed_hi, const void *mlp,
-                           cudaStream_t st, int64_t *nl);
+// the learned correction: the close pairs with their features and the network
+// over them (after the cell list), then its forces (after the potentials)
+void launch_mlp_pairs(const LatticeView &lv, const PartView &pv, const CellListView &cl, const PairBuf &pb,
+                      float gap_lo, float gap_cut, float speed_lo, float speed_hi, const void *mlp, cudaStream_t st,
+                      int64_t *nl);
+void launch_mlp_apply(const PartView &pv, const PairBuf &pb, cudaStream_t st, int64_t *nl);
 // forward pass of a bl_mlp over *count rows of x (at most cap), raw units
 void launch_mlp_forward_dev(const void *mlp, const float *x, const int *count, int cap, float *y, cudaStream_t st);
 // the Lees-Edwards passes after a sweep of parity par

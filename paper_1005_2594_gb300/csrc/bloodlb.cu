@@ -43,7 +43,8 @@ struct bl_ctx {
   cudaEvent_t ev_fork, ev_join;     // cell list and potentials beside the sweep
   cudaEvent_t ev_fork2, ev_join2;   // claims beside the pending terms
   cudaStream_t side2;
-  cudaEvent_t ev_join3;             // contact sums beside the sweep (second side stream)
+  cudaEvent_t ev_join3;             // contact sums (and the network) beside the sweep (second side stream)
+  cudaEvent_t ev_list;              // cell list built: the network's pairs may start
   // repeated steps replay a CUDA graph of two steps (even + odd parity), a
   // lone step a one-step graph, on an internal stream forked from and joined
   // to the caller's stream
@@ -290,7 +291,8 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
         cudaEventCreateWithFlags(&c->ev_fork2, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithPriority(&c->side2, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_join3, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&c->ev_join3, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_list, cudaEventDisableTiming) != cudaSuccess) {
       rc = fail(c, BL_ECUDA, "streams");
       break;
     }
@@ -347,7 +349,7 @@ extern "C" int bl_walls_set(bl_ctx *c, const uint8_t *mask) {
 
 static void free_particles(bl_ctx *c) {
   PartView &pv = c->pv;
-  void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.axis, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
+  void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.axis, pv.qf, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
                   pv.touched, pv.touched_count, pv.lsum, pv.lsum_f, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink, pv.Ftot,
                   pv.Ttot, pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
                   c->chg.count, c->chg.items, c->lv.rec, c->lv.rec_count};
@@ -379,6 +381,8 @@ static int alloc_particles(bl_ctx *c, int n) {
   }
   CU(cudaMalloc(&pv.axis, sizeof(float4) * (size_t)n));
   CU(cudaMemsetAsync(pv.axis, 0, sizeof(float4) * (size_t)n, c->stream));
+  CU(cudaMalloc(&pv.qf, sizeof(float4) * (size_t)n));
+  CU(cudaMemsetAsync(pv.qf, 0, sizeof(float4) * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.oprev, sizeof(float) * 3 * (size_t)n));
   CU(cudaMemsetAsync(pv.oprev, 0, sizeof(float) * 3 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.q, sizeof(double) * 4 * (size_t)n));
@@ -626,11 +630,23 @@ static int enqueue_step(bl_ctx *c, cudaStream_t st) {
     group_begin(c, 1, &slot, c->side);
     launch_cell_list(c->lv, c->pv, c->cl, c->side, &c->launches);
     group_end(c, slot, c->side);
+    if (c->mlp) {
+      // the network's pairs and forward pass need the list alone: beside the
+      // potentials, after the contact sums; its forces are added after both
+      cudaEventRecord(c->ev_list, c->side);
+      cudaStreamWaitEvent(c->side2, c->ev_list, 0);
+      group_begin(c, 2, &slot, c->side2);
+      launch_mlp_pairs(c->lv, c->pv, c->cl, c->pb, c->gap_lo, c->gap_cut, c->speed_lo, c->speed_hi, c->mlp, c->side2,
+                       &c->launches);
+      group_end(c, slot, c->side2);
+      cudaEventRecord(c->ev_join3, c->side2);
+    }
     group_begin(c, 2, &slot, c->side);
     launch_forces(c->lv, c->pv, c->cl, c->sbits, c->side, &c->launches);
-    if (c->mlp)
-      launch_mlp_correction(c->lv, c->pv, c->cl, c->pb, c->gap_lo, c->gap_cut, c->speed_lo, c->speed_hi, c->mlp,
-                            c->side, &c->launches);
+    if (c->mlp) {
+      cudaStreamWaitEvent(c->side, c->ev_join3, 0);
+      launch_mlp_apply(c->pv, c->pb, c->side, &c->launches);
+    }
     group_end(c, slot, c->side);
     cudaEventRecord(c->ev_join, c->side);
   }
@@ -1309,7 +1325,7 @@ extern "C" void bl_destroy(bl_ctx *c) {
   if (c->gstream) cudaStreamDestroy(c->gstream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
-  for (cudaEvent_t e : {c->ev_fork2, c->ev_join2, c->ev_join3})
+  for (cudaEvent_t e : {c->ev_fork2, c->ev_join2, c->ev_join3, c->ev_list})
     if (e) cudaEventDestroy(e);
   if (c->side2) cudaStreamDestroy(c->side2);
   free_particles(c);

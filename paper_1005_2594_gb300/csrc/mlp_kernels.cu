@@ -175,6 +175,7 @@ static_assert(P_W2T % 8 == 0 && P_TOTAL % 8 == 0, "operand copies in 16-byte wor
 __global__ void __launch_bounds__(128) k_mlp_forward(MlpDev m, const float *x, int B, const int *Bdev, float *y) {
   __shared__ __align__(16) __nv_bfloat16 wp[P_TOTAL];
   if (Bdev) B = min(*Bdev, B);
+  if ((int)blockIdx.x * 64 >= B) return;
   load_operands(wp, m.wp, P_W2T);
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;

@@ -1,6 +1,7 @@
 // particle_kernels.cu -- the cell side of the coupled step (arXiv:1005.2594):
 //
-//   cell list      count -> scan -> scatter -> per-bin sort, canonical (bin, id)
+//   cell list      count -> scan -> scatter -> per-bin sort, canonical (bin, id);
+//                  in one block for up to 16384 cells and bins
 //   potentials     Berne-Pechukas-scaled Hookean cell-cell pairs (Sec. III,
 //                  Eqs. phi, epsilon, sigma) and cell-wall spheres (Eq. sigmaw),
 //                  one block per cell, FP64 contact geometry, FP32 forces,
@@ -36,6 +37,7 @@
 // rotation increment are FP32 around FP64 reference values, and the kernels
 // that test nodes against ellipsoids read each cell's position (node + FP32
 // fraction) and axis in the FP32 form the solve leaves them.
+#include <atomic>
 #include <climits>
 
 #include "bl_internal.cuh"
@@ -52,17 +54,102 @@ constexpr float INSIDE_MARGIN = 1e-4f;
 // ---------------------------------------------------------------------------
 // cell list
 
+// bin of a coordinate, floor((X / N) nb) with X / N and the product rounded to
+// FP64 as the plain reference does: from FP32, whose error is below 4e-7 nb,
+// unless the bin's border is that near
+__device__ __forceinline__ int axis_bin(double X, int dim, int nb) {
+  const float t = (float)X * ((float)nb / (float)dim);
+  int b;
+  if (fabsf(t - rintf(t)) > 1e-6f * (float)nb + 1e-5f) b = (int)floorf(t);
+  else b = (int)floor(__dmul_rn(__ddiv_rn(X, (double)dim), (double)nb));
+  return min(max(b, 0), nb - 1);
+}
+
+__device__ __forceinline__ int cell_bin(const LatticeView &lv, const PartView &pv, const CellListView &cl, int i) {
+  const int b0 = axis_bin(pv.X[3 * i], lv.nx, cl.nb[0]), b1 = axis_bin(pv.X[3 * i + 1], lv.ny, cl.nb[1]),
+            b2 = axis_bin(pv.X[3 * i + 2], lv.nz, cl.nb[2]);
+  return b0 + cl.nb[0] * (b1 + cl.nb[1] * b2);
+}
+
+// The whole list in one block of 1024 threads, counts, starts and ids in shared
+// memory: for up to CL_ONE cells and bins the four kernels below were four
+// launches of 3 to 4 us each on the way to the potentials, the longest way
+// through the step of a small lattice.  Larger lists take the four kernels.
+constexpr int CL_ONE = 16384, CL_PER = CL_ONE / 1024;
+
+__global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, CellListView cl) {
+  extern __shared__ int cl_smem[];
+  int *cnt = cl_smem, *ids = cl_smem + cl.nbins;
+  __shared__ int wsum[32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  for (int b = t; b < cl.nbins; b += 1024) cnt[b] = 0;
+  __syncthreads();
+  int bin[CL_PER], slot[CL_PER];
+#pragma unroll
+  for (int u = 0; u < CL_PER; ++u) {
+    const int i = t + 1024 * u;
+    if (i < pv.n) {
+      bin[u] = cell_bin(lv, pv, cl, i);
+      cl.bin_of[i] = bin[u];
+      slot[u] = atomicAdd(&cnt[bin[u]], 1);
+    }
+  }
+  __syncthreads();
+  // exclusive scan: a run of bins per thread, the runs' sums over the block
+  const int per = (cl.nbins + 1023) / 1024, b0 = min(t * per, cl.nbins), b1 = min(b0 + per, cl.nbins);
+  int sum = 0;
+  for (int b = b0; b < b1; ++b) sum += cnt[b];
+  int inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) wsum[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    int w = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += v;
+    }
+    wsum[lane] = w;
+  }
+  __syncthreads();
+  int off = (wid > 0 ? wsum[wid - 1] : 0) + inc - sum;
+  for (int b = b0; b < b1; ++b) {
+    const int c = cnt[b];
+    cnt[b] = off;
+    cl.start[b] = off;
+    off += c;
+  }
+  if (t == 0) cl.start[cl.nbins] = pv.n;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < CL_PER; ++u)
+    if (t + 1024 * u < pv.n) ids[cnt[bin[u]] + slot[u]] = t + 1024 * u;
+  __syncthreads();
+  for (int b = t; b < cl.nbins; b += 1024) {
+    const int s = cnt[b], e = b + 1 < cl.nbins ? cnt[b + 1] : pv.n;
+    for (int i = s + 1; i < e; ++i) {
+      const int v = ids[i];
+      int j = i - 1;
+      while (j >= s && ids[j] > v) {
+        ids[j + 1] = ids[j];
+        --j;
+      }
+      ids[j + 1] = v;
+    }
+  }
+  __syncthreads();
+  for (int i = t; i < pv.n; i += 1024) cl.ids[i] = ids[i];
+}
+
 __global__ void k_cl_bin(LatticeView lv, PartView pv, CellListView cl) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= pv.n) return;
-  const int dims[3] = {lv.nx, lv.ny, lv.nz};
-  int b[3];
-  for (int k = 0; k < 3; ++k) {
-    b[k] = (int)floor(__dmul_rn(__ddiv_rn(pv.X[3 * i + k], (double)dims[k]), (double)cl.nb[k]));
-    if (b[k] < 0) b[k] = 0;
-    if (b[k] > cl.nb[k] - 1) b[k] = cl.nb[k] - 1;
-  }
-  const int bin = b[0] + cl.nb[0] * (b[1] + cl.nb[1] * b[2]);
+  const int bin = cell_bin(lv, pv, cl, i);
   cl.bin_of[i] = bin;
   atomicAdd(&cl.count[bin], 1);
 }
@@ -560,8 +647,8 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
 // ---------------------------------------------------------------------------
 // rigid-body helpers
 
-__device__ void rotmat_f(const double q[4], float R[3][3]) {
-  const float w = (float)q[0], x = (float)q[1], y = (float)q[2], z = (float)q[3];
+__device__ void rotmat_f(const float4 &q, float R[3][3]) {
+  const float w = q.x, x = q.y, y = q.z, z = q.w;
   R[0][0] = 1 - 2 * (y * y + z * z); R[0][1] = 2 * (x * y - w * z);     R[0][2] = 2 * (x * z + w * y);
   R[1][0] = 2 * (x * y + w * z);     R[1][1] = 1 - 2 * (x * x + z * z); R[1][2] = 2 * (y * z - w * x);
   R[2][0] = 2 * (x * z - w * y);     R[2][1] = 2 * (y * z + w * x);     R[2][2] = 1 - 2 * (x * x + y * y);
@@ -570,7 +657,7 @@ __device__ void rotmat_f(const double q[4], float R[3][3]) {
 // I_lab = R diag(I_perp, I_perp, I_par) R^T and its inverse (FP32)
 __device__ void inertia_f(const PartView &pv, const double q[4], float I[3][3], float Iinv[3][3]) {
   float R[3][3];
-  rotmat_f(q, R);
+  rotmat_f(make_float4((float)q[0], (float)q[1], (float)q[2], (float)q[3]), R);
   const float d[3] = {(float)pv.Iperp, (float)pv.Iperp, (float)pv.Ipar};
   const float di[3] = {1.0f / d[0], 1.0f / d[1], 1.0f / d[2]};
   for (int a = 0; a < 3; ++a)
@@ -1045,7 +1132,10 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
     } else if (valid) {
       atomicOr(pv.status, ST_UNSTABLE);
     }
-    if (valid) pv.q[4 * p + k4] = q;
+    if (valid) {
+      pv.q[4 * p + k4] = q;
+      reinterpret_cast<float *>(pv.qf + p)[k4] = (float)q;
+    }
     if (wr) {
       pv.X[c] = X;
       pv.V[c] = V;
@@ -1221,6 +1311,7 @@ __global__ void k_set_state(LatticeView lv, PartView pv, int mode) {
     pv.vw[6 * p + 3 + k] = (float)W[k];
   }
   for (int k = 0; k < 4; ++k) pv.q[4 * p + k] = q[k];
+  pv.qf[p] = make_float4((float)q[0], (float)q[1], (float)q[2], (float)q[3]);
   double o_new[3];
   axis_exact(q, o_new);
   for (int k = 0; k < 3; ++k) {
@@ -1946,7 +2037,7 @@ __device__ void pair_features(const LatticeView &lv, const PartView &pv, int i, 
   const float af[3] = {a0.x, a0.y, a0.z}, bf[3] = {b0.x, b0.y, b0.z};
   float r[3];
   for (int k = 0; k < 3; ++k) r[k] = (float)imin_image(bi[k] - ai[k], dims[k], lv.per[k]) + (bf[k] - af[k]);
-  const double *qi = pv.q + 4 * i, *qj = pv.q + 4 * j;
+  const float4 qi = pv.qf[i], qj = pv.qf[j];
   rotmat_f(qi, R);
   float Rj[3][3];
   rotmat_f(qj, Rj);
@@ -1964,8 +2055,8 @@ __device__ void pair_features(const LatticeView &lv, const PartView &pv, int i, 
     f[8 + k] = R[0][k] * dv[0] + R[1][k] * dv[1] + R[2][k] * dv[2];
     f[11 + k] = R[0][k] * dw[0] + R[1][k] * dw[1] + R[2][k] * dw[2];
   }
-  const float w1 = (float)qi[0], x1 = -(float)qi[1], y1 = -(float)qi[2], z1 = -(float)qi[3];
-  const float w2 = (float)qj[0], x2 = (float)qj[1], y2 = (float)qj[2], z2 = (float)qj[3];
+  const float w1 = qi.x, x1 = -qi.y, y1 = -qi.z, z1 = -qi.w;
+  const float w2 = qj.x, x2 = qj.y, y2 = qj.z, z2 = qj.w;
   float qr[4] = {w1 * w2 - x1 * x2 - y1 * y2 - z1 * z2, w1 * x2 + x1 * w2 + y1 * z2 - z1 * y2,
                  w1 * y2 - x1 * z2 + y1 * w2 + z1 * x2, w1 * z2 + x1 * y2 - y1 * x2 + z1 * w2};
   const float sgn = qr[0] < 0.f ? -1.f : 1.f;
@@ -2033,7 +2124,7 @@ __global__ void k_mlp_apply(PartView pv, PairBuf pb) {
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
     const int i = pb.pairs[s].x;
     float R[3][3];
-    rotmat_f(pv.q + 4 * i, R);
+    rotmat_f(pv.qf[i], R);
     const float *y = pb.out + 6 * s;
     for (int k = 0; k < 3; ++k) {
       atomicAdd(&pv.Fpot[3 * i + k], (double)(R[k][0] * y[0] + R[k][1] * y[1] + R[k][2] * y[2]));
@@ -2047,8 +2138,32 @@ __global__ void k_mlp_apply(PartView pv, PairBuf pb) {
 
 static inline unsigned nblk(unsigned n, unsigned b) { return (n + b - 1) / b; }
 
+// the one-block list's shared memory (up to 128 KB) has to be asked for once
+// per device
+static bool cl_one_ready() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  static std::atomic<int> state[64];  // 0 not asked, 1 granted, 2 refused
+  int s = state[dev].load(std::memory_order_acquire);
+  if (s == 0) {
+    s = cudaFuncSetAttribute(k_cl_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * CL_ONE * sizeof(int))) ==
+                cudaSuccess
+            ? 1
+            : 2;
+    if (s == 2) cudaGetLastError();
+    state[dev].store(s, std::memory_order_release);
+  }
+  return s == 1;
+}
+
 void launch_cell_list(const LatticeView &lv, const PartView &pv, const CellListView &cl, cudaStream_t st, int64_t *nl) {
   if (pv.n == 0) return;
+  const size_t smem = sizeof(int) * ((size_t)cl.nbins + (size_t)pv.n);
+  if (pv.n <= CL_ONE && cl.nbins <= CL_ONE && cl_one_ready()) {
+    k_cl_one<<<1, 1024, smem, st>>>(lv, pv, cl);
+    *nl += 1;
+    return;
+  }
   k_cl_bin<<<nblk(pv.n, 128), 128, 0, st>>>(lv, pv, cl);
   k_cl_scan<<<1, 1024, 0, st>>>(cl);
   k_cl_scatter<<<nblk(pv.n, 128), 128, 0, st>>>(pv, cl);
@@ -2097,15 +2212,20 @@ void launch_pair_features(const LatticeView &lv, const PartView &pv, const int2 
   if (n > 0) k_pair_features<<<nblk(n, 128), 128, 0, st>>>(lv, pv, pairs, n, out);
 }
 
-void launch_mlp_correction(const LatticeView &lv, const PartView &pv, const CellListView &cl, const PairBuf &pb,
-                           float gap_lo, float gap_cut, float speed_lo, float speed_hi, const void *mlp,
-                           cudaStream_t st, int64_t *nl) {
+void launch_mlp_pairs(const LatticeView &lv, const PartView &pv, const CellListView &cl, const PairBuf &pb,
+                      float gap_lo, float gap_cut, float speed_lo, float speed_hi, const void *mlp, cudaStream_t st,
+                      int64_t *nl) {
   if (pv.n == 0) return;
   cudaMemsetAsync(pb.count, 0, sizeof(int), st);
   k_mlp_pairs<<<pv.n, 32, 0, st>>>(lv, pv, cl, pb, gap_lo, gap_cut, speed_lo, speed_hi);
   launch_mlp_forward_dev(mlp, pb.feat, pb.count, pb.cap, pb.out, st);
+  *nl += 2;
+}
+
+void launch_mlp_apply(const PartView &pv, const PairBuf &pb, cudaStream_t st, int64_t *nl) {
+  if (pv.n == 0) return;
   k_mlp_apply<<<nblk((unsigned)pb.cap, 128) < 152u ? nblk((unsigned)pb.cap, 128) : 152u, 128, 0, st>>>(pv, pb);
-  *nl += 3;
+  *nl += 1;
 }
 
 void launch_set_state(const LatticeView &lv, const PartView &pv, int mode, cudaStream_t st, int64_t *nl) {
