@@ -11,6 +11,7 @@
 #include <stdint.h>
 
 #include <type_traits>
+#include <utility>
 
 namespace bl {
 
@@ -116,6 +117,7 @@ struct LatticeView {
   // Lees-Edwards shear (null when off): the sweep leaves (drho, u) of the
   // nodes at x = 0 (first ny nz) and x = nx - 1 (next ny nz), y + ny z
   float4 *le_mom;
+  int dep;  // host: launch programmatic dependents
 };
 
 // Lees-Edwards shear across the plane between x = nx - 1 and x = 0 (Sec. IV,
@@ -262,6 +264,33 @@ struct ChangeList {
   int32_t *items;  // triples (node, old, new)
   int cap;
 };
+
+// Programmatic dependent launch.  A kernel that calls pdl_trigger lets the next
+// kernel of its stream, if that was launched by launch_dependent, start its
+// blocks; that kernel calls pdl_wait before it reads anything the first one
+// writes (the wait ends when the first has finished and its writes are
+// visible).  It hides a launch of 2 to 3 us and what the second kernel can do
+// with older data.  Both calls do nothing in a kernel launched otherwise.  For
+// kernels of few blocks: the sweep launched so filled the SMs before the
+// side streams' kernels, which then waited for its first wave (sheared box 81
+// -> 84 us a step).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... KArgs, class... Args>
+inline void launch_dependent(bool dep, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st,
+                             Args &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = dep ? 1 : 0;  // (else an ordinary launch)
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 // ---------------------------------------------------------------------------
 // launchers (each adds the number of kernels it launched to *nl where given)

@@ -267,6 +267,7 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
   lv.rho0 = (float)p->rho0;
   lv.has_force = 0;
   lv.sweep = AUTO_SWEEP;
+  lv.dep = 1;
   bl::lb_rows_grids(p->store_dtype, lv.rows_grid);
   for (int k = 0; k < 3; ++k) {
     lv.g[k] = (float)p->g[k];
@@ -1202,8 +1203,10 @@ static int ens_capture(bl_ens *e) {
   for (size_t i = 0; i < n && rc == BL_OK; ++i) {
     bl_ctx *c = e->m[i];
     cudaStreamWaitEvent(c->gstream, e->ev_fork, 0);
+    c->lv.dep = 0;  // ordinary launches among the members' branches
     rc = enqueue_step(c, c->gstream);
     if (rc == BL_OK) rc = enqueue_step(c, c->gstream);
+    c->lv.dep = 1;
     cudaEventRecord(e->ev_m[i], c->gstream);
     cudaStreamWaitEvent(e->cap, e->ev_m[i], 0);
   }

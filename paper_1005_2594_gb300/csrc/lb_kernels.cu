@@ -477,6 +477,8 @@ __global__ void __launch_bounds__(128) k_le_gather(LatticeView lv, LeView le) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const S *pop = reinterpret_cast<const S *>(lv.pop);
   float Pc = 0.f;
+  pdl_trigger();
+  pdl_wait();
   if (i < 2 * M) {
     const int pl = i >= M ? 1 : 0;
     const int yz = i - pl * M, y = yz % ny, z = yz / ny;
@@ -519,6 +521,7 @@ __global__ void __launch_bounds__(128) k_le_scatter(LatticeView lv, LeView le) {
   using D = D3Q19;
   const int ny = lv.ny, nz = lv.nz, M = lv.ny * lv.nz;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
   if (i >= 2 * M) return;
   S *pop = reinterpret_cast<S *>(lv.pop);
   const int pl = i >= M ? 1 : 0;
@@ -552,11 +555,11 @@ void launch_lees_edwards(int dtype, const LatticeView &lv, const LeView &le, int
   const unsigned b = 128, g = nblk(2u * (unsigned)lv.ny * (unsigned)lv.nz, b);
 #define BL_LE(S_)                                                   \
   if (par == 0) {                                                   \
-    k_le_gather<S_, 0><<<g, b, 0, st>>>(lv, le);                    \
-    k_le_scatter<S_, 0><<<g, b, 0, st>>>(lv, le);                   \
+    launch_dependent(lv.dep, k_le_gather<S_, 0>, g, b, st, lv, le); \
+    launch_dependent(lv.dep, k_le_scatter<S_, 0>, g, b, st, lv, le); \
   } else {                                                          \
-    k_le_gather<S_, 1><<<g, b, 0, st>>>(lv, le);                    \
-    k_le_scatter<S_, 1><<<g, b, 0, st>>>(lv, le);                   \
+    launch_dependent(lv.dep, k_le_gather<S_, 1>, g, b, st, lv, le); \
+    launch_dependent(lv.dep, k_le_scatter<S_, 1>, g, b, st, lv, le); \
   }
   if (dtype == 0) {
     BL_LE(float)

@@ -443,6 +443,7 @@ __global__ void __launch_bounds__(128, TAU1 || !CELLS ? BL_ONE_MINB : BL_ONE_MIN
   const unsigned zo[3] = {(unsigned)(z == 0 ? lv.nz - 1 : z - 1) * nxy, (unsigned)z * nxy,
                           (unsigned)(z == lv.nz - 1 ? 0 : z + 1) * nxy};
   const S *pop = reinterpret_cast<const S *>(lv.pop);
+  pdl_trigger();  // (the Lees-Edwards passes)
   const uint32_t nbw = valid ? lv.nbm[n] : 0u;
   // the node's populations, neighbour-cell word and pending velocity are
   // requested with its neighbour word, before it is known whether the node

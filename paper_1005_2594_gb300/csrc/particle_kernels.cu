@@ -1,7 +1,7 @@
 // particle_kernels.cu -- the cell side of the coupled step (arXiv:1005.2594):
 //
 //   cell list      count -> scan -> scatter -> per-bin sort, canonical (bin, id);
-//                  in one block for up to 16384 cells and bins
+//                  in one block for up to 4096 cells
 //   potentials     Berne-Pechukas-scaled Hookean cell-cell pairs (Sec. III,
 //                  Eqs. phi, epsilon, sigma) and cell-wall spheres (Eq. sigmaw),
 //                  one block per cell, FP64 contact geometry, FP32 forces,
@@ -37,7 +37,6 @@
 // rotation increment are FP32 around FP64 reference values, and the kernels
 // that test nodes against ellipsoids read each cell's position (node + FP32
 // fraction) and axis in the FP32 form the solve leaves them.
-#include <atomic>
 #include <climits>
 
 #include "bl_internal.cuh"
@@ -71,23 +70,27 @@ __device__ __forceinline__ int cell_bin(const LatticeView &lv, const PartView &p
   return b0 + cl.nb[0] * (b1 + cl.nb[1] * b2);
 }
 
-// The whole list in one block of 1024 threads, counts, starts and ids in shared
-// memory: for up to CL_ONE cells and bins the four kernels below were four
-// launches of 3 to 4 us each on the way to the potentials, the longest way
-// through the step of a small lattice.  Larger lists take the four kernels.
-constexpr int CL_ONE = 16384, CL_PER = CL_ONE / 1024;
+// The whole list in one block, counts, starts and ids in shared memory: for up
+// to CL_ONE cells (and 48 KB of bins and cells) the four kernels below were
+// four launches of 3 to 4 us each on the way to the potentials, the longest way
+// through the step of a small lattice.  Larger lists, which the sweep hides,
+// take the four kernels.  256 threads: a block of 1024 needs a whole SM's
+// registers, and among the kernels of an ensemble none falls free (16-member
+// sweep 368 -> 379 us a step).
+constexpr int CL_T = 256, CL_ONE = 4096, CL_PER = CL_ONE / CL_T;
 
-__global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, CellListView cl) {
+__global__ void __launch_bounds__(CL_T) k_cl_one(LatticeView lv, PartView pv, CellListView cl) {
   extern __shared__ int cl_smem[];
   int *cnt = cl_smem, *ids = cl_smem + cl.nbins;
   __shared__ int wsum[32];
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  for (int b = t; b < cl.nbins; b += 1024) cnt[b] = 0;
+  pdl_trigger();  // the potentials' wall spheres need no list
+  for (int b = t; b < cl.nbins; b += CL_T) cnt[b] = 0;
   __syncthreads();
   int bin[CL_PER], slot[CL_PER];
 #pragma unroll
   for (int u = 0; u < CL_PER; ++u) {
-    const int i = t + 1024 * u;
+    const int i = t + CL_T * u;
     if (i < pv.n) {
       bin[u] = cell_bin(lv, pv, cl, i);
       cl.bin_of[i] = bin[u];
@@ -96,7 +99,7 @@ __global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, Ce
   }
   __syncthreads();
   // exclusive scan: a run of bins per thread, the runs' sums over the block
-  const int per = (cl.nbins + 1023) / 1024, b0 = min(t * per, cl.nbins), b1 = min(b0 + per, cl.nbins);
+  const int per = (cl.nbins + CL_T - 1) / CL_T, b0 = min(t * per, cl.nbins), b1 = min(b0 + per, cl.nbins);
   int sum = 0;
   for (int b = b0; b < b1; ++b) sum += cnt[b];
   int inc = sum;
@@ -108,7 +111,7 @@ __global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, Ce
   if (lane == 31) wsum[wid] = inc;
   __syncthreads();
   if (wid == 0) {
-    int w = wsum[lane];
+    int w = lane < CL_T / 32 ? wsum[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, w, o);
@@ -128,9 +131,9 @@ __global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, Ce
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < CL_PER; ++u)
-    if (t + 1024 * u < pv.n) ids[cnt[bin[u]] + slot[u]] = t + 1024 * u;
+    if (t + CL_T * u < pv.n) ids[cnt[bin[u]] + slot[u]] = t + CL_T * u;
   __syncthreads();
-  for (int b = t; b < cl.nbins; b += 1024) {
+  for (int b = t; b < cl.nbins; b += CL_T) {
     const int s = cnt[b], e = b + 1 < cl.nbins ? cnt[b + 1] : pv.n;
     for (int i = s + 1; i < e; ++i) {
       const int v = ids[i];
@@ -143,7 +146,7 @@ __global__ void __launch_bounds__(1024) k_cl_one(LatticeView lv, PartView pv, Ce
     }
   }
   __syncthreads();
-  for (int i = t; i < pv.n; i += 1024) cl.ids[i] = ids[i];
+  for (int i = t; i < pv.n; i += CL_T) cl.ids[i] = ids[i];
 }
 
 __global__ void k_cl_bin(LatticeView lv, PartView pv, CellListView cl) {
@@ -569,7 +572,6 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
                           (double)(oz + Xi[2]) - pv.X[3 * i + 2]};
     bp_wall(rd, oid, oif, pv, F, T);
   };
-  if (threadIdx.x < 32) near_bins(lv, cl, cl.bin_of[i], s_nb);
   if (sb.bits) {
     const int R = (int)ceilf(pv.sigw_max) + 1;
     const int side = 2 * R + 1;
@@ -603,6 +605,8 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
       }
     }
   }
+  pdl_wait();  // the cell list
+  if (threadIdx.x < 32) near_bins(lv, cl, cl.bin_of[i], s_nb);
   __syncthreads();
   const float rc2 = pv.r_cut * pv.r_cut;
   const float smax = 2.0f * fmaxf(pv.sig_par, pv.sig_perp);
@@ -777,6 +781,7 @@ __global__ void __launch_bounds__(LT, BL_REDUCE_MINB) k_link_reduce(LatticeView 
   __shared__ float shf[LT / 32][27];
   __shared__ int shi[LT / 32][6];
   const int p = blockIdx.x;
+  pdl_trigger();  // the solve's blocks read the cells' state meanwhile
   const int nrec = min(lv.rec_count[p], lv.rec_cap);
   const float4 k0 = pv.kin[3 * p], k1 = pv.kin[3 * p + 1], k2 = pv.kin[3 * p + 2];
   const int Xi[3] = {(int)k0.w, (int)k1.w, (int)k2.w};
@@ -924,21 +929,46 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
   const double Xold = X, o_old = pv.o[c];
   const float *kf = reinterpret_cast<const float *>(pv.kin + 3 * p);
   const float Vpf = kf[4 + k], Wpf = kf[8 + k];
+  // beside the link sums that this kernel waits for: all that needs the state,
+  // the potentials and the contact sums alone, with f = X - rint(X) the
+  // fraction the sweep's lever arms used
+  const int cK = pv.cK[c], cIT = pv.cIT[c];
+  const double f = X - rint(X);
+  const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+  const double f1 = at(f, k1), f2 = at(f, k2);
+  const double cst = pv.rho0 / 18.0;
+  const double Fo = pv.Fpot[c] + pv.PF[c] + (pv.bfc ? pv.m * pv.g[k] : 0.0), To = pv.Tpot[c] + pv.PT[c];
+  const float oldf = (float)o_old;
+  float I[3][3];
+  double dP = 0.0, dL = 0.0;  // m (Vp - V(t-1/2)) and L(t-1/2) - I Wp (small differences, in FP64)
+  if (pv.move == 1) {
+    const float qf = (float)q;
+    const float w = at(qf, 0), x = at(qf, 1), y = at(qf, 2), z = at(qf, 3);
+    const float R[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
+                           {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
+                           {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
+    const float d0 = (float)pv.Iperp, d2 = (float)pv.Ipar;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        I[a][b] = R[a][0] * d0 * R[b][0] + R[a][1] * d0 * R[b][1] + R[a][2] * d2 * R[b][2];
+    double IW = 0.0;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) IW += (double)pick3f(k, I[0][t], I[1][t], I[2][t]) * (double)at(Wpf, t);
+    dL = L - IW;
+    dP = pv.m * ((double)Vpf - V);
+  }
+  pdl_wait();
   float Zs[21];
 #pragma unroll
   for (int i = 0; i < 21; ++i) Zs[i] = pv.lsum_f[21 * p + i];
   // (the link reduction and the contact kernel rewrite these every step)
-  const double K = (double)(pv.lsum_i[6 * p + k] + pv.cK[c]), IT = (double)(pv.lsum_i[6 * p + 3 + k] + pv.cIT[c]);
-  // link force at the predictor: variable part + exact constant part, with
-  // f = X - rint(X) the fraction the sweep's lever arms used
-  const double cst = pv.rho0 / 18.0;
-  const double f = X - rint(X);
-  const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
-  const double fxK = at(f, k1) * at(K, k2) - at(f, k2) * at(K, k1);
+  const double K = (double)(pv.lsum_i[6 * p + k] + cK), IT = (double)(pv.lsum_i[6 * p + 3 + k] + cIT);
+  // link force at the predictor: variable part + exact constant part
+  const double fxK = f1 * at(K, k2) - f2 * at(K, k1);
   double Fl = pv.lsum[6 * p + k] + cst * K, Tl = pv.lsum[6 * p + 3 + k] + cst * (IT - fxK);
-  double Ft = Fl + pv.Fpot[c] + pv.PF[c] + (pv.bfc ? pv.m * pv.g[k] : 0.0);
-  double Tt = Tl + pv.Tpot[c] + pv.PT[c];
-  const float oldf = (float)o_old;
+  double Ft = Fl + Fo, Tt = Tl + To;
   if (wr) {
     pv.PF[c] = 0.0;
     pv.PT[c] = 0.0;
@@ -946,20 +976,6 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
   }
   const bool move = pv.move != 0;
   if (pv.move == 1) {  // free cells; 2: prescribed, V and W stay as set
-    float I[3][3];
-    {
-      const float qf = (float)q;
-      const float w = at(qf, 0), x = at(qf, 1), y = at(qf, 2), z = at(qf, 3);
-      const float R[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
-                             {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
-                             {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
-      const float d0 = (float)pv.Iperp, d2 = (float)pv.Ipar;
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-          I[a][b] = R[a][0] * d0 * R[b][0] + R[a][1] * d0 * R[b][1] + R[a][2] * d2 * R[b][2];
-    }
     float Z[6][6], A[6][6], rhs[6], d[6], inv[6];
     {
       int i = 0;
@@ -977,11 +993,7 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
         for (int t = s; t < 3; ++t, ++i) Z[3 + s][3 + t] = Z[3 + t][3 + s] = Zs[i];
     }
     {
-      // L(t-1/2) - I Wp: a small difference of O(I W) numbers, in FP64
-      double IW = 0.0;
-#pragma unroll
-      for (int t = 0; t < 3; ++t) IW += (double)pick3f(k, I[0][t], I[1][t], I[2][t]) * (double)at(Wpf, t);
-      const float r0 = (float)(Ft - pv.m * ((double)Vpf - V)), r1 = (float)(Tt + (L - IW));
+      const float r0 = (float)(Ft - dP), r1 = (float)(Tt + dL);
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         rhs[s] = at(r0, s);
@@ -1629,6 +1641,7 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
                                                       ChangeList chg, int par_next, int impulses, int replaced) {
   using D = D3Q19;
   const int p = blockIdx.x;
+  pdl_trigger();
   const unsigned long long *touched = pv.touched + (size_t)p * pv.touched_cap;
   // the first touched node of this thread is requested with the count (the
   // list holds touched_cap entries)
@@ -1875,6 +1888,7 @@ __device__ __forceinline__ uint32_t node_word(const LatticeView &lv, int x, int 
 // it; the whole lattice if the change list overflowed (grid-stride)
 __global__ void k_nbm_update(LatticeView lv, ChangeList chg) {
   using D = D3Q19;
+  pdl_wait();
   const int cnt = *chg.count;
   const bool all = cnt > chg.cap;
   const long long total = all ? (long long)lv.N : (long long)cnt * Q;
@@ -2138,29 +2152,18 @@ __global__ void k_mlp_apply(PartView pv, PairBuf pb) {
 
 static inline unsigned nblk(unsigned n, unsigned b) { return (n + b - 1) / b; }
 
-// the one-block list's shared memory (up to 128 KB) has to be asked for once
-// per device
-static bool cl_one_ready() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-  static std::atomic<int> state[64];  // 0 not asked, 1 granted, 2 refused
-  int s = state[dev].load(std::memory_order_acquire);
-  if (s == 0) {
-    s = cudaFuncSetAttribute(k_cl_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * CL_ONE * sizeof(int))) ==
-                cudaSuccess
-            ? 1
-            : 2;
-    if (s == 2) cudaGetLastError();
-    state[dev].store(s, std::memory_order_release);
-  }
-  return s == 1;
-}
+// whether this context's cell kernels are launched as programmatic dependents:
+// not in an ensemble, whose members' kernels would wait for SM slots that the
+// waiting blocks hold (16 members: 368 -> 388 us a step), and not for
+// thousands of cells, whose kernels fill the GPU by themselves (8446: 1081 ->
+// 1084 us); 20 cells 44 -> 41 us, 1022 cells 160 -> 157 us
+static inline bool dependents(const LatticeView &lv, const PartView &pv) { return lv.dep && pv.n <= 4096; }
 
 void launch_cell_list(const LatticeView &lv, const PartView &pv, const CellListView &cl, cudaStream_t st, int64_t *nl) {
   if (pv.n == 0) return;
   const size_t smem = sizeof(int) * ((size_t)cl.nbins + (size_t)pv.n);
-  if (pv.n <= CL_ONE && cl.nbins <= CL_ONE && cl_one_ready()) {
-    k_cl_one<<<1, 1024, smem, st>>>(lv, pv, cl);
+  if (pv.n <= CL_ONE && smem <= 48 * 1024) {
+    k_cl_one<<<1, CL_T, smem, st>>>(lv, pv, cl);
     *nl += 1;
     return;
   }
@@ -2174,7 +2177,9 @@ void launch_cell_list(const LatticeView &lv, const PartView &pv, const CellListV
 void launch_forces(const LatticeView &lv, const PartView &pv, const CellListView &cl, const SurfBits &sb,
                    cudaStream_t st, int64_t *nl) {
   if (pv.n == 0) return;
-  k_forces<<<pv.n, FB, 0, st>>>(lv, pv, cl, sb);
+  // few blocks may wait for the list on the SMs; a thousand would keep the sweep
+  // beside them from its slots
+  launch_dependent(dependents(lv, pv) && pv.n <= 2 * 152, k_forces, pv.n, FB, st, lv, pv, cl, sb);
   *nl += 1;
 }
 
@@ -2184,7 +2189,7 @@ void launch_sums_solve(int dtype, const LatticeView &lv, const PartView &pv, int
   if (pv.n == 0) return;
   if (lv.has_force) k_link_reduce<true><<<pv.n, LT, 0, st>>>(lv, pv);
   else k_link_reduce<false><<<pv.n, LT, 0, st>>>(lv, pv);
-  k_solve<<<nblk(pv.n, SOLVE_CELLS), 32, 0, st>>>(lv, pv);
+  launch_dependent(dependents(lv, pv), k_solve, nblk(pv.n, SOLVE_CELLS), 32, st, lv, pv);
   *nl += 2;
 }
 
@@ -2244,7 +2249,7 @@ void launch_claims(const LatticeView &lv, const PartView &pv, int *claim, const 
 void launch_nbm_update(const LatticeView &lv, const PartView &pv, const ChangeList &chg, cudaStream_t st,
                        int64_t *nl) {
   if (pv.n == 0) return;
-  k_nbm_update<<<4 * 152, 256, 0, st>>>(lv, chg);
+  launch_dependent(dependents(lv, pv), k_nbm_update, 4 * 152, 256, st, lv, chg);
   *nl += 1;
 }
 
