@@ -82,6 +82,12 @@ struct bl_ctx {
   // scratch for read-outs
   double *scratch;
   size_t scratch_bytes;
+  // the cells' state and forces lie in one device block (F, T, X, q, V, L) that
+  // a read-out copies as a whole into pinned memory; pin_set holds the state of
+  // the last set until its upload has finished (ev_set); pin_small takes scalars
+  double *slab, *pin_get, *pin_set;
+  cudaEvent_t ev_set;
+  double *pin_small;
   // timing
   // Lees-Edwards shear (bl_lees_edwards_set): its passes run after every
   // sweep; masked: a wall mask was set (the shear needs fluid planes)
@@ -99,6 +105,8 @@ struct bl_ctx {
 
 static void drop_graph(bl_ctx *c);
 static int read_status(bl_ctx *c);
+static int fetch_status(bl_ctx *c);
+static int status_of(bl_ctx *c);
 static void fill_particle_constants(bl_ctx *c);
 
 static int fail(bl_ctx *c, int code, const char *fmt, ...) {
@@ -293,7 +301,9 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
         cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithPriority(&c->side2, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join3, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_list, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&c->ev_list, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_set, cudaEventDisableTiming) != cudaSuccess ||
+        cudaMallocHost(&c->pin_small, 4 * sizeof(double)) != cudaSuccess) {
       rc = fail(c, BL_ECUDA, "streams");
       break;
     }
@@ -350,12 +360,19 @@ extern "C" int bl_walls_set(bl_ctx *c, const uint8_t *mask) {
 
 static void free_particles(bl_ctx *c) {
   PartView &pv = c->pv;
-  void *ptrs[] = {pv.X, pv.q, pv.V, pv.L, pv.Om, pv.o, pv.axis, pv.qf, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
-                  pv.touched, pv.touched_count, pv.lsum, pv.lsum_f, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink, pv.Ftot,
-                  pv.Ttot, pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
+  void *ptrs[] = {pv.Om, pv.o, pv.axis, pv.qf, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
+                  pv.touched, pv.touched_count, pv.lsum, pv.lsum_f, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink,
+                  pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
                   c->chg.count, c->chg.items, c->lv.rec, c->lv.rec_count};
   for (void *p : ptrs)
     if (p) cudaFree(p);
+  if (c->slab) cudaFree(c->slab);
+  if (c->pin_get) cudaFreeHost(c->pin_get);
+  if (c->pin_set) {
+    cudaEventSynchronize(c->ev_set);
+    cudaFreeHost(c->pin_set);
+  }
+  c->slab = c->pin_get = c->pin_set = nullptr;
   c->lv.rec = nullptr;
   c->lv.rec_count = nullptr;
   c->lv.rec_cap = 0;
@@ -374,8 +391,17 @@ static void free_particles(bl_ctx *c) {
 static int alloc_particles(bl_ctx *c, int n) {
   PartView &pv = c->pv;
   const size_t n3 = sizeof(double) * 3 * (size_t)n;
-  double **d3[] = {&pv.X, &pv.V, &pv.L, &pv.Om, &pv.o, &pv.Fpot, &pv.Tpot, &pv.PF, &pv.PT,
-                   &pv.Flink, &pv.Tlink, &pv.Ftot, &pv.Ttot};
+  CU(cudaMalloc(&c->slab, sizeof(double) * 19 * (size_t)n));
+  CU(cudaMemsetAsync(c->slab, 0, sizeof(double) * 19 * (size_t)n, c->stream));
+  CU(cudaMallocHost(&c->pin_get, sizeof(double) * 19 * (size_t)n));
+  CU(cudaMallocHost(&c->pin_set, sizeof(double) * 13 * (size_t)n));
+  pv.Ftot = c->slab;
+  pv.Ttot = c->slab + 3 * (size_t)n;
+  pv.X = c->slab + 6 * (size_t)n;
+  pv.q = c->slab + 9 * (size_t)n;
+  pv.V = c->slab + 13 * (size_t)n;
+  pv.L = c->slab + 16 * (size_t)n;
+  double **d3[] = {&pv.Om, &pv.o, &pv.Fpot, &pv.Tpot, &pv.PF, &pv.PT, &pv.Flink, &pv.Tlink};
   for (double **d : d3) {
     CU(cudaMalloc(d, n3));
     CU(cudaMemsetAsync(*d, 0, n3, c->stream));
@@ -386,8 +412,6 @@ static int alloc_particles(bl_ctx *c, int n) {
   CU(cudaMemsetAsync(pv.qf, 0, sizeof(float4) * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.oprev, sizeof(float) * 3 * (size_t)n));
   CU(cudaMemsetAsync(pv.oprev, 0, sizeof(float) * 3 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.q, sizeof(double) * 4 * (size_t)n));
-  CU(cudaMemsetAsync(pv.q, 0, sizeof(double) * 4 * (size_t)n, c->stream));
   CU(cudaMalloc(&pv.kin, sizeof(float4) * 3 * (size_t)n));
   CU(cudaMalloc(&pv.kin_next, sizeof(float4) * 3 * (size_t)n));
   CU(cudaMemsetAsync(pv.kin, 0, sizeof(float4) * 3 * (size_t)n, c->stream));
@@ -567,7 +591,15 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
     c->pp = *pp;
   }
   fill_particle_constants(c);
-  std::vector<double> st(13 * (size_t)n);
+  const int dims[3] = {c->lv.nx, c->lv.ny, c->lv.nz};
+  for (int i = 0; i < n; ++i)
+    for (int k = 0; k < 3; ++k)
+      if (!(X[3 * i + k] >= 0.0 && X[3 * i + k] < (double)dims[k]))
+        return fail(c, BL_EINVAL, "cell %d: X outside [0, N)", i);
+  // staged in pinned memory (once the upload of the last set has left it), so
+  // that the copy needs neither the caller's arrays nor a wait
+  CU(cudaEventSynchronize(c->ev_set));
+  double *st = c->pin_set;
   for (int i = 0; i < n; ++i) {
     for (int k = 0; k < 3; ++k) {
       st[13 * i + k] = X[3 * i + k];
@@ -575,12 +607,9 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
       st[13 * i + 10 + k] = L[3 * i + k];
     }
     for (int k = 0; k < 4; ++k) st[13 * i + 3 + k] = q[4 * i + k];
-    const int dims[3] = {c->lv.nx, c->lv.ny, c->lv.nz};
-    for (int k = 0; k < 3; ++k)
-      if (!(X[3 * i + k] >= 0.0 && X[3 * i + k] < (double)dims[k]))
-        return fail(c, BL_EINVAL, "cell %d: X outside [0, N)", i);
   }
-  CU(cudaMemcpyAsync(c->pv.stage, st.data(), sizeof(double) * st.size(), cudaMemcpyHostToDevice, c->stream));
+  CU(cudaMemcpyAsync(c->pv.stage, st, sizeof(double) * 13 * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+  CU(cudaEventRecord(c->ev_set, c->stream));
   launch_set_state(c->lv, c->pv, first ? 1 : 2, c->stream, &c->launches);
   // the search for new owners of nodes that a cell leaves uses the cell list
   // of the new positions
@@ -820,17 +849,25 @@ extern "C" int bl_lees_edwards_get(bl_ctx *c, double *P_sum, int64_t *steps) {
   if (c->sticky) return c->sticky;
   if (!c->le_on) return fail(c, BL_ESTATE, "no Lees-Edwards shear set");
   long long n = 0;
-  CU(cudaMemcpyAsync(P_sum, c->le.P, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaMemcpyAsync(&n, c->le.n, sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaMemcpyAsync(c->pin_small, c->le.P, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaMemcpyAsync(c->pin_small + 1, c->le.n, sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
+  if (fetch_status(c)) return c->sticky;
   CU(cudaStreamSynchronize(c->stream));
+  *P_sum = c->pin_small[0];
+  memcpy(&n, c->pin_small + 1, sizeof(n));
   *steps = (int64_t)n;
-  return read_status(c);
+  return status_of(c);
 }
 
-static int read_status(bl_ctx *c) {
+// copies the status word to pinned memory; status_of, after a wait, judges it
+static int fetch_status(bl_ctx *c) {
+  CU(cudaMemcpyAsync(c->pin_small + 3, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  return BL_OK;
+}
+
+static int status_of(bl_ctx *c) {
   int st = 0;
-  CU(cudaMemcpyAsync(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaStreamSynchronize(c->stream));
+  memcpy(&st, c->pin_small + 3, sizeof(int));
   if (st & ST_UNSTABLE) return fail(c, BL_EUNSTABLE, "unstable: rho <= 0, NaN or |u| >= 0.3 at some node, or a cell speed >= 0.5");
   if (st & ST_OVERFLOW) return fail(c, BL_EOVERFLOW, "internal list overflow");
   if (st & ST_BARRIER) return fail(c, BL_EBARRIER, "a bounded wait for asynchronous copies timed out");
@@ -838,12 +875,19 @@ static int read_status(bl_ctx *c) {
   return BL_OK;
 }
 
+static int read_status(bl_ctx *c) {
+  if (fetch_status(c)) return c->sticky;
+  CU(cudaStreamSynchronize(c->stream));
+  return status_of(c);
+}
+
 extern "C" int bl_sync(bl_ctx *c) {
   if (!c) return BL_EINVAL;
+  cudaMemcpyAsync(c->pin_small + 3, c->status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return fail(c, BL_ECUDA, "stream: %s", cudaGetErrorString(e));
   if (c->sticky) return c->sticky;
-  return read_status(c);
+  return status_of(c);
 }
 
 extern "C" int bl_fields_get(bl_ctx *c, double *rho, double *u, int32_t *owner, int on_device) {
@@ -877,10 +921,13 @@ static int copy_n3(bl_ctx *c, double *dst, const double *src, int comps) {
 extern "C" int bl_forces_get(bl_ctx *c, double *F, double *T, double *X, double *q, double *V, double *L) {
   if (!c) return BL_EINVAL;
   if (c->sticky) return c->sticky;
-  if (copy_n3(c, F, c->pv.Ftot, 3) || copy_n3(c, T, c->pv.Ttot, 3) || copy_n3(c, X, c->pv.X, 3) ||
-      copy_n3(c, q, c->pv.q, 4) || copy_n3(c, V, c->pv.V, 3) || copy_n3(c, L, c->pv.L, 3))
-    return c->sticky;
+  const size_t n = (size_t)c->np;
+  if (n > 0) CU(cudaMemcpyAsync(c->pin_get, c->slab, sizeof(double) * 19 * n, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));
+  double *out[6] = {F, T, X, q, V, L};
+  const size_t at[7] = {0, 3, 6, 9, 13, 16, 19};
+  for (int k = 0; k < 6; ++k)
+    if (out[k] && n > 0) memcpy(out[k], c->pin_get + at[k] * n, sizeof(double) * (at[k + 1] - at[k]) * n);
   return BL_OK;
 }
 
@@ -1332,6 +1379,8 @@ extern "C" void bl_destroy(bl_ctx *c) {
     if (e) cudaEventDestroy(e);
   if (c->side2) cudaStreamDestroy(c->side2);
   free_particles(c);
+  if (c->ev_set) cudaEventDestroy(c->ev_set);
+  if (c->pin_small) cudaFreeHost(c->pin_small);
   void *ptrs[] = {c->lv.pop, c->lv.owner, c->lv.nbm, c->lv.nbc, c->lv.nbx, c->lv.pu, c->claim, c->status,
                   c->wacc.F, c->wacc.K, c->sbits.bits, c->sbits.rows, c->scratch,
                   c->lv.le_mom, c->le.T, c->le.D, c->le.t, c->le.P, c->le.n};

@@ -17,7 +17,7 @@
 // Parameter layout (FP32 master copy, row-major): W1 64 x 14, b1 64,
 // W2 64 x 64, b2 64, W3 6 x 64, b3 6 (5510 values).  Normalisation: inputs
 // x~ = (x - mx) / sx, outputs y = y~ sy + my.
-#include <mutex>
+#include <cstring>
 
 #include "../../include/bloodlb.h"
 #include "bl_internal.cuh"
@@ -449,7 +449,8 @@ struct bl_mlp {
   float *theta, *grad, *m1, *m2, *norm, *partial;
   __nv_bfloat16 *wp;
   int nblocks;
-  int k;  // Adam steps taken
+  float *pin;  // pinned: gradient and loss, or the parameters, on their way to the caller
+  int k;       // Adam steps taken
   char err[128];
 };
 
@@ -476,7 +477,8 @@ extern "C" int bl_mlp_create(bl_mlp **out, void *cuda_stream) {
             cudaMalloc(&m->m2, sizeof(float) * NPAR) == cudaSuccess &&
             cudaMalloc(&m->norm, sizeof(float) * 40) == cudaSuccess &&
             cudaMalloc(&m->partial, sizeof(float) * (NPAR + 1) * MLP_BLOCKS) == cudaSuccess &&
-            cudaMalloc(&m->wp, sizeof(__nv_bfloat16) * P_TOTAL) == cudaSuccess;
+            cudaMalloc(&m->wp, sizeof(__nv_bfloat16) * P_TOTAL) == cudaSuccess &&
+            cudaMallocHost(&m->pin, sizeof(float) * (NPAR + 1)) == cudaSuccess;
   if (ok) {
     cudaMemsetAsync(m->theta, 0, sizeof(float) * NPAR, m->stream);
     cudaMemsetAsync(m->m1, 0, sizeof(float) * NPAR, m->stream);
@@ -519,11 +521,13 @@ extern "C" int bl_mlp_params_set(bl_mlp *m, const float *theta, const float *nor
 
 extern "C" int bl_mlp_params_get(bl_mlp *m, float *theta, float *norm) {
   if (!m) return BL_EINVAL;
-  if (theta && cudaMemcpyAsync(theta, m->theta, sizeof(float) * NPAR, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  if (theta && cudaMemcpyAsync(m->pin, m->theta, sizeof(float) * NPAR, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return BL_ECUDA;
   if (norm && cudaMemcpyAsync(norm, m->norm, sizeof(float) * 40, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
     return BL_ECUDA;
-  return cudaStreamSynchronize(m->stream) == cudaSuccess ? BL_OK : BL_ECUDA;
+  if (cudaStreamSynchronize(m->stream) != cudaSuccess) return BL_ECUDA;
+  if (theta) memcpy(theta, m->pin, sizeof(float) * NPAR);
+  return BL_OK;
 }
 
 static MlpDev mlp_dev(const bl_mlp *m) { return MlpDev{m->wp, m->theta, m->norm}; }
@@ -543,11 +547,15 @@ extern "C" int bl_mlp_grad(bl_mlp *m, const float *x, const float *y, int B, flo
   k_mlp_grad<<<nb, 32 * GW, grad_smem(), m->stream>>>(mlp_dev(m), x, y, B, m->partial);
   k_mlp_reduce<<<(NPAR + 1 + 31) / 32, 256, 0, m->stream>>>(m->partial, nb, m->grad);
   if (cudaGetLastError() != cudaSuccess) return BL_ECUDA;
-  if (loss && cudaMemcpyAsync(loss, m->grad + NPAR, sizeof(float), cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
+  if (!loss && !grad) return BL_OK;
+  // gradient and loss lie together: one copy (the loss alone where that is all)
+  const int o = grad ? 0 : NPAR;
+  if (cudaMemcpyAsync(m->pin + o, m->grad + o, sizeof(float) * (NPAR + 1 - o), cudaMemcpyDeviceToHost, m->stream) !=
+          cudaSuccess ||
+      cudaStreamSynchronize(m->stream) != cudaSuccess)
     return BL_ECUDA;
-  if (grad && cudaMemcpyAsync(grad, m->grad, sizeof(float) * NPAR, cudaMemcpyDeviceToHost, m->stream) != cudaSuccess)
-    return BL_ECUDA;
-  if ((loss || grad) && cudaStreamSynchronize(m->stream) != cudaSuccess) return BL_ECUDA;
+  if (loss) *loss = m->pin[NPAR];
+  if (grad) memcpy(grad, m->pin, sizeof(float) * NPAR);
   return BL_OK;
 }
 
@@ -579,5 +587,6 @@ extern "C" void bl_mlp_destroy(bl_mlp *m) {
   void *p[] = {m->theta, m->grad, m->m1, m->m2, m->norm, m->partial, m->wp};
   for (void *q : p)
     if (q) cudaFree(q);
+  if (m->pin) cudaFreeHost(m->pin);
   delete m;
 }
