@@ -376,48 +376,70 @@ static int node_wall(const bl_lb_params *p, const uint8_t *mask, int x, int y, i
   return -1;
 }
 
-extern "C" int bl_sparse_index_build(const bl_lb_params *p, const uint8_t *mask, int64_t *n_fluid, int32_t *dense_of,
-                                     int32_t *nbr) {
-  if (!p || !n_fluid || p->nx < 1 || p->ny < 1 || p->nz < 1) return BL_EINVAL;
-  const long long N = (long long)p->nx * p->ny * p->nz;
-  if (N >= (1ll << 31)) return BL_EINVAL;
-  for (int k = 0; k < 3; ++k) {
-    const int n = k == 0 ? p->nx : (k == 1 ? p->ny : p->nz);
-    if (!p->periodic[k] && n < 3) return BL_EINVAL;
-  }
-  if (mask)
-    for (long long n = 0; n < N; ++n)
-      if (mask[n] > NWALL) return BL_EINVAL;
-  std::vector<int32_t> id((size_t)N, -1);
-  long long nf = 0;
+// the number of each node among the fluid nodes, -1 - wall id at walls; their number
+static long long index_ids(const bl_lb_params *p, const uint8_t *mask, std::vector<int32_t> &id) {
+  long long nf = 0, n = 0;
   for (int z = 0; z < p->nz; ++z)
     for (int y = 0; y < p->ny; ++y)
-      for (int x = 0; x < p->nx; ++x) {
-        const long long n = (long long)x + (long long)p->nx * ((long long)y + (long long)p->ny * z);
+      for (int x = 0; x < p->nx; ++x, ++n) {
         const int w = node_wall(p, mask, x, y, z);
         id[(size_t)n] = w >= 0 ? -1 - w : (int32_t)nf++;
       }
-  const long long prev = *n_fluid;
-  *n_fluid = nf;
-  if (!dense_of && !nbr) return BL_OK;
-  if (prev < nf) return BL_EINVAL;  // the arrays hold fewer nodes than the lattice has
-  for (int z = 0; z < p->nz; ++z)
-    for (int y = 0; y < p->ny; ++y)
-      for (int x = 0; x < p->nx; ++x) {
-        const long long n = (long long)x + (long long)p->nx * ((long long)y + (long long)p->ny * z);
+  return nf;
+}
+
+// dense index and neighbours of every fluid node (either array may be null)
+static void index_fill(const bl_lb_params *p, const std::vector<int32_t> &id, long long nf, int32_t *dense_of,
+                       int32_t *nbr) {
+  const long long nx = p->nx, ny = p->ny, nz = p->nz;
+  long long n = 0;
+  for (long long z = 0; z < nz; ++z)
+    for (long long y = 0; y < ny; ++y) {
+      // a fluid node's neighbours lie in the box: a walled axis has wall
+      // layers at its ends, a periodic one wraps
+      long long row[3][3];
+      for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+          row[dz + 1][dy + 1] = nx * ((y + dy + ny) % ny + ny * ((z + dz + nz) % nz));
+      for (long long x = 0; x < nx; ++x, ++n) {
         const int32_t i = id[(size_t)n];
         if (i < 0) continue;
         if (dense_of) dense_of[i] = (int32_t)n;
         if (!nbr) continue;
-        for (int r = 1; r < Q; ++r) {
-          // a fluid node's neighbours lie in the box: a walled axis has wall
-          // layers at its ends, a periodic one wraps
-          const int xx = (x + D3Q19::cx(r) + p->nx) % p->nx, yy = (y + D3Q19::cy(r) + p->ny) % p->ny,
-                    zz = (z + D3Q19::cz(r) + p->nz) % p->nz;
-          const long long m = (long long)xx + (long long)p->nx * ((long long)yy + (long long)p->ny * zz);
-          nbr[(size_t)(r - 1) * nf + i] = id[(size_t)m];
-        }
+        const long long xs[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
+        for (int r = 1; r < Q; ++r)
+          nbr[(size_t)(r - 1) * nf + i] =
+              id[(size_t)(row[1 + D3Q19::cz(r)][1 + D3Q19::cy(r)] + xs[1 + D3Q19::cx(r)])];
       }
+    }
+}
+
+// what an index needs of its parameters
+static bool index_ok(const bl_lb_params *p, const uint8_t *mask) {
+  if (p->nx < 1 || p->ny < 1 || p->nz < 1) return false;
+  const long long N = (long long)p->nx * p->ny * p->nz;
+  if (N >= (1ll << 31)) return false;
+  for (int k = 0; k < 3; ++k) {
+    const int n = k == 0 ? p->nx : (k == 1 ? p->ny : p->nz);
+    if (!p->periodic[k] && n < 3) return false;
+  }
+  if (mask)
+    for (long long n = 0; n < N; ++n)
+      if (mask[n] > NWALL) return false;
+  return true;
+}
+
+extern "C" int bl_sparse_index_build(const bl_lb_params *p, const uint8_t *mask, int64_t *n_fluid, int32_t *dense_of,
+                                     int32_t *nbr) {
+  if (!p || !n_fluid || !index_ok(p, mask)) return BL_EINVAL;
+  const long long N = (long long)p->nx * p->ny * p->nz;
+  std::vector<int32_t> id((size_t)N);
+  const long long nf = index_ids(p, mask, id);
+  const long long prev = *n_fluid;
+  *n_fluid = nf;
+  if (!dense_of && !nbr) return BL_OK;
+  if (prev < nf) return BL_EINVAL;  // the arrays hold fewer nodes than the lattice has
+  index_fill(p, id, nf, dense_of, nbr);
   return BL_OK;
 }
 
@@ -543,13 +565,13 @@ extern "C" int bl_sparse_init(bl_sparse **out, const bl_lb_params *p, const uint
   if (!out) return BL_EINVAL;
   *out = nullptr;
   if (!p || !(p->tau > 0.5) || !(p->rho0 > 0) || p->store_dtype < 0 || p->store_dtype > 2) return BL_EINVAL;
-  int64_t nf = 0;
-  int rc = bl_sparse_index_build(p, mask, &nf, nullptr, nullptr);
-  if (rc != BL_OK) return rc;
+  if (!index_ok(p, mask)) return BL_EINVAL;
+  int rc = BL_OK;
+  std::vector<int32_t> id((size_t)p->nx * p->ny * p->nz);
+  const int64_t nf = index_ids(p, mask, id);
   if (nf < 1 || (unsigned long long)nf * Q >= (1ull << 32)) return BL_EINVAL;
   std::vector<int32_t> dense((size_t)nf), nbr((size_t)nf * 18);
-  rc = bl_sparse_index_build(p, mask, &nf, dense.data(), nbr.data());
-  if (rc != BL_OK) return rc;
+  index_fill(p, id, nf, dense.data(), nbr.data());
   RowIndex rows;
   build_rows(p->nx, p->periodic[0] != 0, dense, nbr, rows);
   bl_sparse *s = new bl_sparse();
