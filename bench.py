@@ -262,8 +262,9 @@ SWEEP_KERNELS = {
 
 def sweep_kernel(nx, store, variant=None, cells=True):
     """the sweep kernel the library runs for this row length, storage type
-    and variant (None: the context's own choice, one node per thread with
-    cells, else the bulk-copy pipeline where rows are 16-byte aligned); the
+    and variant (None: with cells the context's own choice, one node per
+    thread; cells=False names the copy pipeline of these rows, which a context
+    without cells runs only where it is set); the
     bulk-copy variants need 16-byte aligned rows and the per-thread pipeline
     FP32, else the library runs one node per thread"""
     name = {0: "FP32", 1: "BF16", 2: "FP16"}[store]

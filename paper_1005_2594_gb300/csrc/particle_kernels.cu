@@ -9,7 +9,7 @@
 //   link sums      per cell over the link records the sweep wrote (Eq.
 //                  deltap): link momentum at the predictor and the drag
 //                  matrices
-//   solve          one thread per cell: velocities of the half step (reading
+//   solve          four lanes per cell: velocities of the half step (reading
 //                  Q3), leap-frog on unit quaternions (reading Q4)
 //   second links   the moving-boundary term C (Eq. c) on the rare links to a
 //                  node's second cell; the first cell's C is added by the
@@ -767,6 +767,11 @@ __device__ __forceinline__ void arm64(const LatticeView &lv, const PartView &pv,
 // bounced populations f~*_r are evaluated again here by the function the
 // sweep collides with.
 
+// One block per cell over its bucket.  Bound by issue: about 480 warp
+// instructions per 32 records, 62 % of the issue slots busy (14.7 us for 628k
+// records of 1022 cells; 83 us, half of that HBM, for 5.2 M of 8446).  The pair
+// terms replaced a loop over each record's directions (18.6 us at 1022 cells,
+// 123 at 8446).
 constexpr int LT = 128;  // threads of a link-reduction block
 // blocks of the link reduction and of the claims resident per SM: enough
 // that one wave holds a thousand cells (the register cap this sets)
@@ -1176,7 +1181,9 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
 // populations it reads; the records of a second or third cell of one node
 // (marked REC_DIRECT) get their C in place.  V, W: the cell's half-step
 // velocities of the solve; d: node minus the cell's position of this step.
-// Every link is one cell's, so no two blocks touch the same slot.
+// Every link is one cell's, so no two blocks touch the same slot.  Bound by
+// scattered 16- and 4-byte accesses: 12.2 us for 1022 cells, 119 us (0.4 GB in
+// 32-byte sectors) for 8446.
 template <class S>
 __global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView pv, int par) {
   constexpr int PQ = 512;  // queue of a block's second- and third-cell records
@@ -1409,6 +1416,9 @@ constexpr int PB = 128;  // threads of the claims and resolve blocks (8 blocks f
 // owned by another cell need no claim: their owner keeps them while it
 // covers them (first arrival), and hands them on through TOUCHED.
 // mode 1: no old ellipsoid (first particles_set, all owners fluid).
+// Bound by latency and issue (10.3 us for 1022 cells, 47 us for 8446); with
+// each thread forming the cell's geometry from its FP64 state it was bound by
+// FP64 issue (19.2 and 112 us).
 // In particles_set (modes 1, 2) also clears the cell's link count and
 // contact sums for the lattice-wide geometry pass, which adds to them; in a
 // step (mode 0) the contact sums of this step are in use, and the next
@@ -1635,7 +1645,8 @@ __device__ __forceinline__ void gather_cands(const LatticeView &lv, const PartVi
 // uncovered ones (a cell leaves) from the back; then each kind is worked off
 // by warps of its own, so that the FP64 of the momentum balance is issued once
 // for up to 32 nodes instead of for the few of one warp's nodes that take a
-// branch.
+// branch.  Bound by latency: a chain of dependent reads per block (17 us for
+// 1022 cells, 84 us for 8446; 23.5 and 128 before).
 template <class S>
 __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv, CellListView cl, int *claim,
                                                       ChangeList chg, int par_next, int impulses, int replaced) {
