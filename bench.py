@@ -247,7 +247,7 @@ def make_workload(name):
 # workload at FP32 storage kept with the profiles, valid for the sweep source
 # it was taken on (lb_sweep.cuh, first 16 hex digits of its SHA-256) and that
 # workload only
-SWEEP_TRAFFIC = {"sha": "bc31081e20bd634a", "config": "shear128", "store": 0, "bytes": 328095360}
+SWEEP_TRAFFIC = {"sha": "7468576a20f18eec", "config": "shear128", "store": 0, "bytes": 330838656}
 
 
 SWEEP_KERNELS = {
@@ -859,10 +859,10 @@ def run_vessel_loop(args, ws, rank, local):
     fl = mask == 0
     diff = float(np.abs(u_sp[fl] - u_dn[fl]).max() / max(np.abs(u_dn[fl]).max(), 1e-30))
     hbm, src = peaks()
-    bytes_per_node = 2 * 19 * dsize + 18 * 4
+    bytes_per_node = 2 * 19 * dsize + 5  # the row index: a word a node, segments
     achieved = bytes_per_node * nf / (ms_sp / args.steps * 1e-3) / 1e9
     value = nf * args.steps / (ms_sp * 1e-3) / 1e6
-    mem_sp = nf * (19 * dsize + 18 * 4 + 4)
+    mem_sp = nf * (19 * dsize + 6 + 4)
     mem_dn = N * (19 * dsize + 4 + 4 + 4 + 16)
     return {
         "metric": METRIC, "value": round(value, 1), "unit": UNIT + " (fluid nodes)", "n_gpus": ws,
@@ -872,7 +872,7 @@ def run_vessel_loop(args, ws, rank, local):
         "config": {"workload": "vessel loop 1024x512x128 (parent radius 32, daughters 25.4), indexed lattice, "
                                "g = 1e-6; value: fluid-node updates per second",
                    "fluid_nodes": int(nf), "box_nodes": int(N), "lumen_fraction": round(nf / N, 4),
-                   "l2": "indexed populations and table %.0f MB > 129 MB L2, no flush" % (mem_sp / 1e6)},
+                   "l2": "indexed populations and row index %.0f MB > 129 MB L2, no flush" % (mem_sp / 1e6)},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                      "frac": round(achieved / hbm, 4), "traffic": None,
                      "peak_source": src + " (MEASURED_PEAKS.json hbm_gbs)" if src == "measured" else "fallback 6.8 TB/s",
