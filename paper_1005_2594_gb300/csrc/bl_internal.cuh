@@ -396,6 +396,29 @@ __device__ __forceinline__ int imin_image(int d, int n, int per) {
   return d;
 }
 
+// periodic image of a separation of two points, each given as its nearest node
+// and the rest: d between the nodes, f between the rests (|f| <= 1).  The nearer
+// image of the separation itself: of the nodes alone it would be the farther one
+// for separations within a node of half a period, which two cells in contact
+// have where a period is short (2 max(R) + 4 at least).
+__device__ __forceinline__ float image_f(int d, float f, int n, int per) {
+  int m = imin_image(d, n, per);
+  if (per) {
+    const float r = (float)m + f, h = 0.5f * (float)n;
+    m -= r > h ? n : (r < -h ? -n : 0);
+  }
+  return (float)m + f;
+}
+
+// the same of an FP64 separation dX, d between the nodes nearest its ends: the
+// image from the nodes (two integer operations where the exact rule takes six
+// FP64 ones) but within a node of half a period
+__device__ __forceinline__ double image_64(double dX, int d, int n, int per) {
+  const int m = imin_image(d, n, per);
+  if (per && 2 * abs(m) > n - 2) return min_image_exact(dX, n, per);
+  return dX + (double)(m - d);
+}
+
 // periodic wrap for coordinates at most a few periods out (no division)
 __device__ __forceinline__ int wrapi(int v, int n) {
   while (v < 0) v += n;

@@ -1,0 +1,59 @@
+"""Separations near half a period, against the oracle: the periodic image is
+the nearest one of the exact separation, not of the positions rounded to
+nodes.  A period may be as short as 2 max(R) + 4, where cells in contact and
+cells that hand a node over can be half a period apart.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import torch
+
+    torch.cuda.init()
+    yield
+
+
+def rel(a, b):
+    return np.abs(np.asarray(a) - np.asarray(b)).max() / np.abs(np.asarray(b)).max()
+
+
+# axis: the axis on which the cells lie just over half a period apart; period:
+# even (the rounded separation can be half a period exactly) or odd
+@pytest.mark.parametrize("period", [18, 19])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_pair_force_takes_the_nearest_image(axis, period):
+    import oracle
+    from paper_1005_2594_gb300 import bloodlb as bl
+    from paper_1005_2594_gb300 import workloads
+
+    shape = [20, 20, 20]
+    shape[axis] = period
+    p = workloads.base_params(*shape, R=(7.0, 3.0), eps=0.01)
+    rng = np.random.default_rng(10 * axis + period)
+    seen = 0
+    while seen < 4:
+        X = np.full((2, 3), 9.0) + rng.uniform(-0.4, 0.4, (2, 3))
+        X[0, axis] = rng.integers(0, 4) + rng.uniform(0.5, 0.6)
+        X[1, axis] = X[0, axis] + 0.5 * period + rng.uniform(0.05, 0.8 if period % 2 == 0 else 0.4)
+        _, q = workloads.random_axes_and_quaternions(rng, 2)
+        r = X[1] - X[0]
+        r[axis] -= period
+        if not np.abs(oracle.pair(p, r, oracle.axis(q[0]), oracle.axis(q[1]))[1]).max() > 1e-5:
+            continue  # out of contact: another orientation
+        seen += 1
+        orc, sim = oracle.Oracle(p), bl.Simulation(p)
+        orc.set_particles(X, q)
+        sim.set_particles(X, q)
+        orc.step(1)
+        sim.step(1)
+        fo, fg = orc.force_parts(), sim.force_parts()
+        # the force of one pair in FP32 (the bar of the other parity tests)
+        assert rel(fg["Fp"], fo["Fp"]) < 1e-5 and rel(fg["Tp"], fo["Tp"]) < 1e-5, (X, q)
+        sim.close()
