@@ -731,13 +731,19 @@ __device__ __forceinline__ bool inside_cell(int x, int y, int z, int p, const Ce
 
 // lever arm of a node from the centre of cell p in FP64: the image of the node
 // nearest the cell chosen in integers, one conversion and one subtraction per
-// axis
+// axis, but within half a node of half a period (a node left by a cell that was
+// set elsewhere) by the exact position
 __device__ __forceinline__ void arm64(const LatticeView &lv, const PartView &pv, const float4 *kin, int p,
                                       const int xyz[3], double a[3]) {
   const int Xi[3] = {(int)kin[3 * p].w, (int)kin[3 * p + 1].w, (int)kin[3 * p + 2].w};
   const int dims[3] = {lv.nx, lv.ny, lv.nz};
-  for (int k = 0; k < 3; ++k)
-    a[k] = __dsub_rn((double)(Xi[k] + imin_image(xyz[k] - Xi[k], dims[k], lv.per[k])), pv.X[3 * p + k]);
+  for (int k = 0; k < 3; ++k) {
+    const int m = imin_image(xyz[k] - Xi[k], dims[k], lv.per[k]);
+    if (lv.per[k] && 2 * abs(m) >= dims[k] - 1)
+      a[k] = min_image_exact(__dsub_rn((double)xyz[k], pv.X[3 * p + k]), dims[k], 1);
+    else
+      a[k] = __dsub_rn((double)(Xi[k] + m), pv.X[3 * p + k]);
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -57,3 +57,30 @@ def test_pair_force_takes_the_nearest_image(axis, period):
         # the force of one pair in FP32 (the bar of the other parity tests)
         assert rel(fg["Fp"], fo["Fp"]) < 1e-5 and rel(fg["Tp"], fo["Tp"]) < 1e-5, (X, q)
         sim.close()
+
+
+@pytest.mark.parametrize("axis", [1, 2])
+@pytest.mark.parametrize("frac", [-0.3, 0.2])
+def test_impulses_of_a_cell_set_half_a_period_away(axis, frac):
+    """the nodes it leaves lie around half a period from its new centre: their
+    lever arms are those of the nearest image of the exact position"""
+    import oracle
+    from paper_1005_2594_gb300 import bloodlb as bl
+    from paper_1005_2594_gb300 import workloads
+
+    p = workloads.base_params(20, 20, 20, R=(3.5, 1.5))
+    rng = np.random.default_rng(axis)
+    X = np.array([[6.2, 6.7, 7.1]])
+    _, q = workloads.random_axes_and_quaternions(rng, 1)
+    X2 = X.copy()
+    X2[0, axis] = 16.0 + frac
+    V = np.array([[0.013, -0.011, 0.017]])
+    L = np.zeros((1, 3))
+    orc, sim = oracle.Oracle(p), bl.Simulation(p)
+    for s in (orc, sim):
+        s.set_particles(X, q, V, L)
+        s.set_particles(X2, q, V, L)
+    PF, PT = orc.pending()
+    got = sim.force_parts()
+    assert rel(got["PF"], PF) < 1e-6 and rel(got["PT"], PT) < 1e-6  # (the bar of the other re-placements)
+    sim.close()
