@@ -1630,7 +1630,7 @@ __device__ __forceinline__ void gather_cands(const LatticeView &lv, const PartVi
       cell_geo(pv, pv.kin_next, j, h);
       float d2 = 0.f;
       for (int m = 0; m < 3; ++m) {
-        const float d = (float)imin_image(h.Xi[m] - g.Xi[m], dims[m], lv.per[m]) + (h.Xf[m] - g.Xf[m]);
+        const float d = image_f(h.Xi[m] - g.Xi[m], h.Xf[m] - g.Xf[m], dims[m], lv.per[m]);
         d2 += d * d;
       }
       if (d2 > reach * reach) continue;

@@ -84,3 +84,32 @@ def test_impulses_of_a_cell_set_half_a_period_away(axis, frac):
     got = sim.force_parts()
     assert rel(got["PF"], PF) < 1e-6 and rel(got["PT"], PT) < 1e-6  # (the bar of the other re-placements)
     sim.close()
+
+
+# spheres of radius 4 in a 12^3 box: cell 0 leaves a node that cell 1 covers
+# through the boundary; on two axes they are just under half a period apart,
+# and the positions rounded to nodes just over it
+@pytest.mark.parametrize("X,v", [
+    ([[1.3298, 8.7825, 0.3315], [8.4863, 0.7281, 7.4738]], [0.17137, -0.1396, 0.17188]),
+    ([[3.3311, 1.3282, 2.8234], [10.4822, 8.4037, 6.6342]], [0.17203, 0.17472, -0.1352]),
+    ([[3.3818, 3.3489, 10.8101], [10.4578, 10.4678, 2.5878]], [0.17462, 0.17309, -0.13397]),
+])
+def test_node_handed_over_through_the_boundary(X, v):
+    import oracle
+    from paper_1005_2594_gb300 import bloodlb as bl
+    from paper_1005_2594_gb300 import workloads
+
+    p = workloads.base_params(12, 12, 12, R=(4.0, 4.0), eps=0.0, r_cut=5.0)
+    p["move_particles"] = 2
+    X, V = np.array(X), np.array([v, [0.0, 0.0, 0.0]])
+    q = np.tile([1.0, 0.0, 0.0, 0.0], (2, 1))
+    orc, sim = oracle.Oracle(p), bl.Simulation(p)
+    for s in (orc, sim):
+        s.set_particles(X, q, V, np.zeros((2, 3)))
+    before = orc.owner()
+    orc.step(1)
+    sim.step(1)
+    after = orc.owner()
+    assert ((before == 0) & (after == 1)).any()  # a direct change of owner
+    np.testing.assert_array_equal(sim.owner(), after)
+    sim.close()
