@@ -1479,13 +1479,21 @@ __global__ void __launch_bounds__(PB, BL_CLAIMS_MINB) k_claims(LatticeView lv, P
       int ao2, bo2, ai2, bi2;
       row_range(qo, 1.0f + ROW_EPS, xfo[0], ao2, bo2);
       row_range(qo, 1.0f - ROW_EPS, xfo[0], ai2, bi2);
-      if (ao2 <= bo2) {
+      const int oa = ao2 + shift, ob = bo2 + shift;
+      if (ao2 <= bo2 && lv.per[0] && (oa < imin || ob > imax)) {
+        // set far away: the old interval reaches over the end of the period
+        // counted from the new centre, so every node of the row is looked at
+        ao = imin;
+        bo = imax;
+        ai2 = 1;
+        bi2 = 0;
+      } else if (ao2 <= bo2) {
         if (ao > bo) {
-          ao = ao2 + shift;
-          bo = bo2 + shift;
+          ao = oa;
+          bo = ob;
         } else {
-          ao = min(ao, ao2 + shift);
-          bo = max(bo, bo2 + shift);
+          ao = min(ao, oa);
+          bo = max(bo, ob);
         }
       }
       if (ai2 <= bi2) {

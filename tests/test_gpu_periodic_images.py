@@ -86,6 +86,36 @@ def test_impulses_of_a_cell_set_half_a_period_away(axis, frac):
     sim.close()
 
 
+@pytest.mark.parametrize("shape,periodic", [((20, 20, 20), (1, 1, 1)), ((21, 24, 20), (1, 1, 1)),
+                                            ((44, 20, 22), (0, 1, 1)), ((40, 21, 24), (1, 0, 1))])
+def test_cells_set_anywhere_leave_their_nodes(shape, periodic):
+    """re-placements by any distance, owner maps exact and the impulses of the nodes left and entered"""
+    import oracle
+    from paper_1005_2594_gb300 import bloodlb as bl
+    from paper_1005_2594_gb300 import workloads
+
+    p = workloads.base_params(*shape, periodic=periodic, R=(3.5, 1.5))
+    rng = np.random.default_rng(sum(shape))
+    n = 3
+    lo = np.array([0.0 if k else 6.0 for k in periodic])
+    hi = np.array([s if k else s - 7.0 for s, k in zip(shape, periodic)])
+    draw = lambda: (lo + rng.uniform(0.0, 1.0, (n, 3)) * (hi - lo), workloads.random_axes_and_quaternions(rng, n)[1])
+    orc, sim = oracle.Oracle(p), bl.Simulation(p)
+    X, q = draw()
+    V, L = rng.uniform(-0.02, 0.02, (n, 3)), np.zeros((n, 3))
+    for s in (orc, sim):
+        s.set_particles(X, q, V, L)
+    for _ in range(8):
+        X, q = draw()
+        for s in (orc, sim):
+            s.set_particles(X, q, V, L)
+        np.testing.assert_array_equal(sim.owner(), orc.owner())
+        PF, PT = orc.pending()
+        got = sim.force_parts()
+        assert rel(got["PF"], PF) < 1e-6 and rel(got["PT"], PT) < 1e-6
+    sim.close()
+
+
 # spheres of radius 4 in a 12^3 box: cell 0 leaves a node that cell 1 covers
 # through the boundary; on two axes they are just under half a period apart,
 # and the positions rounded to nodes just over it
