@@ -630,6 +630,12 @@ __device__ __forceinline__ float wall_term(float rho, const float (&v)[3]) {
   return __fmul_rn(__fmul_rn(-(D::m(R) / 6.0f), rho), cv);
 }
 
+// a population with the pending moving-boundary term of its bounce along r
+// added, f + C with C = -(m_r / 6) c_r . u, cu = c_r . u.  One function with the
+// contraction written out: the field read-out and the flush of the pending
+// terms form the same number, which FP16 storage then rounds alike
+__device__ __forceinline__ float add_pending(float f, int m, float cu) { return fmaf(-((float)m / 6.0f), cu, f); }
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

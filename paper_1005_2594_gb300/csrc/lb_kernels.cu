@@ -157,10 +157,10 @@ __global__ void __launch_bounds__(FT) k_fields(LatticeView lv, int par, double r
         sfor<1, Q>([&](auto R) {
           constexpr int r = decltype(R)::value;
           if ((pm >> r) & 1u) {
-            const float C = -(D::m(r) / 6.0f) * (D::cx(r) * pu.x + D::cy(r) * pu.y + D::cz(r) * pu.z);
-            // in the storage type, as a read-out has always shown it
+            // in the storage type, as bl_populations_get shows it
             S v;
-            Store<S>::st(&v, f[D::opp(r)] + C);
+            Store<S>::st(&v, add_pending(f[D::opp(r)], D::m(r),
+                                         D::cx(r) * pu.x + D::cy(r) * pu.y + D::cz(r) * pu.z));
             f[D::opp(r)] = Store<S>::ld(&v);
           }
         });

@@ -1293,10 +1293,10 @@ __global__ void k_flush_pending(LatticeView lv, int par) {
     node_xyz(lv, n, yc);
     for (uint32_t m = pm; m; m &= m - 1u) {
       const int r = __ffs(m) - 1;
-      const float C = -(D::m(r) / 6.0f) * (D::cx(r) * pu.x + D::cy(r) * pu.y + D::cz(r) * pu.z);
       // the slot from which node n reads direction rbar in layout par
       const unsigned slot = bounce_slot(lv, par ^ 1, n, yc, r);
-      Store<S>::st(pop + slot, Store<S>::ld(pop + slot) + C);
+      Store<S>::st(pop + slot, add_pending(Store<S>::ld(pop + slot), D::m(r),
+                                           D::cx(r) * pu.x + D::cy(r) * pu.y + D::cz(r) * pu.z));
     }
     reinterpret_cast<float *>(lv.pu + n)[3] = 0.f;
   }
