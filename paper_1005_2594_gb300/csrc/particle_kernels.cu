@@ -227,35 +227,41 @@ __global__ void k_cl_sort(CellListView cl) {
 // proportional to it: rounding r and sigma to FP32 (~1e-7) would put ~1e-5
 // into the force.  With sigma = sigma_bar / sqrt(S) and P = r^2 S,
 //   h = (sigma_bar^2 - P) / (sigma_bar (sigma_bar + sqrt(P))),
-// so the one difference is formed in FP64, from products of the positions and
-// axes without a root or a normalised vector, and its quotient in FP32.  Two
-// FP64 reciprocals (Newton from the FP32 one) replace six roots and divisions
-// of some 20 FP64 instructions each: the contact geometry was 170 FP64
-// instructions per warp, each holding the SM's FP64 pipe for 16 cycles, and
-// bound the kernel (104 us on 256^3 with 8446 cells).  The strength, its
-// derivatives and the force and torque, which multiply h without cancelling
-// it, are FP32.
+//   sigma = sigma_bar r / sqrt(P),
+// so the one difference is formed from products of the positions and axes
+// without a root or a normalised vector.  h, sigma and S are formed in FP64 and
+// rounded to FP32 once (their quotients in FP32 raised the force's error from
+// 8.6e-8 to 1.0e-7 rms).  FP64 reciprocals (Newton from the FP32 one) replace
+// roots and divisions of some 20 FP64 instructions each: two steps where the
+// result enters the difference, one where it is rounded to FP32 next.  The
+// contact geometry was 170 FP64 instructions per warp, each holding the SM's
+// FP64 pipe for 16 cycles, and bound the kernel (104 us on 256^3 with 8446
+// cells).  The strength, its derivatives and the force and torque, which
+// multiply h without cancelling it, are FP32.
 
-// 1 / x and 1 / sqrt(x) in FP64 to about an ulp, for x within FP32's range
-// (rsqrt64: the root and quotient themselves below it)
+// 1 / x in FP64 to about an ulp, or (STEPS = 1) to 2^-43, for x within FP32's range
+template <int STEPS>
 __device__ __forceinline__ double rcp64(double x) {
   double y = (double)(1.0f / (float)x);
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k) y = fma(y, fma(-x, y, 1.0), y);
+  return y;
 }
+// 1 / sqrt(x) to 2^-43 (below FP32's range the root and quotient themselves)
 __device__ __forceinline__ double rsqrt64(double x) {
   if (!(x > 1e-30)) return 1.0 / sqrt(x);
-  double y = (double)rsqrtf((float)x);
-  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  const double y = (double)rsqrtf((float)x);
   return fma(0.5 * y, fma(-x * y, y, 1.0), y);
 }
 __device__ __forceinline__ double dot64(const double a[3], const double b[3]) {
   return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
 }
 
-// h from sigma_bar^2 - P (> 0) and P
-__device__ __forceinline__ float overlap(double D, double P, float sigbar) {
-  return (float)D / (sigbar * (sigbar + sqrtf((float)P)));
+// h and sigma from sigma_bar^2 - P (> 0), P and r
+__device__ __forceinline__ void overlap(double D, double P, double r, double sigbar, float &h, float &sigma) {
+  const double y = rsqrt64(P);
+  h = (float)(D * rcp64<1>(sigbar * fma(P, y, sigbar)));
+  sigma = (float)(sigbar * (r * y));
 }
 
 // FP32 test of a pair against its contact distance (Eq. sigma) with a
@@ -282,13 +288,13 @@ __device__ __forceinline__ void bp_pair(const double rd[3], const double oid[3],
   const double A = dot64(rd, oid), B = dot64(rd, ojd), cd = dot64(oid, ojd);
   const double Ap = A + B, Am = A - B, qp = fma(pv.chi_d, cd, 1.0), qm = fma(-pv.chi_d, cd, 1.0);
   // (A + B)^2 / (1 + chi c) + (A - B)^2 / (1 - chi c)
-  const double X = fma(Ap * Ap, qm, Am * Am * qp) * rcp64(qp * qm);
+  const double X = fma(Ap * Ap, qm, Am * Am * qp) * rcp64<2>(qp * qm);
   const double P = fma(-0.5 * pv.chi_d, X, r2), D = pv.sigbar_d * pv.sigbar_d - P;
   if (!(D > 0.0)) return;
-  const double ird = rsqrt64(r2);
-  const float h = overlap(D, P, pv.sigbar);
-  const float rl = (float)(r2 * ird), ir = (float)ird, S = (float)(P * (ird * ird));
-  const float sigma = pv.sigbar / sqrtf(S);
+  const double ird = rsqrt64(r2), rld = r2 * ird;
+  float h, sigma;
+  overlap(D, P, rld, pv.sigbar_d, h, sigma);
+  const float rl = (float)rld, ir = (float)ird, S = (float)(P * (ird * ird));
   const float rh[3] = {(float)(rd[0] * ird), (float)(rd[1] * ird), (float)(rd[2] * ird)};
   const float a = (float)(A * ird), b = (float)(B * ird), c = (float)cd;
   const float chi = pv.chi;
@@ -335,10 +341,10 @@ __device__ __forceinline__ void bp_wall(const double rd[3], const double oid[3],
   const double A = dot64(rd, oid);
   const double P = fma(-pv.chi_w_d * A, A, r2), D = pv.sigbar_w_d * pv.sigbar_w_d - P;
   if (!(D > 0.0)) return;
-  const double ird = rsqrt64(r2);
-  const float h = overlap(D, P, pv.sigbar_w);
-  const float rl = (float)(r2 * ird), ir = (float)ird, S = (float)(P * (ird * ird)), a = (float)(A * ird);
-  const float sigma = pv.sigbar_w / sqrtf(S);
+  const double ird = rsqrt64(r2), rld = r2 * ird;
+  float h, sigma;
+  overlap(D, P, rld, pv.sigbar_w_d, h, sigma);
+  const float rl = (float)rld, ir = (float)ird, S = (float)(P * (ird * ird)), a = (float)(A * ird);
   const float rh[3] = {(float)(rd[0] * ird), (float)(rd[1] * ird), (float)(rd[2] * ird)};
   const float eps = pv.eps_w;
   const float dsig_a = sigma * pv.chi_w * a / S;
