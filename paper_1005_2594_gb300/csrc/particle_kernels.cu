@@ -71,18 +71,21 @@ __device__ __forceinline__ int cell_bin(const LatticeView &lv, const PartView &p
 }
 
 // The whole list in one block, counts, starts and ids in shared memory: for up
-// to CL_ONE cells (and 48 KB of bins and cells) the four kernels below were
+// to CL_ONE cells (and CL_SMEM bytes of bins and cells) the four kernels below were
 // four launches of 3 to 4 us each on the way to the potentials, the longest way
 // through the step of a small lattice.  Larger lists, which the sweep hides,
 // take the four kernels.  256 threads: a block of 1024 needs a whole SM's
 // registers, and among the kernels of an ensemble none falls free (16-member
 // sweep 368 -> 379 us a step).
 constexpr int CL_T = 256, CL_ONE = 4096, CL_PER = CL_ONE / CL_T;
+constexpr int CL_WSUM = 32;  // warp sums of the scan
+// dynamic shared memory: a block has 48 KB without an opt-in, its static part included
+constexpr size_t CL_SMEM = 48 * 1024 - sizeof(int) * CL_WSUM;
 
 __global__ void __launch_bounds__(CL_T) k_cl_one(LatticeView lv, PartView pv, CellListView cl) {
   extern __shared__ int cl_smem[];
   int *cnt = cl_smem, *ids = cl_smem + cl.nbins;
-  __shared__ int wsum[32];
+  __shared__ int wsum[CL_WSUM];
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   pdl_trigger();  // the potentials' wall spheres need no list
   for (int b = t; b < cl.nbins; b += CL_T) cnt[b] = 0;
@@ -2190,7 +2193,7 @@ static inline bool dependents(const LatticeView &lv, const PartView &pv) { retur
 void launch_cell_list(const LatticeView &lv, const PartView &pv, const CellListView &cl, cudaStream_t st, int64_t *nl) {
   if (pv.n == 0) return;
   const size_t smem = sizeof(int) * ((size_t)cl.nbins + (size_t)pv.n);
-  if (pv.n <= CL_ONE && smem <= 48 * 1024) {
+  if (pv.n <= CL_ONE && smem <= CL_SMEM) {
     k_cl_one<<<1, CL_T, smem, st>>>(lv, pv, cl);
     *nl += 1;
     return;
