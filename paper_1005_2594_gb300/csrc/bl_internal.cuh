@@ -170,7 +170,8 @@ constexpr uint32_t NBX_NONE = 0xFFFFu;
 // WALL_COPIES sets of sums, a block adding to one of them: every warp beside a
 // wall adds to its wall's six words, and on one set those additions stood in
 // line at one L2 slice (the indexed sweep of a 2.2 M node vessel loop took 132
-// us in the even step, 85 of them for this).  The read-out adds the sets up.
+// us in the even step, 85 of them for this).  The read-out adds the sets up
+// (launch_wall_read).
 constexpr int WALL_COPIES = 128;
 constexpr int WALL_SUMS = NWALL * 3;
 struct WallAcc {
@@ -182,19 +183,6 @@ struct WallAcc {
 __device__ __forceinline__ WallAcc wall_copy(const WallAcc &wa) {
   const unsigned c = (blockIdx.x + 31u * blockIdx.y + 57u * blockIdx.z) % (unsigned)WALL_COPIES;
   return WallAcc{wa.F + c * WALL_SUMS, wa.K + c * WALL_SUMS};
-}
-
-// the sets' sums as momentum per wall and component (host)
-inline void wall_total(const double *F, const long long *K, double rho0, double *out) {
-  for (int i = 0; i < WALL_SUMS; ++i) {
-    double f = 0.0;
-    long long k = 0;
-    for (int c = 0; c < WALL_COPIES; ++c) {
-      f += F[c * WALL_SUMS + i];
-      k += K[c * WALL_SUMS + i];
-    }
-    out[i] = f + rho0 / 18.0 * (double)k;
-  }
 }
 
 // Cells.  Their bounce links come from the sweep's link records
@@ -296,6 +284,8 @@ inline void launch_dependent(bool dep, void (*kernel)(KArgs...), dim3 grid, dim3
 // launchers (each adds the number of kernels it launched to *nl where given)
 
 void launch_lb_step(int dtype, const LatticeView &lv, int par, const WallAcc &wa, int *status, cudaStream_t st);
+// the walls' momentum of all sets (WALL_SUMS values) to pinned host memory; the sums start anew
+void launch_wall_read(const WallAcc &wa, double rho0, double *out, cudaStream_t st);
 // the persistent row sweep's grid per instantiation (LatticeView::rows_grid)
 void lb_rows_grids(int dtype, int out[8]);
 // pend: add the pending moving-boundary terms (there are cells)

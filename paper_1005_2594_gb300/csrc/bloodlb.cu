@@ -303,7 +303,7 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
         cudaEventCreateWithFlags(&c->ev_join3, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_list, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_set, cudaEventDisableTiming) != cudaSuccess ||
-        cudaMallocHost(&c->pin_small, 4 * sizeof(double)) != cudaSuccess) {
+        cudaMallocHost(&c->pin_small, bl::WALL_SUMS * sizeof(double)) != cudaSuccess) {
       rc = fail(c, BL_ECUDA, "streams");
       break;
     }
@@ -946,14 +946,11 @@ extern "C" int bl_force_parts_get(bl_ctx *c, double *Fh, double *Th, double *Fp,
 extern "C" int bl_wall_momentum_get(bl_ctx *c, double *wallmom) {
   if (!c || !wallmom) return BL_EINVAL;
   if (c->sticky) return c->sticky;
-  double F[bl::WALL_COPIES * bl::WALL_SUMS];
-  long long K[bl::WALL_COPIES * bl::WALL_SUMS];
-  CU(cudaMemcpyAsync(F, c->wacc.F, sizeof(F), cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaMemcpyAsync(K, c->wacc.K, sizeof(K), cudaMemcpyDeviceToHost, c->stream));
+  launch_wall_read(c->wacc, c->lp.rho0, c->pin_small, c->stream);
+  c->launches++;
+  if (check_launch(c, "wall momentum")) return c->sticky;
   CU(cudaStreamSynchronize(c->stream));
-  CU(cudaMemsetAsync(c->wacc.F, 0, sizeof(F), c->stream));
-  CU(cudaMemsetAsync(c->wacc.K, 0, sizeof(K), c->stream));
-  wall_total(F, K, c->lp.rho0, wallmom);
+  memcpy(wallmom, c->pin_small, sizeof(double) * bl::WALL_SUMS);
   return BL_OK;
 }
 

@@ -343,6 +343,7 @@ struct bl_sparse {
   int64_t launches;
   double *scratch;
   size_t scratch_bytes;
+  double *pin;  // pinned: the walls' momentum, written by its kernel
 };
 
 static int sp_fail(bl_sparse *s, int code, const char *fmt, ...) {
@@ -542,6 +543,7 @@ extern "C" void bl_sparse_destroy(bl_sparse *s) {
                   (void *)s->sv.dense, s->sv.status, s->wa.F, s->wa.K, s->scratch};
   for (void *q : ptrs)
     if (q) cudaFree(q);
+  if (s->pin) cudaFreeHost(s->pin);
   delete s;
 }
 
@@ -604,6 +606,10 @@ extern "C" int bl_sparse_init(bl_sparse **out, const bl_lb_params *p, const uint
         !put(s->wa.F, nullptr, sizeof(double) * WALL_COPIES * WALL_SUMS) ||
         !put(s->wa.K, nullptr, sizeof(long long) * WALL_COPIES * WALL_SUMS)) {
       rc = sp_fail(s, BL_ENOMEM, "indexed lattice");
+      break;
+    }
+    if (cudaMallocHost(&s->pin, sizeof(double) * WALL_SUMS) != cudaSuccess) {
+      rc = sp_fail(s, BL_ENOMEM, "pinned memory");
       break;
     }
     if (cudaStreamCreateWithFlags(&s->gstream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -751,14 +757,11 @@ extern "C" int bl_sparse_populations_set(bl_sparse *s, const double *pop) {
 extern "C" int bl_sparse_wall_momentum_get(bl_sparse *s, double *wallmom) {
   if (!s || !wallmom) return BL_EINVAL;
   if (s->sticky) return s->sticky;
-  double F[WALL_COPIES * WALL_SUMS];
-  long long K[WALL_COPIES * WALL_SUMS];
-  SPCU(cudaMemcpyAsync(F, s->wa.F, sizeof(F), cudaMemcpyDeviceToHost, s->stream));
-  SPCU(cudaMemcpyAsync(K, s->wa.K, sizeof(K), cudaMemcpyDeviceToHost, s->stream));
+  launch_wall_read(s->wa, s->lp.rho0, s->pin, s->stream);
+  s->launches++;
+  if (sp_check(s, "wall momentum")) return s->sticky;
   SPCU(cudaStreamSynchronize(s->stream));
-  SPCU(cudaMemsetAsync(s->wa.F, 0, sizeof(F), s->stream));
-  SPCU(cudaMemsetAsync(s->wa.K, 0, sizeof(K), s->stream));
-  wall_total(F, K, s->lp.rho0, wallmom);
+  memcpy(wallmom, s->pin, sizeof(double) * WALL_SUMS);
   return BL_OK;
 }
 

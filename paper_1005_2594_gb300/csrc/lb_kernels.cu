@@ -111,6 +111,27 @@ __global__ void __launch_bounds__(128) k_geometry(LatticeView lv, PartView pv) {
 }
 
 // ---------------------------------------------------------------------------
+// the walls' momentum: one warp per value, its lanes over the sets, in a fixed
+// order; a block each, so that their FP64 additions share no SM.  Written to
+// pinned host memory by the kernel: a copy after it is a second round trip, and
+// the round trip of the call (25 KB are read) is what it takes.
+__global__ void __launch_bounds__(32) k_wall_read(WallAcc wa, double rho18, double *out) {
+  const int i = blockIdx.x;
+  double f = 0.0;
+  long long k = 0;
+  for (int c = threadIdx.x; c < WALL_COPIES; c += 32) {
+    f += wa.F[c * WALL_SUMS + i];
+    k += wa.K[c * WALL_SUMS + i];
+    wa.F[c * WALL_SUMS + i] = 0.0;
+    wa.K[c * WALL_SUMS + i] = 0;
+  }
+  f = warp_sum_d(f);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  if (threadIdx.x == 0) out[i] = f + rho18 * (double)k;
+}
+
+// ---------------------------------------------------------------------------
 // moments of the current populations (layout of parity par), with the pending
 // moving-boundary terms of the last step's bounces off cells (pend: there are
 // cells) added to the populations as they are read, so that a read-out leaves
@@ -360,6 +381,10 @@ void launch_geometry(const LatticeView &lv, const PartView &pv, cudaStream_t st,
   dim3 grid((lv.nx + bx - 1) / bx, lv.ny, lv.nz);
   k_geometry<<<grid, bx, 0, st>>>(lv, pv);
   if (nl) ++*nl;
+}
+
+void launch_wall_read(const WallAcc &wa, double rho0, double *out, cudaStream_t st) {
+  k_wall_read<<<WALL_SUMS, 32, 0, st>>>(wa, rho0 / 18.0, out);
 }
 
 void launch_fields(int dtype, const LatticeView &lv, int par, int pend, double *rho, double *u, int32_t *owner,
