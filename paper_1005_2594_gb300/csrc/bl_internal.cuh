@@ -100,7 +100,7 @@ struct LatticeView {
   int32_t *owner;  // N
   uint32_t *nbm;   // N neighbour words of the current owner map (NB_* bits), written by the geometry pass
   uint32_t *nbc;   // N neighbour-cell words (NBC_*), written with the neighbour words
-  uint4 *nbx;      // N mixed words (NBX_*): read for nodes between a cell and another cell or a wall
+  uint4 *nbx;      // N mixed words (NBX_*): read for nodes between a cell and another cell or a wall (null without cells)
   // Cell links of the sweep.  A fluid node next to a cell writes one link
   // record per cell into that cell's bucket, for the link-momentum sums.
   // The moving-boundary term C of its bounced populations needs the cell's

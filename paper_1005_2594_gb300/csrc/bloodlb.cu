@@ -318,7 +318,6 @@ extern "C" int bl_lb_init(bl_ctx **out, const bl_lb_params *p, void *cuda_stream
     if ((rc = check_launch(c, "init")) != BL_OK) break;
     if (cudaMalloc(&lv.nbm, sizeof(uint32_t) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "neighbour words"); break; }
     if (cudaMalloc(&lv.nbc, sizeof(uint32_t) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "neighbour-cell words"); break; }
-    if (cudaMalloc(&lv.nbx, sizeof(uint4) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "mixed words"); break; }
     if (cudaMalloc(&lv.pu, sizeof(float4) * N) != cudaSuccess) { rc = fail(c, BL_ENOMEM, "pending velocities"); break; }
     cudaMemsetAsync(lv.pu, 0, sizeof(float4) * N, c->stream);
     lv.status = c->status;
@@ -391,6 +390,9 @@ static void free_particles(bl_ctx *c) {
 static int alloc_particles(bl_ctx *c, int n) {
   PartView &pv = c->pv;
   const size_t n3 = sizeof(double) * 3 * (size_t)n;
+  // the mixed words, which only nodes beside a cell have: with the first cells,
+  // until a call without cells (16 bytes per node)
+  if (!c->lv.nbx) CU(cudaMalloc(&c->lv.nbx, sizeof(uint4) * (size_t)c->lv.N));
   CU(cudaMalloc(&c->slab, sizeof(double) * 19 * (size_t)n));
   CU(cudaMemsetAsync(c->slab, 0, sizeof(double) * 19 * (size_t)n, c->stream));
   CU(cudaMallocHost(&c->pin_get, sizeof(double) * 19 * (size_t)n));
@@ -580,6 +582,8 @@ extern "C" int bl_particles_set(bl_ctx *c, int n, const bl_particle_params *pp, 
     free_particles(c);
     c->pp = *pp;
     if (n == 0) {
+      cudaFree(c->lv.nbx);
+      c->lv.nbx = nullptr;
       launch_geometry(c->lv, c->pv, c->stream, &c->launches);
       if (check_launch(c, "geometry")) return c->sticky;
       CU(cudaStreamSynchronize(c->stream));
