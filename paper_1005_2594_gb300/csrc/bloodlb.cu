@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -30,6 +31,7 @@ using namespace bl;
 namespace {
 constexpr int NGROUPS = 5;
 constexpr int MAX_TIMED = 1 << 16;
+constexpr int STATE_GET = 19, STATE_SET = 13;  // doubles per cell of a state read-out and of a set (X, q, V, L)
 }  // namespace
 
 struct bl_ctx {
@@ -82,10 +84,12 @@ struct bl_ctx {
   // scratch for read-outs
   double *scratch;
   size_t scratch_bytes;
-  // the cells' state and forces lie in one device block (F, T, X, q, V, L) that
-  // a read-out copies as a whole into pinned memory; pin_set holds the state of
-  // the last set until its upload has finished (ev_set); pin_small takes scalars
-  double *slab, *pin_get, *pin_set;
+  // the cells' arrays lie in one device block; state is its first part, the state
+  // and forces (F, T, X, q, V, L) that a read-out copies into pinned memory
+  // (pin_get); pin_set, behind that, holds the state of the last set until its
+  // upload has finished (ev_set); pin_small takes scalars
+  char *slab;
+  double *state, *pin_get, *pin_set;
   cudaEvent_t ev_set;
   double *pin_small;
   // timing
@@ -357,21 +361,63 @@ extern "C" int bl_walls_set(bl_ctx *c, const uint8_t *mask) {
   return build_surface_bits(c);
 }
 
+// places the cells' arrays, all but the per-cell lists, in one block at base
+// (null: only its size, which is returned).  One allocation and one clearing:
+// some thirty of each took 0.1 ms of a first placement.
+static size_t place_cells(bl_ctx *c, size_t n, size_t nbins, char *base) {
+  size_t at = 0;
+  auto put = [&](auto *&p, size_t count) {
+    at = (at + 255) & ~(size_t)255;
+    if (base) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + at);
+    at += sizeof(*p) * count;
+  };
+  PartView &pv = c->pv;
+  put(c->state, STATE_GET * n);
+  if (base) {
+    pv.Ftot = c->state;
+    pv.Ttot = c->state + 3 * n;
+    pv.X = c->state + 6 * n;
+    pv.q = c->state + 9 * n;
+    pv.V = c->state + 13 * n;
+    pv.L = c->state + 16 * n;
+  }
+  for (double **d : {&pv.Om, &pv.o, &pv.Fpot, &pv.Tpot, &pv.PF, &pv.PT, &pv.Flink, &pv.Tlink}) put(*d, 3 * n);
+  put(pv.lsum, 6 * n);
+  put(pv.stage, STATE_SET * n);
+  put(pv.kin, 3 * n);
+  put(pv.kin_next, 3 * n);
+  put(pv.axis, n);
+  put(pv.qf, n);
+  put(pv.oprev, 3 * n);
+  put(pv.lsum_f, 21 * n);
+  put(pv.vw, 6 * n);
+  put(pv.lsum_i, 6 * n);
+  put(pv.cK, 3 * n);
+  put(pv.cIT, 3 * n);
+  put(pv.box, 6 * n);
+  put(c->lv.rec_count, n);
+  put(pv.rec_last, n);
+  put(pv.touched_count, n);
+  put(c->cl.bin_of, n);
+  put(c->cl.ids, n);
+  put(c->cl.count, nbins);
+  put(c->cl.cursor, nbins);
+  put(c->cl.start, nbins + 1);
+  put(c->chg.count, 1);
+  return at;
+}
+
 static void free_particles(bl_ctx *c) {
   PartView &pv = c->pv;
-  void *ptrs[] = {pv.Om, pv.o, pv.axis, pv.qf, pv.oprev, pv.kin, pv.kin_next, pv.rec_last, pv.cK, pv.cIT,
-                  pv.touched, pv.touched_count, pv.lsum, pv.lsum_f, pv.lsum_i, pv.vw, pv.Fpot, pv.Tpot, pv.PF, pv.PT, pv.Flink, pv.Tlink,
-                  pv.box, pv.stage, c->cl.bin_of, c->cl.count, c->cl.start, c->cl.cursor, c->cl.ids,
-                  c->chg.count, c->chg.items, c->lv.rec, c->lv.rec_count};
+  void *ptrs[] = {c->slab, pv.touched, c->chg.items, c->lv.rec};
   for (void *p : ptrs)
     if (p) cudaFree(p);
-  if (c->slab) cudaFree(c->slab);
-  if (c->pin_get) cudaFreeHost(c->pin_get);
-  if (c->pin_set) {
-    cudaEventSynchronize(c->ev_set);
-    cudaFreeHost(c->pin_set);
+  if (c->pin_get) {
+    cudaEventSynchronize(c->ev_set);  // (the last set's upload)
+    cudaFreeHost(c->pin_get);
   }
-  c->slab = c->pin_get = c->pin_set = nullptr;
+  c->slab = nullptr;
+  c->state = c->pin_get = c->pin_set = nullptr;
   c->lv.rec = nullptr;
   c->lv.rec_count = nullptr;
   c->lv.rec_cap = 0;
@@ -389,50 +435,6 @@ static void free_particles(bl_ctx *c) {
 
 static int alloc_particles(bl_ctx *c, int n) {
   PartView &pv = c->pv;
-  const size_t n3 = sizeof(double) * 3 * (size_t)n;
-  // the mixed words, which only nodes beside a cell have: with the first cells,
-  // until a call without cells (16 bytes per node)
-  if (!c->lv.nbx) CU(cudaMalloc(&c->lv.nbx, sizeof(uint4) * (size_t)c->lv.N));
-  CU(cudaMalloc(&c->slab, sizeof(double) * 19 * (size_t)n));
-  CU(cudaMemsetAsync(c->slab, 0, sizeof(double) * 19 * (size_t)n, c->stream));
-  CU(cudaMallocHost(&c->pin_get, sizeof(double) * 19 * (size_t)n));
-  CU(cudaMallocHost(&c->pin_set, sizeof(double) * 13 * (size_t)n));
-  pv.Ftot = c->slab;
-  pv.Ttot = c->slab + 3 * (size_t)n;
-  pv.X = c->slab + 6 * (size_t)n;
-  pv.q = c->slab + 9 * (size_t)n;
-  pv.V = c->slab + 13 * (size_t)n;
-  pv.L = c->slab + 16 * (size_t)n;
-  double **d3[] = {&pv.Om, &pv.o, &pv.Fpot, &pv.Tpot, &pv.PF, &pv.PT, &pv.Flink, &pv.Tlink};
-  for (double **d : d3) {
-    CU(cudaMalloc(d, n3));
-    CU(cudaMemsetAsync(*d, 0, n3, c->stream));
-  }
-  CU(cudaMalloc(&pv.axis, sizeof(float4) * (size_t)n));
-  CU(cudaMemsetAsync(pv.axis, 0, sizeof(float4) * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.qf, sizeof(float4) * (size_t)n));
-  CU(cudaMemsetAsync(pv.qf, 0, sizeof(float4) * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.oprev, sizeof(float) * 3 * (size_t)n));
-  CU(cudaMemsetAsync(pv.oprev, 0, sizeof(float) * 3 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.kin, sizeof(float4) * 3 * (size_t)n));
-  CU(cudaMalloc(&pv.kin_next, sizeof(float4) * 3 * (size_t)n));
-  CU(cudaMemsetAsync(pv.kin, 0, sizeof(float4) * 3 * (size_t)n, c->stream));
-  CU(cudaMemsetAsync(pv.kin_next, 0, sizeof(float4) * 3 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.box, sizeof(int) * 6 * (size_t)n));
-  CU(cudaMemsetAsync(pv.box, 0, sizeof(int) * 6 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.stage, sizeof(double) * 13 * (size_t)n));
-  CU(cudaMalloc(&pv.lsum, sizeof(double) * 6 * (size_t)n));
-  CU(cudaMemsetAsync(pv.lsum, 0, sizeof(double) * 6 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.lsum_f, sizeof(float) * 21 * (size_t)n));
-  CU(cudaMemsetAsync(pv.lsum_f, 0, sizeof(float) * 21 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.lsum_i, sizeof(int) * 6 * (size_t)n));
-  CU(cudaMemsetAsync(pv.lsum_i, 0, sizeof(int) * 6 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.vw, sizeof(float) * 6 * (size_t)n));
-  CU(cudaMemsetAsync(pv.vw, 0, sizeof(float) * 6 * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.cK, sizeof(int) * 3 * (size_t)n));
-  CU(cudaMalloc(&pv.cIT, sizeof(int) * 3 * (size_t)n));
-  CU(cudaMemsetAsync(pv.cK, 0, sizeof(int) * 3 * (size_t)n, c->stream));
-  CU(cudaMemsetAsync(pv.cIT, 0, sizeof(int) * 3 * (size_t)n, c->stream));
   // per-cell lists: link records of the sweep (one per fluid node next to
   // the cell: at most the nodes within one node of its surface, fewer than
   // twice the area of a sphere of radius max(R) + 1) and nodes touched by
@@ -444,14 +446,6 @@ static int alloc_particles(bl_ctx *c, int n) {
   if (rec_cap * n > 2.0e9 || t_cap * n > 2.0e9 || n > 65535) return fail(c, BL_EINVAL, "cell lists too large");
   c->lv.rec_cap = (int)rec_cap;
   pv.touched_cap = (int)t_cap;
-  CU(cudaMalloc(&c->lv.rec, sizeof(float4) * 2 * (size_t)c->lv.rec_cap * n));
-  CU(cudaMalloc(&c->lv.rec_count, sizeof(int) * (size_t)n));
-  CU(cudaMemsetAsync(c->lv.rec_count, 0, sizeof(int) * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.rec_last, sizeof(int) * (size_t)n));
-  CU(cudaMemsetAsync(pv.rec_last, 0, sizeof(int) * (size_t)n, c->stream));
-  CU(cudaMalloc(&pv.touched, sizeof(unsigned long long) * (size_t)pv.touched_cap * n));
-  CU(cudaMalloc(&pv.touched_count, sizeof(int) * (size_t)n));
-  CU(cudaMemsetAsync(pv.touched_count, 0, sizeof(int) * (size_t)n, c->stream));
   // cell list bins: nb_k = max(1, floor(N_k / r_cut))
   const int dims[3] = {c->lv.nx, c->lv.ny, c->lv.nz};
   // bin counts in double, checked before any conversion to int
@@ -465,18 +459,20 @@ static int alloc_particles(bl_ctx *c, int n) {
   if (!(nbins_d <= (double)(1 << 26))) return fail(c, BL_EINVAL, "r_cut gives too many bins");
   const long long nbins = (long long)nbins_d;
   c->cl.nbins = (int)nbins;
-  CU(cudaMalloc(&c->cl.bin_of, sizeof(int) * (size_t)n));
-  CU(cudaMalloc(&c->cl.count, sizeof(int) * (size_t)nbins));
-  CU(cudaMalloc(&c->cl.cursor, sizeof(int) * (size_t)nbins));
-  CU(cudaMalloc(&c->cl.start, sizeof(int) * (size_t)(nbins + 1)));
-  CU(cudaMalloc(&c->cl.ids, sizeof(int) * (size_t)n));
-  CU(cudaMemsetAsync(c->cl.count, 0, sizeof(int) * (size_t)nbins, c->stream));
-  CU(cudaMemsetAsync(c->cl.cursor, 0, sizeof(int) * (size_t)nbins, c->stream));
+  // the mixed words, which only nodes beside a cell have: with the first cells,
+  // until a call without cells (16 bytes per node)
+  if (!c->lv.nbx) CU(cudaMalloc(&c->lv.nbx, sizeof(uint4) * (size_t)c->lv.N));
+  const size_t bytes = place_cells(c, (size_t)n, (size_t)nbins, nullptr);
+  CU(cudaMalloc(&c->slab, bytes));
+  CU(cudaMemsetAsync(c->slab, 0, bytes, c->stream));
+  place_cells(c, (size_t)n, (size_t)nbins, c->slab);
+  CU(cudaMallocHost(&c->pin_get, sizeof(double) * (STATE_GET + STATE_SET) * (size_t)n));
+  c->pin_set = c->pin_get + STATE_GET * (size_t)n;
+  CU(cudaMalloc(&c->lv.rec, sizeof(float4) * 2 * (size_t)c->lv.rec_cap * n));
+  CU(cudaMalloc(&pv.touched, sizeof(unsigned long long) * (size_t)pv.touched_cap * n));
   // diagnostic list of changed nodes (overflow only truncates the list)
   c->chg.cap = 64 * n + 4096;
-  CU(cudaMalloc(&c->chg.count, sizeof(int)));
   CU(cudaMalloc(&c->chg.items, sizeof(int32_t) * 3 * (size_t)c->chg.cap));
-  CU(cudaMemsetAsync(c->chg.count, 0, sizeof(int), c->stream));
   c->np = n;
   pv.n = n;
   return BL_OK;
@@ -936,7 +932,7 @@ extern "C" int bl_forces_get(bl_ctx *c, double *F, double *T, double *X, double 
   while (k1 > k0 && !out[k1 - 1]) --k1;
   if (n > 0 && k0 < k1) {
     const bool one = k1 - k0 == 1;
-    CU(cudaMemcpyAsync(one ? out[k0] : c->pin_get + at[k0] * n, c->slab + at[k0] * n,
+    CU(cudaMemcpyAsync(one ? out[k0] : c->pin_get + at[k0] * n, c->state + at[k0] * n,
                        sizeof(double) * (at[k1] - at[k0]) * n, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     for (int k = k0; k < k1 && !one; ++k)
