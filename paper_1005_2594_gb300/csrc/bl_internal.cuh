@@ -306,7 +306,7 @@ void launch_forces(const LatticeView &lv, const PartView &pv, const CellListView
 // link sums from the sweep's records and the implicit solve + leap-frog;
 // then the pending C of the records (independent of the claims, which need
 // only the solve)
-void launch_sums_solve(int dtype, const LatticeView &lv, const PartView &pv, int par, cudaStream_t st, int64_t *nl);
+void launch_sums_solve(const LatticeView &lv, const PartView &pv, cudaStream_t st, int64_t *nl);
 void launch_link_pending(int dtype, const LatticeView &lv, const PartView &pv, int par, cudaStream_t st,
                          int64_t *nl);
 void launch_set_state(const LatticeView &lv, const PartView &pv, int mode, cudaStream_t st, int64_t *nl);

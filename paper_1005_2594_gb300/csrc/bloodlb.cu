@@ -691,7 +691,7 @@ static int enqueue_step(bl_ctx *c, cudaStream_t st) {
     cudaStreamWaitEvent(st, c->ev_join, 0);
     cudaStreamWaitEvent(st, c->ev_join3, 0);
     group_begin(c, 3, &slot, st);
-    launch_sums_solve(c->dtype, c->lv, c->pv, c->parity, st, &c->launches);
+    launch_sums_solve(c->lv, c->pv, st, &c->launches);
     group_end(c, slot, st);
     // the claims need only the solve: beside the pending C of the records
     cudaEventRecord(c->ev_fork2, st);

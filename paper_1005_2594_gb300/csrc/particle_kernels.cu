@@ -2214,9 +2214,7 @@ void launch_forces(const LatticeView &lv, const PartView &pv, const CellListView
   *nl += 1;
 }
 
-void launch_sums_solve(int dtype, const LatticeView &lv, const PartView &pv, int par, cudaStream_t st, int64_t *nl) {
-  (void)dtype;
-  (void)par;
+void launch_sums_solve(const LatticeView &lv, const PartView &pv, cudaStream_t st, int64_t *nl) {
   if (pv.n == 0) return;
   if (lv.has_force) k_link_reduce<true><<<pv.n, LT, 0, st>>>(lv, pv);
   else k_link_reduce<false><<<pv.n, LT, 0, st>>>(lv, pv);
