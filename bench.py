@@ -863,7 +863,7 @@ def run_vessel_loop(args, ws, rank, local):
     achieved = bytes_per_node * nf / (ms_sp / args.steps * 1e-3) / 1e9
     value = nf * args.steps / (ms_sp * 1e-3) / 1e6
     mem_sp = nf * (19 * dsize + 6 + 4)
-    mem_dn = N * (19 * dsize + 4 + 4 + 4 + 16)
+    mem_dn = N * (19 * dsize + 4 * 4 + 16)  # owner, claim, neighbour and neighbour-cell word, pending velocity
     return {
         "metric": METRIC, "value": round(value, 1), "unit": UNIT + " (fluid nodes)", "n_gpus": ws,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms_sp / args.steps, 5),
