@@ -251,10 +251,13 @@ int bl_cell_list_build_static(const double *X, int n, const int32_t dims[3], dou
    walking its share of the rows through one bulk-copy pipeline.  3 to 5
    need rows of a multiple of 16 bytes (nx a multiple of 4 in FP32, of 8 in
    BF16 / FP16; otherwise they run as variant 0).  A context that was given
-   no variant runs 0 (with cells the block-wide barriers of 1 to 5 make
-   every warp wait for the slowest; without, it already streams at the copy
-   bandwidth).  bl_sweep_variant sets one and keeps it (BL_EINVAL for an unknown variant, or variant 1 or 2
-   with 16-bit storage).  A bounded wait for the bulk copies that gives up
+   no variant runs 0: with cells the block-wide barriers of 1 to 5 make
+   every warp wait for the slowest (128^3 with 1022 cells: 162 us a step in
+   FP32, the others 171 to 203; 149 in BF16, 156 to 165); without, on seven
+   boxes from 32^3 to 256^3 in each storage type, none of the others was
+   faster by more than 1.5 %, most slower by 5 to 100 %.  They are there to
+   be set or tried (bl_autotune).  bl_sweep_variant sets one and keeps it
+   (BL_EINVAL for an unknown variant, or variant 1 or 2 with 16-bit storage).  A bounded wait for the bulk copies that gives up
    makes the next bl_sync return BL_EBARRIER.
    bl_autotune times every variant the storage type allows over trial_steps
    steps (>= 2; the context advances by those steps, so call it before the
@@ -283,8 +286,7 @@ int bl_autotune(bl_ctx *c, int trial_steps, int *choice);
    the dense lattice's plasma update of Sec. II (moments, Guo forcing, BGK
    toward the third-order equilibrium, mid-link bounce-back with the
    moving-wall term C, the walls' momentum); cells are not coupled to it.
-   Fluid nodes are numbered in dense node order (x fastest); a table gives
-   each one's 18 neighbours.  Walls: the face layers of non-periodic axes
+   Fluid nodes are numbered in dense node order (x fastest).  Walls: the face layers of non-periodic axes
    (ids 0..5, first walled axis in x, y, z order) and a mask of N bytes as
    for bl_walls_set (value k in 1..8: wall id k - 1, overriding). */
 typedef struct bl_sparse bl_sparse;
@@ -301,7 +303,8 @@ int bl_sparse_index_build(const bl_lb_params *p, const uint8_t *mask, int64_t *n
 
 /* Creates an indexed lattice: builds the index on the host, uploads it and
    sets resting fluid n^eq(rho_bar, 0).  Storage 19 x n_fluid elements of
-   p->store_dtype plus 18 x n_fluid int32.  cuda_stream as in bl_lb_init. */
+   p->store_dtype plus about 10 bytes per fluid node (a word and a share of a
+   segment for its neighbours, its dense index).  cuda_stream as in bl_lb_init. */
 int bl_sparse_init(bl_sparse **out, const bl_lb_params *p, const uint8_t *mask, void *cuda_stream);
 /* nsteps steps (pairs of steps replay one CUDA graph). */
 int bl_sparse_step(bl_sparse *s, int nsteps);

@@ -169,9 +169,9 @@ constexpr uint32_t NBX_NONE = 0xFFFFu;
 // FP64, constant part 2 alpha_r rho_bar c_r as exact integer sums of m_r c_r.
 // WALL_COPIES sets of sums, a block adding to one of them: every warp beside a
 // wall adds to its wall's six words, and on one set those additions stood in
-// line at one L2 slice (the indexed sweep of a 2.2 M node vessel loop took 132
-// us in the even step, 85 of them for this).  The read-out adds the sets up
-// (launch_wall_read).
+// line at one L2 slice (about 85 us of the even step of a 2.2 M node vessel
+// loop, 223 -> 61 us with these sets and the row index).  The read-out adds the
+// sets up (launch_wall_read).
 constexpr int WALL_COPIES = 128;
 constexpr int WALL_SUMS = NWALL * 3;
 struct WallAcc {

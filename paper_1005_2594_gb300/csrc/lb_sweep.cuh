@@ -47,13 +47,14 @@ namespace bl {
 #ifndef BL_LB_MINB
 #define BL_LB_MINB 8
 #endif
-// the one-node sweep: 9 blocks (56 registers, no spill at tau = 1) keep more
-// loads in flight than 8 (64 registers): 94 -> 89.5 us at 128^3 with cells
+// the one-node sweep: 9 blocks (56 registers; no spill without cells, 8 to 24
+// bytes with cells at tau = 1) keep more loads in flight than 8 (64 registers):
+// 94 -> 89.5 us at 128^3 with cells
 #ifndef BL_ONE_MINB
 #define BL_ONE_MINB 9
 #endif
 // with cells at tau != 1 the old populations stay live through the collision:
-// 72 registers instead of 190 spilled bytes
+// 7 blocks (72 registers, 108 to 144 spilled bytes; 190 at 56 registers)
 #ifndef BL_ONE_MINB_BGK
 #define BL_ONE_MINB_BGK 7
 #endif

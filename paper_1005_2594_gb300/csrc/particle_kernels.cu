@@ -1195,7 +1195,8 @@ __global__ void __launch_bounds__(32) k_solve(LatticeView lv, PartView pv) {
 // velocities of the solve; d: node minus the cell's position of this step.
 // Every link is one cell's, so no two blocks touch the same slot.  Bound by
 // scattered 16- and 4-byte accesses: 12.2 us for 1022 cells, 119 us (0.4 GB in
-// 32-byte sectors) for 8446.
+// 32-byte sectors) for 8446.  The second-cell records hold 18 populations and
+// slots at once: 72 registers and 72 to 104 spilled bytes, on their rare path.
 template <class S>
 __global__ void __launch_bounds__(LT, 7) k_link_pending(LatticeView lv, PartView pv, int par) {
   constexpr int PQ = 512;  // queue of a block's second- and third-cell records
