@@ -219,6 +219,7 @@ struct PartView {
   double inv_rpar2, inv_rperp2, R_par, R_perp;
   float Rpar2_f, Rperp2_f, Rmax_f;  // R^2 and the larger half-axis in FP32
   float inv_rpar2_f, inv_rperp2_f, kk_f;  // 1 / R^2 in FP32, kk = 1 / R_par^2 - 1 / R_perp^2
+  int near_image;  // some period is shorter than two contact distances and two nodes
   float sig_par, sig_perp, eps, eps_w, mu, nu, chi_prime, r_cut;
   float chi, sigbar, sigbar_w, chi_w, sigw_max;
   double chi_d, sigbar_d, sigbar_w_d, chi_w_d;  // the same in FP64 (contact geometry)
@@ -398,15 +399,6 @@ __device__ __forceinline__ float image_f(int d, float f, int n, int per) {
     m -= r > h ? n : (r < -h ? -n : 0);
   }
   return (float)m + f;
-}
-
-// the same of an FP64 separation dX, d between the nodes nearest its ends: the
-// image from the nodes (two integer operations where the exact rule takes six
-// FP64 ones) but within a node of half a period
-__device__ __forceinline__ double image_64(double dX, int d, int n, int per) {
-  const int m = imin_image(d, n, per);
-  if (per && 2 * abs(m) > n - 2) return min_image_exact(dX, n, per);
-  return dX + (double)(m - d);
 }
 
 // periodic wrap for coordinates at most a few periods out (no division)

@@ -517,6 +517,13 @@ static void fill_particle_constants(bl_ctx *c) {
   pv.kk_f = (float)(pv.inv_rpar2 - pv.inv_rperp2);
   pv.R_par = pp.R_par;
   pv.R_perp = pp.R_perp;
+  // an image chosen by the nodes nearest two cells can be the farther one where
+  // they are within a node of half a period apart: beyond every contact
+  // distance (2 max(sigma)) in a period of at least two of those and two nodes
+  const int dims[3] = {c->lv.nx, c->lv.ny, c->lv.nz};
+  pv.near_image = 0;
+  for (int k = 0; k < 3; ++k)
+    if (c->lv.per[k] && (double)dims[k] < 4.0 * fmax(pp.sig_par, pp.sig_perp) + 2.1) pv.near_image = 1;
   pv.sig_par = (float)pp.sig_par;
   pv.sig_perp = (float)pp.sig_perp;
   pv.eps = (float)pp.eps;

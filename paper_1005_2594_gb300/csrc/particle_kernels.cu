@@ -558,12 +558,17 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
   const int dims[3] = {lv.nx, lv.ny, lv.nz};
   float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
   // the FP64 state (of the step's start: the solve rewrites it only after the
-  // join) is read where a contact is evaluated
+  // join) is read where a contact is evaluated; the periodic image comes from
+  // the nearest nodes, in integers, but in a box so short that a contact can
+  // reach half a period (near_image)
   auto pair_force = [&](int j) {
     const int Xj[3] = {(int)pv.kin[3 * j].w, (int)pv.kin[3 * j + 1].w, (int)pv.kin[3 * j + 2].w};
     double rd[3];
-    for (int m = 0; m < 3; ++m)
-      rd[m] = image_64(__dsub_rn(pv.X[3 * j + m], pv.X[3 * i + m]), Xj[m] - Xi[m], dims[m], lv.per[m]);
+    for (int m = 0; m < 3; ++m) {
+      const double d = __dsub_rn(pv.X[3 * j + m], pv.X[3 * i + m]);
+      const int dn = Xj[m] - Xi[m];
+      rd[m] = pv.near_image ? min_image_exact(d, dims[m], lv.per[m]) : d + (double)(imin_image(dn, dims[m], lv.per[m]) - dn);
+    }
     const double oid[3] = {pv.o[3 * i], pv.o[3 * i + 1], pv.o[3 * i + 2]};
     const double ojd[3] = {pv.o[3 * j], pv.o[3 * j + 1], pv.o[3 * j + 2]};
     const float4 aj = pv.axis[j];
@@ -624,7 +629,10 @@ __global__ void __launch_bounds__(FB, 7) k_forces(LatticeView lv, PartView pv, C
     const int Xj[3] = {(int)b0.w, (int)b1.w, (int)b2.w};
     const float fj[3] = {b0.x, b0.y, b0.z};
     float r[3];
-    for (int m = 0; m < 3; ++m) r[m] = image_f(Xj[m] - Xi[m], fj[m] - fi[m], dims[m], lv.per[m]);
+    if (pv.near_image)
+      for (int m = 0; m < 3; ++m) r[m] = image_f(Xj[m] - Xi[m], fj[m] - fi[m], dims[m], lv.per[m]);
+    else
+      for (int m = 0; m < 3; ++m) r[m] = (float)imin_image(Xj[m] - Xi[m], dims[m], lv.per[m]) + (fj[m] - fi[m]);
     const float r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
     // no contact distance exceeds 2 max(sigma_perp, sigma_par); nearer
     // pairs first get the contact distance in FP32 (its error is ~1e-6
