@@ -220,6 +220,7 @@ struct PartView {
   float Rpar2_f, Rperp2_f, Rmax_f;  // R^2 and the larger half-axis in FP32
   float inv_rpar2_f, inv_rperp2_f, kk_f;  // 1 / R^2 in FP32, kk = 1 / R_par^2 - 1 / R_perp^2
   int near_image;  // some period is shorter than two contact distances and two nodes
+  int near_reach;  // some period is shorter than twice the owner search's reach and two nodes
   float sig_par, sig_perp, eps, eps_w, mu, nu, chi_prime, r_cut;
   float chi, sigbar, sigbar_w, chi_w, sigw_max;
   double chi_d, sigbar_d, sigbar_w_d, chi_w_d;  // the same in FP64 (contact geometry)

@@ -519,11 +519,15 @@ static void fill_particle_constants(bl_ctx *c) {
   pv.R_perp = pp.R_perp;
   // an image chosen by the nodes nearest two cells can be the farther one where
   // they are within a node of half a period apart: beyond every contact
-  // distance (2 max(sigma)) in a period of at least two of those and two nodes
+  // distance (2 max(sigma)) in a period of at least two of those and two nodes, and
+  // beyond the owner search's reach (2 max(R) + 2) likewise
   const int dims[3] = {c->lv.nx, c->lv.ny, c->lv.nz};
-  pv.near_image = 0;
-  for (int k = 0; k < 3; ++k)
-    if (c->lv.per[k] && (double)dims[k] < 4.0 * fmax(pp.sig_par, pp.sig_perp) + 2.1) pv.near_image = 1;
+  pv.near_image = pv.near_reach = 0;
+  for (int k = 0; k < 3; ++k) {
+    if (!c->lv.per[k]) continue;
+    if ((double)dims[k] < 4.0 * fmax(pp.sig_par, pp.sig_perp) + 2.1) pv.near_image = 1;
+    if ((double)dims[k] < 4.0 * fmax(pp.R_par, pp.R_perp) + 6.1) pv.near_reach = 1;
+  }
   pv.sig_par = (float)pp.sig_par;
   pv.sig_perp = (float)pp.sig_perp;
   pv.eps = (float)pp.eps;

@@ -748,15 +748,17 @@ __device__ __forceinline__ bool inside_cell(int x, int y, int z, int p, const Ce
 
 // lever arm of a node from the centre of cell p in FP64: the image of the node
 // nearest the cell chosen in integers, one conversion and one subtraction per
-// axis, but within half a node of half a period (a node left by a cell that was
-// set elsewhere) by the exact position
+// axis, but within half a node of half a period by the exact position (SET: a node
+// left by a cell that was set elsewhere; in a step a node is within max(R) + 1 of
+// the cell's nearest node, and a period is 2 max(R) + 4 at least)
+template <bool SET>
 __device__ __forceinline__ void arm64(const LatticeView &lv, const PartView &pv, const float4 *kin, int p,
                                       const int xyz[3], double a[3]) {
   const int Xi[3] = {(int)kin[3 * p].w, (int)kin[3 * p + 1].w, (int)kin[3 * p + 2].w};
   const int dims[3] = {lv.nx, lv.ny, lv.nz};
   for (int k = 0; k < 3; ++k) {
     const int m = imin_image(xyz[k] - Xi[k], dims[k], lv.per[k]);
-    if (lv.per[k] && 2 * abs(m) >= dims[k] - 1)
+    if (SET && lv.per[k] && 2 * abs(m) >= dims[k] - 1)
       a[k] = min_image_exact(__dsub_rn((double)xyz[k], pv.X[3 * p + k]), dims[k], 1);
     else
       a[k] = __dsub_rn((double)(Xi[k] + m), pv.X[3 * p + k]);
@@ -1498,8 +1500,8 @@ __global__ void __launch_bounds__(PB, BL_CLAIMS_MINB) k_claims(LatticeView lv, P
       row_range(qo, 1.0f + ROW_EPS, xfo[0], ao2, bo2);
       row_range(qo, 1.0f - ROW_EPS, xfo[0], ai2, bi2);
       const int oa = ao2 + shift, ob = bo2 + shift;
-      if (ao2 <= bo2 && lv.per[0] && (oa < imin || ob > imax)) {
-        // set far away: the old interval reaches over the end of the period
+      if (mode == 2 && ao2 <= bo2 && lv.per[0] && (oa < imin || ob > imax)) {
+        // set far away (a step moves less than half a node): the old interval reaches over the end of the period
         // counted from the new centre, so every node of the row is looked at
         ao = imin;
         bo = imax;
@@ -1656,7 +1658,9 @@ __device__ __forceinline__ void gather_cands(const LatticeView &lv, const PartVi
       cell_geo(pv, pv.kin_next, j, h);
       float d2 = 0.f;
       for (int m = 0; m < 3; ++m) {
-        const float d = image_f(h.Xi[m] - g.Xi[m], h.Xf[m] - g.Xf[m], dims[m], lv.per[m]);
+        const int dn = h.Xi[m] - g.Xi[m];
+        const float df = h.Xf[m] - g.Xf[m];
+        const float d = pv.near_reach ? image_f(dn, df, dims[m], lv.per[m]) : (float)imin_image(dn, dims[m], lv.per[m]) + df;
         d2 += d * d;
       }
       if (d2 > reach * reach) continue;
@@ -1676,9 +1680,10 @@ __device__ __forceinline__ void gather_cands(const LatticeView &lv, const PartVi
 // for up to 32 nodes instead of for the few of one warp's nodes that take a
 // branch.  Bound by latency: a chain of dependent reads per block (17 us for
 // 1022 cells, 84 us for 8446; 23.5 and 128 before).
-template <class S>
+// SET: the cells were set anew (bl_particles_set), not moved by a step.
+template <class S, bool SET>
 __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv, CellListView cl, int *claim,
-                                                      ChangeList chg, int par_next, int impulses, int replaced) {
+                                                      ChangeList chg, int par_next, int impulses) {
   using D = D3Q19;
   const int p = blockIdx.x;
   pdl_trigger();
@@ -1697,9 +1702,9 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
   __shared__ Cands s_cd;
   if (nt == 0) return;
   // (a re-placement can put cells anywhere: its nodes are searched one by one)
-  if (threadIdx.x == 0) s_cd.n = replaced ? NCAND + 1 : 0;
+  if (threadIdx.x == 0) s_cd.n = SET ? NCAND + 1 : 0;
   __syncthreads();
-  if (!replaced) gather_cands(lv, pv, cl, p, s_cd);
+  if constexpr (!SET) gather_cands(lv, pv, cl, p, s_cd);
   for (int t0 = 0; t0 < nt; t0 += PB) {
     const int t = t0 + threadIdx.x;
     int old = 0, nw = 0, xyz[3] = {0, 0, 0};
@@ -1812,7 +1817,7 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
             mf[2] -= C * cz;
           }
           double arm[3];
-          arm64(lv, pv, pv.kin_next, nw, xyz, arm);
+          arm64<SET>(lv, pv, pv.kin_next, nw, xyz, arm);
           const double mom[3] = {mf[0], mf[1], mf[2]};
           const double tq[3] = {arm[1] * mom[2] - arm[2] * mom[1], arm[2] * mom[0] - arm[0] * mom[2],
                                 arm[0] * mom[1] - arm[1] * mom[0]};
@@ -1822,7 +1827,7 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
         if (pm) reinterpret_cast<float *>(lv.pu + idx)[3] = 0.f;
       } else {
         double arm[3];
-        arm64(lv, pv, pv.kin_next, old, xyz, arm);
+        arm64<SET>(lv, pv, pv.kin_next, old, xyz, arm);
         const double *W = pv.Om + 3 * old, *V = pv.V + 3 * old;
         const float u[3] = {(float)(V[0] + (W[1] * arm[2] - W[2] * arm[1])),
                             (float)(V[1] + (W[2] * arm[0] - W[0] * arm[2])),
@@ -1845,7 +1850,7 @@ __global__ void __launch_bounds__(PB) k_resolve_fill(LatticeView lv, PartView pv
         } else {
           // direct change of owner: uncover by the old, cover by the new (reading Q6)
           double an[3];
-          arm64(lv, pv, pv.kin_next, nw, xyz, an);
+          arm64<SET>(lv, pv, pv.kin_next, nw, xyz, an);
           const double tq2[3] = {an[1] * mom[2] - an[2] * mom[1], an[2] * mom[0] - an[0] * mom[2],
                                  an[0] * mom[1] - an[1] * mom[0]};
           atomic_add3(pv.PF + 3 * nw, mom);
@@ -2301,9 +2306,17 @@ void launch_resolve_fill(int dtype, const LatticeView &lv, const PartView &pv, c
                          const ChangeList &chg, int par_next, int impulses, int replaced, cudaStream_t st,
                          int64_t *nl) {
   if (pv.n == 0) return;
-  if (dtype == 0) k_resolve_fill<float><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
-  else if (dtype == 1) k_resolve_fill<__nv_bfloat16><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
-  else k_resolve_fill<__half><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses, replaced);
+#define BL_RESOLVE(S_)                                                                              \
+  if (replaced) k_resolve_fill<S_, true><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses); \
+  else k_resolve_fill<S_, false><<<pv.n, PB, 0, st>>>(lv, pv, cl, claim, chg, par_next, impulses)
+  if (dtype == 0) {
+    BL_RESOLVE(float);
+  } else if (dtype == 1) {
+    BL_RESOLVE(__nv_bfloat16);
+  } else {
+    BL_RESOLVE(__half);
+  }
+#undef BL_RESOLVE
   *nl += 1;
 }
 
