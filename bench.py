@@ -247,7 +247,7 @@ def make_workload(name):
 # workload at FP32 storage kept with the profiles, valid for the sweep source
 # it was taken on (lb_sweep.cuh, first 16 hex digits of its SHA-256) and that
 # workload only
-SWEEP_TRAFFIC = {"sha": "7468576a20f18eec", "config": "shear128", "store": 0, "bytes": 330838656}
+SWEEP_TRAFFIC = {"sha": "3992332bb59576f6", "config": "shear128", "store": 0, "bytes": 330525440}
 
 
 SWEEP_KERNELS = {
